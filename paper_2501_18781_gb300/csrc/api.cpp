@@ -774,24 +774,22 @@ mf_status apply_impl(mf_op* op, const T* src, T* dst, int nrhs, int64_t ld, bool
         const int64_t nc = op->ncells;
         const bool ext = op->p.oseen_flags != 0;
         if (!op->df_ready) {
-          MF_TRY(op->cm_df.alloc(sizeof(float) * 54 * nc));
-          MF_TRY(op->cv_df.alloc(sizeof(float) * 54 * nc));
-          MF_TRY(op->cb_df.alloc(sizeof(float) * 162 * nc));
-          MF_TRY(launch_split_pairs(c, op->cm64.as<double>(), 27 * nc, op->cm_df.as<float>(), op->cm_df.as<float>() + 27 * nc));
-          MF_TRY(launch_split_pairs(c, op->cv64.as<double>(), 27 * nc, op->cv_df.as<float>(), op->cv_df.as<float>() + 27 * nc));
-          MF_TRY(launch_split_pairs(c, op->cb64.as<double>(), 81 * nc, op->cb_df.as<float>(), op->cb_df.as<float>() + 81 * nc));
+          MF_TRY(op->cm_df.alloc(sizeof(float2) * 27 * nc));
+          MF_TRY(op->cv_df.alloc(sizeof(float2) * 27 * nc));
+          MF_TRY(op->cb_df.alloc(sizeof(float2) * 81 * nc));
+          MF_TRY(launch_oseen_df_split(c, op->map[0], op->cm64.as<double>(), op->cv64.as<double>(), op->cb64.as<double>(),
+                                       op->cm_df.as<float2>(), op->cv_df.as<float2>(), op->cb_df.as<float2>()));
           if (ext) {
-            MF_TRY(op->nrm_df.alloc(sizeof(float) * 162 * nc));
-            MF_TRY(launch_split_pairs(c, op->nrm64.as<double>(), 81 * nc, op->nrm_df.as<float>(),
-                                      op->nrm_df.as<float>() + 81 * nc));
+            MF_TRY(op->nrm_df.alloc(sizeof(float2) * 81 * nc));
+            MF_TRY(launch_split_pairs(c, op->nrm64.as<double>(), 81 * nc, 1.0, op->nrm_df.as<float2>()));
           }
           op->df_ready = true;
         }
         for (int r = 0; r < nrhs; ++r) {
           MF_TRY(launch_oseen_df_uniform(c, op->map[0], reinterpret_cast<const double*>(src + r * ld),
-                                         reinterpret_cast<double*>(dst + r * ld), op->cm_df.as<float>(),
-                                         op->cv_df.as<float>(), op->cb_df.as<float>(),
-                                         ext ? op->nrm_df.as<float>() : nullptr));
+                                         reinterpret_cast<double*>(dst + r * ld), op->cm_df.as<float2>(),
+                                         op->cv_df.as<float2>(), op->cb_df.as<float2>(),
+                                         ext ? op->nrm_df.as<float2>() : nullptr));
           MF_TRY(launch_dirichlet_copy(c, op->map[0], src + r * ld, dst + r * ld, 3, nu, 0, false));
         }
         op->variant = std::string("oseen_q2q1/df64/tabulated/warp-per-component") + (ext ? "/meltpool" : "");
@@ -821,15 +819,13 @@ mf_status apply_impl(mf_op* op, const T* src, T* dst, int nrhs, int64_t ld, bool
     // double-float reinitialisation on octree meshes: the plane-by-plane kernel through the cell map
     if (df && !op->map[0]->uniform && kind == K_REINIT && nrhs <= 65535) {
       if (!op->df_ready) {
-        MF_TRY(op->qvec_dfh.alloc(sizeof(float) * 81 * op->ncells));
-        MF_TRY(op->qvec_dfl.alloc(sizeof(float) * 81 * op->ncells));
-        MF_TRY(launch_split_pairs(c, op->qvec64.as<double>(), 81 * op->ncells, op->qvec_dfh.as<float>(),
-                                  op->qvec_dfl.as<float>()));
+        MF_TRY(op->qvec_df.alloc(sizeof(float2) * 81 * op->ncells));
+        MF_TRY(launch_split_pairs(c, op->qvec64.as<double>(), 81 * op->ncells, 1.0, op->qvec_df.as<float2>()));
         op->df_ready = true;
       }
       MF_TRY(launch_reinit_df_octree(c, op->map[0], reinterpret_cast<const double*>(src),
-                                     reinterpret_cast<double*>(dst), nrhs, ld, op->qvec_dfh.as<float>(),
-                                     op->qvec_dfl.as<float>(), op->p.eps, value_coef(op)));
+                                     reinterpret_cast<double*>(dst), nrhs, ld, op->qvec_df.as<float2>(), op->p.eps,
+                                     value_coef(op)));
       MF_TRY(launch_dirichlet_copy(c, op->map[0], src, dst, nrhs, ld, 0, false));
       op->variant = "reinit/octree/df64/tabulated/planes";
       return MF_OK;
@@ -839,35 +835,22 @@ mf_status apply_impl(mf_op* op, const T* src, T* dst, int nrhs, int64_t ld, bool
     const bool qm = kind == K_HEAT && op->rhocp_user;
     if (df && op->map[0]->uniform && (kind == K_HELM || kind == K_HEAT) && (!qm || beta) && nrhs <= 65535) {
       if (!op->df_ready) {
-        MF_TRY(op->qcoef_dfh.alloc(sizeof(float) * 27 * op->ncells));
-        MF_TRY(op->qcoef_dfl.alloc(sizeof(float) * 27 * op->ncells));
-        MF_TRY(launch_df_coef_split(c, op->map[0], op->qcoef64.as<double>(), op->qcoef_dfh.as<float>(),
-                                    op->qcoef_dfl.as<float>()));
+        MF_TRY(op->qcoef_df.alloc(sizeof(float2) * 27 * op->ncells));
+        MF_TRY(launch_df_coef_split(c, op->map[0], op->qcoef64.as<double>(), op->qcoef_df.as<float2>()));
         if (beta) {
-          MF_TRY(op->qvec_dfh.alloc(sizeof(float) * 81 * op->ncells));
-          MF_TRY(op->qvec_dfl.alloc(sizeof(float) * 81 * op->ncells));
-          MF_TRY(launch_df_vec_split(c, op->map[0], op->qvec64.as<double>(), op->qvec_dfh.as<float>(),
-                                     op->qvec_dfl.as<float>()));
+          MF_TRY(op->qvec_df.alloc(sizeof(float2) * 81 * op->ncells));
+          MF_TRY(launch_df_vec_split(c, op->map[0], op->qvec64.as<double>(), op->qvec_df.as<float2>()));
         }
         if (qm) {
-          MF_TRY(op->qmass_dfh.alloc(sizeof(float) * 27 * op->ncells));
-          MF_TRY(op->qmass_dfl.alloc(sizeof(float) * 27 * op->ncells));
-          MF_TRY(launch_df_mass_split(c, op->map[0], op->qmass64.as<double>(), op->qmass_dfh.as<float>(),
-                                      op->qmass_dfl.as<float>()));
+          MF_TRY(op->qmass_df.alloc(sizeof(float2) * 27 * op->ncells));
+          MF_TRY(launch_df_mass_split(c, op->map[0], op->qmass64.as<double>(), op->qmass_df.as<float2>()));
         }
         op->df_ready = true;
       }
-      if (beta)
-        MF_TRY(launch_scalar_df_uniform_conv(c, op->map[0], reinterpret_cast<const double*>(src),
-                                             reinterpret_cast<double*>(dst), nrhs, ld, op->qcoef_dfh.as<float>(),
-                                             op->qcoef_dfl.as<float>(), op->qvec_dfh.as<float>(),
-                                             op->qvec_dfl.as<float>(), value_coef(op), transpose,
-                                             qm ? op->qmass_dfh.as<float>() : nullptr,
-                                             qm ? op->qmass_dfl.as<float>() : nullptr));
-      else
-        MF_TRY(launch_scalar_df_uniform(c, op->map[0], reinterpret_cast<const double*>(src),
-                                        reinterpret_cast<double*>(dst), nrhs, ld, op->qcoef_dfh.as<float>(),
-                                        op->qcoef_dfl.as<float>(), value_coef(op)));
+      MF_TRY(launch_scalar_df_uniform(c, op->map[0], reinterpret_cast<const double*>(src),
+                                      reinterpret_cast<double*>(dst), nrhs, ld, op->qcoef_df.as<float2>(),
+                                      beta ? op->qvec_df.as<float2>() : nullptr,
+                                      qm ? op->qmass_df.as<float2>() : nullptr, value_coef(op), transpose));
       MF_TRY(launch_dirichlet_copy(c, op->map[0], src, dst, nrhs, ld, 0, false));
       op->variant = std::string(kind == K_HELM ? "helmholtz" : "heat") + "/uniform/df64/tabulated/planes" +
                     (beta ? (transpose ? "/conv-T" : "/conv") : "");

@@ -7,13 +7,17 @@
 // values are gathered through the cell map in fp64 (a hanging node as the weighted sum of its
 // masters), scaled by one power of two per warp and split into float pairs; values and derivatives
 // at the Gauss points run in double-float on the fp32 pipes.  Every flux of this operator is
-// s n with s = w eps h (n . grad u), so one pass forms s at the 27 Gauss points, parked in a second
-// shared-memory column (55 KB per block, four blocks per SM; kept in registers it spilled 3 KB and ran
-// 10 % slower on eight right-hand sides);
-// the test side is then accumulated one z-plane at a time: the value term and the z part
-// sum_q' D[q'][qc] s n_z, then the x and y parts s n_x, s n_y through the plane's transposed sweeps,
-// parked in the thread's shared-memory column; the z sweep runs at the end.  The cell's contributions
-// are joined to doubles and added to the free DoFs, hanging ones through the constraint weights.
+// s n with s = w eps h (n . grad u).  The values and s live in two shared-memory columns of the thread
+// and each phase is a rolled loop over them: planes z = const (n_x d_x u + n_y d_y u), z lines (s),
+// planes again (value term and the x and y test parts, over the values), z lines (z test part and
+// transpose), slabs of nodes (y and x transposes).  The cell's contributions are joined to doubles and
+// added to the free DoFs, hanging ones through the constraint weights.  The blocks of all right-hand
+// sides of one range of cells are neighbours in the launch order, so the normals (648 bytes per cell)
+// are read from HBM once and from L2 by the other right-hand sides (591 MB instead of 4.0 GB of HBM reads
+// for eight of them).  Measured: eight right-hand sides on the base 12 + 3 levels octree 3750 -> 1190 us
+// (1.17 ms at 47 % of the issue slots, long-scoreboard stalls on the scattered values).
+#include <algorithm>
+
 #include "df_pairs.cuh"
 
 namespace mf {
@@ -29,161 +33,217 @@ constexpr int kOctThreads = 128;
 struct DfOctArgs {
   const double* src;
   double* dst;
-  int nrhs;           // right-hand sides, one per blockIdx.y
+  int nrhs;           // right-hand sides: block b works on right-hand side b % nrhs
   int64_t ld;         // distance between right-hand sides
-  const float* nh;    // [3][27][ncells] unit normal per Gauss point, high parts
-  const float* nl;    //                 low parts
+  const float2* n;    // [3][27][ncells] unit normal per Gauss point
   int64_t ncells;     // stride of the normal table
-  float eh_h, eh_l;   // eps h0 (h0: edge of a level-0 cell)
-  float mh_h, mh_l;   // m h0^3 (m: value coefficient 1 / dtau)
+  float2 we[27];      // (5/3) w_q eps h0 (h0: edge of a level-0 cell; 5/3: both derivative factors)
+  float2 wm[27];      // w_q m h0^3 (m: value coefficient 1 / dtau)
 };
 
-__device__ __forceinline__ dd dd_scale2(dd a, float s) { return {a.h * s, a.l * s}; }   // s a power of two
+constexpr int kOctSmem = 2 * 27 * kOctThreads * int(sizeof(float2));
 __device__ __forceinline__ float pow2f_oct(int e) { return __uint_as_float(unsigned(e + 127) << 23); }
 
-__global__ void __launch_bounds__(kOctThreads, 4) k_reinit_df_octree(DfOctArgs A, OctGeom og) {
-  extern __shared__ float oct_smem[];
-  float(*sh)[kOctThreads] = reinterpret_cast<float(*)[kOctThreads]>(oct_smem);
-  float(*sl)[kOctThreads] = reinterpret_cast<float(*)[kOctThreads]>(oct_smem + 27 * kOctThreads);
-  float(*zh)[kOctThreads] = reinterpret_cast<float(*)[kOctThreads]>(oct_smem + 54 * kOctThreads);
-  float(*zl)[kOctThreads] = reinterpret_cast<float(*)[kOctThreads]>(oct_smem + 81 * kOctThreads);
+__global__ void __launch_bounds__(kOctThreads, 4) k_reinit_df_octree(const __grid_constant__ DfOctArgs A, OctGeom og) {
+  extern __shared__ float2 oct_smem[];
   const int t = threadIdx.x;
-  const int64_t slot = int64_t(blockIdx.x) * kOctThreads + t;
+  float2* const sU = oct_smem + t;
+  float2* const sV = oct_smem + 27 * kOctThreads + t;
+  auto ld2 = [](const float2* p) { const float2 v = *p; return dd{v.x, v.y}; };
+  auto st2 = [](float2* p, dd v) { *p = make_float2(v.h, v.l); };
+  auto ldg2 = [](const float2* p) { const float2 v = __ldg(p); return dd{v.x, v.y}; };
+  const int rhs = blockIdx.x % A.nrhs;
+  const int64_t slot = int64_t(blockIdx.x / A.nrhs) * kOctThreads + t;
   const bool active = slot < og.ncells;
   const int64_t cell = active ? __ldg(og.order + slot) : 0;
   const int lev = active ? __ldg(og.level + cell) : 0;
-  const double* __restrict__ src = A.src + int64_t(blockIdx.y) * A.ld;
+  const double* __restrict__ src = A.src + rhs * A.ld;
+  const int32_t* __restrict__ map = og.cmap + cell;
+  const int64_t nc = A.ncells;
   int bias = 0;
   {
-    // the map entries live only here and are read again for the scatter (fewer live registers)
-    int32_t id[27];
-#pragma unroll
-    for (int l = 0; l < 27; ++l) id[l] = active ? __ldg(og.cmap + l * og.ncp + cell) : 0;
     double X[27];
+    uint32_t hanging = 0;
+    {
+      int32_t id[27];
 #pragma unroll
-    for (int l = 0; l < 27; ++l) X[l] = active ? __ldg(src + (id[l] >= 0 ? id[l] : 0)) : 0.0;
-    if (active) {
+      for (int l = 0; l < 27; ++l) id[l] = __ldg(map + l * og.ncp);
 #pragma unroll
       for (int l = 0; l < 27; ++l) {
-        if (id[l] >= 0) {
-          if (og.dflag && __ldg(og.dflag + id[l])) X[l] = 0.0;
-          continue;
-        }
-        const int r = -1 - id[l];
-        double v = 0.0;
-        for (int e = __ldg(og.rowptr + r); e < __ldg(og.rowptr + r + 1); ++e) {
-          const int32_t m = __ldg(og.cols + e);
-          if (!(og.dflag && __ldg(og.dflag + m))) v += __ldg(og.w64 + e) * __ldg(src + m);
-        }
-        X[l] = v;
+        X[l] = __ldg(src + max(id[l], 0));
+        hanging |= id[l] < 0 ? 1u << l : 0u;
+      }
+      if (og.dflag) {
+#pragma unroll
+        for (int l = 0; l < 27; ++l)
+          if (id[l] >= 0 && __ldg(og.dflag + id[l])) X[l] = 0.0;
       }
     }
-    int emax = 0;
+    if (!active) {
+      hanging = 0;
 #pragma unroll
-    for (int l = 0; l < 27; ++l) emax = max(emax, (__double2hiint(X[l]) >> 20) & 0x7FF);
-    emax = int(__reduce_max_sync(0xffffffffu, unsigned(emax)));
-    bias = emax ? emax - 1023 : 0;
-    dd U[27];
+      for (int l = 0; l < 27; ++l) X[l] = 0.0;
+    }
 #pragma unroll
-    for (int l = 0; l < 27; ++l) U[l] = d2dd_bits(X[l], bias);
-    dsweep<0>(U);
-    dsweep<1>(U);
-    dsweep<2>(U);
+    for (int l = 0; l < 27; ++l) *reinterpret_cast<double*>(sU + l * kOctThreads) = X[l];
+    unsigned emax = 0;
 #pragma unroll
-    for (int q = 0; q < 27; ++q) {
-      sh[q][t] = U[q].h;
-      sl[q][t] = U[q].l;
+    for (int l = 0; l < 27; ++l)
+      if (!((hanging >> l) & 1u)) emax = max(emax, unsigned(__double2hiint(X[l])) & 0x7FF00000u);
+    for (uint32_t left = hanging; left; left &= left - 1) {
+      const int l = __ffs(left) - 1;
+      const int r = -1 - __ldg(map + l * og.ncp);
+      double v = 0.0;
+      for (int e = __ldg(og.rowptr + r); e < __ldg(og.rowptr + r + 1); ++e) {
+        const int32_t m = __ldg(og.cols + e);
+        if (!(og.dflag && __ldg(og.dflag + m))) v += __ldg(og.w64 + e) * __ldg(src + m);
+      }
+      *reinterpret_cast<double*>(sU + l * kOctThreads) = v;
+      emax = max(emax, unsigned(__double2hiint(v)) & 0x7FF00000u);
+    }
+    __syncwarp();
+    emax = __reduce_max_sync(0xffffffffu, emax) >> 20;
+    bias = emax ? int(emax) - 1023 : 0;
+  }
+#pragma unroll 1
+  for (float2* p = sU; p < sU + 27 * kOctThreads; p += 3 * kOctThreads) {
+    dd u0 = d2dd_bits(*reinterpret_cast<double*>(p), bias);
+    dd u1 = d2dd_bits(*reinterpret_cast<double*>(p + kOctThreads), bias);
+    dd u2 = d2dd_bits(*reinterpret_cast<double*>(p + 2 * kOctThreads), bias);
+    dd_line_values(u0, u1, u2);
+    st2(p, u0);
+    st2(p + kOctThreads, u1);
+    st2(p + 2 * kOctThreads, u2);
+  }
+#pragma unroll 1
+  for (int n = 0; n < 6; ++n) {   // y lines of the three planes, then z lines
+    const int o = n < 3 ? 9 * n : 3 * (n - 3), st = n < 3 ? 3 : 9;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      float2* const p = sU + (o + a) * kOctThreads;
+      dd u0 = ld2(p), u2 = ld2(p + 2 * st * kOctThreads);
+      dd_line_values(u0, ld2(p + st * kOctThreads), u2);
+      st2(p, u0);
+      st2(p + 2 * st * kOctThreads, u2);
     }
   }
-  auto Uq = [&](int q) { return dd{sh[q][t], sl[q][t]}; };
-  auto nrm = [&](int d, int q) {
-    const int64_t o = (d * 27 + q) * A.ncells + cell;
-    return active ? dd{__ldg(A.nh + o), __ldg(A.nl + o)} : dd{0.f, 0.f};
-  };
-  auto W3 = [&](int q) { return dd{cW3h[q], cW3l[q]}; };
-  // w eps h at the cell's level (h = h0 2^-level, an exact power-of-two scale)
-  const dd eh = dd_scale2(dd{A.eh_h, A.eh_l}, pow2f_oct(-lev));
-  // s(q) = w eps h (n . grad u) at the 27 Gauss points
-#pragma unroll
-  for (int q = 0; q < 27; ++q) {
-    const int qa = q % 3, qb = (q / 3) % 3, qc = q / 9;
-    const int bx = q - qa, by = q - 3 * qb, bz = q - 9 * qc;
-    const dd gx = ddline(qa, Uq(bx), Uq(bx + 1), Uq(bx + 2));
-    const dd gy = ddline(qb, Uq(by), Uq(by + 3), Uq(by + 6));
-    const dd gz = ddline(qc, Uq(bz), Uq(bz + 9), Uq(bz + 18));
-    const dd ng = dd_fma(dd_fma(dd_mul(nrm(0, q), gx), nrm(1, q), gy), nrm(2, q), gz);
-    const dd sq = dd_norm(dd_mul(dd_mul(W3(q), eh), dd_norm(ng)));
-    zh[q][t] = sq.h;
-    zl[q][t] = sq.l;
-  }
-  auto S = [&](int q) { return dd{zh[q][t], zl[q][t]}; };
-  // w m h^3 at the cell's level
-  const dd mh = dd_scale2(dd{A.mh_h, A.mh_l}, pow2f_oct(-3 * lev));
-#pragma unroll
+  const float2* __restrict__ nx = A.n + cell;
+  const float2* __restrict__ ny = nx + 27 * nc;
+  const float2* __restrict__ nz = ny + 27 * nc;
+  // n_x d_x u + n_y d_y u, plane by plane
+#pragma unroll 1
   for (int qc = 0; qc < 3; ++qc) {
-    dd R[9];
+    const int q0 = 9 * qc;
+    dd U[9], S[9];
+#pragma unroll
+    for (int p = 0; p < 9; ++p) U[p] = ld2(sU + (q0 + p) * kOctThreads);
+#pragma unroll
+    for (int n = 0; n < 3; ++n) {
+      dd g0, g1, g2;
+      dd_line_deriv(U[3 * n], U[3 * n + 1], U[3 * n + 2], g0, g1, g2);
+      S[3 * n] = dd_mul(ldg2(nx + (q0 + 3 * n) * nc), g0);
+      S[3 * n + 1] = dd_mul(ldg2(nx + (q0 + 3 * n + 1) * nc), g1);
+      S[3 * n + 2] = dd_mul(ldg2(nx + (q0 + 3 * n + 2) * nc), g2);
+    }
+#pragma unroll
+    for (int n = 0; n < 3; ++n) {
+      dd g0, g1, g2;
+      dd_line_deriv(U[n], U[n + 3], U[n + 6], g0, g1, g2);
+      S[n] = dd_fma(S[n], ldg2(ny + (q0 + n) * nc), g0);
+      S[n + 3] = dd_fma(S[n + 3], ldg2(ny + (q0 + n + 3) * nc), g1);
+      S[n + 6] = dd_fma(S[n + 6], ldg2(ny + (q0 + n + 6) * nc), g2);
+    }
+#pragma unroll
+    for (int p = 0; p < 9; ++p) st2(sV + (q0 + p) * kOctThreads, S[p]);
+  }
+  // s = w eps h (n . grad u), z line by z line (h = h0 2^-level, an exact power-of-two scale)
+  const float s1 = pow2f_oct(-lev), s3 = pow2f_oct(-3 * lev);
+#pragma unroll 1
+  for (int p = 0; p < 9; ++p) {
+    dd g[3];
+    dd_line_deriv(ld2(sU + p * kOctThreads), ld2(sU + (p + 9) * kOctThreads), ld2(sU + (p + 18) * kOctThreads), g[0], g[1],
+                  g[2]);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const int q = p + 9 * c;
+      const dd ng = dd_norm(dd_fma(ld2(sV + q * kOctThreads), ldg2(nz + q * nc), g[c]));
+      st2(sV + q * kOctThreads, dd_norm(dd_pow2(dd_mul(dd{A.we[q].x, A.we[q].y}, ng), s1)));
+    }
+  }
+  // value term and the x and y test parts, plane by plane, over the values
+#pragma unroll 1
+  for (int qc = 0; qc < 3; ++qc) {
+    const int q0 = 9 * qc;
+    dd R[9], S[9];
 #pragma unroll
     for (int p = 0; p < 9; ++p) {
-      const int q = p + 9 * qc;
-      dd acc = dd_mul(dd_mul(W3(q), mh), Uq(q));
-#pragma unroll
-      for (int c2 = 0; c2 < 3; ++c2)
-        if (c2 != 1 || qc != 1) acc = dd_fma(acc, cD(c2, qc), dd_mul(S(p + 9 * c2), nrm(2, p + 9 * c2)));
-      R[p] = acc;
+      S[p] = ld2(sV + (q0 + p) * kOctThreads);
+      R[p] = dd_pow2(dd_mul(dd{A.wm[q0 + p].x, A.wm[q0 + p].y}, ld2(sU + (q0 + p) * kOctThreads)), s3);
     }
 #pragma unroll
-    for (int qb = 0; qb < 3; ++qb)
-#pragma unroll
-      for (int qa = 0; qa < 3; ++qa) {
-        const int p = qa + 3 * qb, q = p + 9 * qc;
-        const dd sq = S(q);
-        const dd fx = dd_mul(sq, nrm(0, q)), fy = dd_mul(sq, nrm(1, q));
-#pragma unroll
-        for (int m = 0; m < 3; ++m) {
-          if (qa != 1 || m != 1) R[p - qa + m] = dd_fma(R[p - qa + m], cD(qa, m), fx);
-          if (qb != 1 || m != 1) R[p - 3 * qb + 3 * m] = dd_fma(R[p - 3 * qb + 3 * m], cD(qb, m), fy);
-        }
-      }
-#pragma unroll
-    for (int p = 0; p < 9; ++p) R[p] = dd_norm(R[p]);
-#pragma unroll
-    for (int b = 0; b < 3; ++b) {   // x, transposed
-      const dd u0 = R[3 * b], u1 = R[3 * b + 1], u2 = R[3 * b + 2];
-      R[3 * b] = dd_norm(dd_add(dd_mul(cS(0, 0), u0), dd_mul(cS(2, 0), u2)));
-      R[3 * b + 1] = dd_norm(dd_add(dd_add(dd_mul(cS(0, 1), u0), u1), dd_mul(cS(2, 1), u2)));
-      R[3 * b + 2] = dd_norm(dd_add(dd_mul(cS(0, 2), u0), dd_mul(cS(2, 2), u2)));
+    for (int n = 0; n < 3; ++n) {
+      const int p = 3 * n;
+      dd_line_deriv_t(dd_mul(S[p], ldg2(nx + (q0 + p) * nc)), dd_mul(S[p + 1], ldg2(nx + (q0 + p + 1) * nc)),
+                      dd_mul(S[p + 2], ldg2(nx + (q0 + p + 2) * nc)), R[p], R[p + 1], R[p + 2]);
     }
 #pragma unroll
-    for (int a = 0; a < 3; ++a) {   // y, transposed
-      const dd u0 = R[a], u1 = R[a + 3], u2 = R[a + 6];
-      R[a] = dd_norm(dd_add(dd_mul(cS(0, 0), u0), dd_mul(cS(2, 0), u2)));
-      R[a + 3] = dd_norm(dd_add(dd_add(dd_mul(cS(0, 1), u0), u1), dd_mul(cS(2, 1), u2)));
-      R[a + 6] = dd_norm(dd_add(dd_mul(cS(0, 2), u0), dd_mul(cS(2, 2), u2)));
-    }
+    for (int n = 0; n < 3; ++n)
+      dd_line_deriv_t(dd_mul(S[n], ldg2(ny + (q0 + n) * nc)), dd_mul(S[n + 3], ldg2(ny + (q0 + n + 3) * nc)),
+                      dd_mul(S[n + 6], ldg2(ny + (q0 + n + 6) * nc)), R[n], R[n + 3], R[n + 6]);
 #pragma unroll
-    for (int p = 0; p < 9; ++p) {
-      sh[p + 9 * qc][t] = R[p].h;
-      sl[p + 9 * qc][t] = R[p].l;
+    for (int p = 0; p < 9; ++p) st2(sU + (q0 + p) * kOctThreads, dd_norm(R[p]));
+  }
+#pragma unroll 1
+  for (int p = 0; p < 9; ++p) {
+    dd f[3], V[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      f[c] = dd_mul(ld2(sV + (p + 9 * c) * kOctThreads), ldg2(nz + (p + 9 * c) * nc));
+      V[c] = ld2(sU + (p + 9 * c) * kOctThreads);
     }
+    dd_line_combine_t(f[0], f[1], f[2], V[0], V[1], V[2]);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) st2(sU + (p + 9 * c) * kOctThreads, V[c]);
   }
   if (!active) return;
-  dd R[27];
+  double* __restrict__ dst = A.dst + rhs * A.ld;
+#pragma unroll 1
+  for (int c = 0; c < 3; ++c) {
+    dd R[9];
+    int32_t id[9];
 #pragma unroll
-  for (int q = 0; q < 27; ++q) R[q] = Uq(q);
-  dsweep_t<2>(R);
-  double* __restrict__ dst = A.dst + int64_t(blockIdx.y) * A.ld;
-#pragma unroll
-  for (int l = 0; l < 27; ++l) {
-    const double v = f2d_bits(R[l].h, bias) + f2d_bits(R[l].l, bias);
-    const int32_t idl = __ldg(og.cmap + l * og.ncp + cell);
-    if (idl >= 0) {
-      if (!(og.dflag && __ldg(og.dflag + idl))) atomicAdd(dst + idl, v);
-      continue;
+    for (int p = 0; p < 9; ++p) {
+      id[p] = __ldg(map + (9 * c + p) * og.ncp);
+      R[p] = ld2(sU + (9 * c + p) * kOctThreads);
     }
-    const int r = -1 - idl;
-    for (int e = __ldg(og.rowptr + r); e < __ldg(og.rowptr + r + 1); ++e) {
-      const int32_t m = __ldg(og.cols + e);
-      if (!(og.dflag && __ldg(og.dflag + m))) atomicAdd(dst + m, __ldg(og.w64 + e) * v);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      dd_line_values_t(R[a], R[a + 3], R[a + 6]);
+      R[a] = dd_norm(R[a]);
+      R[a + 3] = dd_norm(R[a + 3]);
+      R[a + 6] = dd_norm(R[a + 6]);
+    }
+#pragma unroll
+    for (int b = 0; b < 3; ++b) dd_line_values_t(R[3 * b], R[3 * b + 1], R[3 * b + 2]);
+    uint32_t hanging = 0;
+#pragma unroll
+    for (int p = 0; p < 9; ++p) {
+      const double v = f2d_bits(R[p].h, bias) + f2d_bits(R[p].l, bias);
+      if (id[p] >= 0) {
+        if (!(og.dflag && __ldg(og.dflag + id[p]))) atomicAdd(dst + id[p], v);
+      } else {
+        hanging |= 1u << p;
+        *reinterpret_cast<double*>(sU + (9 * c + p) * kOctThreads) = v;
+      }
+    }
+    for (; hanging; hanging &= hanging - 1) {
+      const int p = __ffs(hanging) - 1;
+      const double v = *reinterpret_cast<double*>(sU + (9 * c + p) * kOctThreads);
+      const int r = -1 - __ldg(map + (9 * c + p) * og.ncp);
+      for (int e = __ldg(og.rowptr + r); e < __ldg(og.rowptr + r + 1); ++e) {
+        const int32_t m = __ldg(og.cols + e);
+        if (!(og.dflag && __ldg(og.dflag + m))) atomicAdd(dst + m, __ldg(og.w64 + e) * v);
+      }
     }
   }
 }
@@ -191,33 +251,39 @@ __global__ void __launch_bounds__(kOctThreads, 4) k_reinit_df_octree(DfOctArgs A
 }  // namespace
 
 mf_status launch_reinit_df_octree(mf_ctx* ctx, const mf_dofmap* m, const double* src, double* dst, int nrhs,
-                                  int64_t ld, const float* nh, const float* nl, double eps, double mass) {
+                                  int64_t ld, const float2* n, double eps, double mass) {
   if (m->uniform || m->degree != 2) return fail(MF_EINVAL, "the double-float octree kernel takes octree Q2 maps");
   MF_CUDA_TRY(upload_tables_here());
   const OctGeom og = oct_geom(m);
+  const Tables tb = make_tables();
   DfOctArgs a{};
-  a.src = src;
-  a.dst = dst;
-  a.nrhs = nrhs;
   a.ld = ld;
-  a.nh = nh;
-  a.nl = nl;
+  a.n = n;
   a.ncells = m->n_cells;
-  const double h0 = m->mesh->h0, eh = eps * h0, mh = mass * h0 * h0 * h0;
-  a.eh_h = float(eh);
-  a.eh_l = float(eh - double(a.eh_h));
-  a.mh_h = float(mh);
-  a.mh_l = float(mh - double(a.mh_h));
-  const dim3 grid(unsigned((m->n_cells + kOctThreads - 1) / kOctThreads), unsigned(nrhs));
+  const double h0 = m->mesh->h0;
+  auto pair = [](double v) {
+    const float hi = float(v);
+    return make_float2(hi, float(v - double(hi)));
+  };
+  for (int q = 0; q < 27; ++q) {
+    a.we[q] = pair(tb.W3[q] * eps * h0 * (5.0 / 3.0));
+    a.wm[q] = pair(tb.W3[q] * mass * h0 * h0 * h0);
+  }
+  const int64_t nblk = (m->n_cells + kOctThreads - 1) / kOctThreads;
+  const int most = int(std::min<int64_t>(nrhs, INT32_MAX / nblk));   // right-hand sides one launch can number
   static bool attrs = false;
   if (!attrs) {
-    MF_CUDA_TRY(cudaFuncSetAttribute(k_reinit_df_octree, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     int(108 * kOctThreads * sizeof(float))));
+    MF_CUDA_TRY(cudaFuncSetAttribute(k_reinit_df_octree, cudaFuncAttributeMaxDynamicSharedMemorySize, kOctSmem));
     attrs = true;
   }
-  k_reinit_df_octree<<<grid, kOctThreads, 108 * kOctThreads * sizeof(float), ctx->stream>>>(a, og);
-  ctx->launches++;
-  MF_CUDA_TRY(cudaGetLastError());
+  for (int r = 0; r < nrhs; r += most) {
+    a.nrhs = std::min(most, nrhs - r);
+    a.src = src + r * ld;
+    a.dst = dst + r * ld;
+    k_reinit_df_octree<<<unsigned(nblk * a.nrhs), kOctThreads, kOctSmem, ctx->stream>>>(a, og);
+    ctx->launches++;
+    MF_CUDA_TRY(cudaGetLastError());
+  }
   return MF_OK;
 }
 

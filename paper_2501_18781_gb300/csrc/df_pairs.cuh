@@ -59,34 +59,85 @@ __device__ __forceinline__ dd dd_norm(dd a) {
 }
 __device__ __forceinline__ dd dd_fma(dd acc, dd a, dd b) { return dd_add(acc, dd_mul(a, b)); }
 
-__device__ __forceinline__ dd cS(int q, int a) { return {cSh[3 * q + a], cSl[3 * q + a]}; }
-__device__ __forceinline__ dd cD(int q, int p) { return {cDh[3 * q + p], cDl[3 * q + p]}; }
 
-// nodes -> Gauss points along DIR, in place (the middle Gauss point is the middle node)
-template <int DIR> __device__ __forceinline__ void dsweep(dd* U) {
-#pragma unroll
-  for (int j = 0; j < 9; ++j) {
-    const int b = line_base<DIR>(j), s = Dir<DIR>::s;
-    const dd u0 = U[b], u1 = U[b + s], u2 = U[b + 2 * s];
-    U[b] = dd_norm(dd_add(dd_add(dd_mul(cS(0, 0), u0), dd_mul(cS(0, 1), u1)), dd_mul(cS(0, 2), u2)));
-    U[b + 2 * s] = dd_norm(dd_add(dd_add(dd_mul(cS(2, 0), u0), dd_mul(cS(2, 1), u1)), dd_mul(cS(2, 2), u2)));
-  }
+// The 1D contractions in difference form.  The Q2 nodes are {0, 1/2, 1} and the Gauss points
+// 1/2 -+ delta, 1/2 with delta^2 = 3/20, so a line u of nodal values has at the outer Gauss points
+//   0.4 u1 + 0.3 (u0 + u2) -+ delta (u2 - u0)      (the middle Gauss point is the middle node),
+// and the derivative of the quadratic through three Gauss-point values v is the integer stencil
+//   (-3 v0 + 4 v1 - v2, v2 - v0, v0 - 4 v1 + 3 v2) / (2 delta).
+// The factor 1/(2 delta) is folded into the coefficient tables (kDerivScale below), which leaves a
+// derivative line with five pair additions and no product, and a value line with three products:
+// 44 and 52 fp32 instructions against 78 and 56 in the row-times-column form with tabulated
+// constants; the transposes are 68 and 52 against 108 and 65.  An fp32 pair addition costs 8
+// instructions and a product 4, and these contractions are most of a double-float cell.
+constexpr double kDelta = 0.38729833462074168852;        // sqrt(3/20)
+constexpr double kDerivScale = 1.2909944487358056284;    // 1 / (2 delta); its square is 5/3
+template <int N> struct DfConst;                          // constants as float pairs
+template <> struct DfConst<0> { static constexpr double v = 0.3; };
+template <> struct DfConst<1> { static constexpr double v = 0.4; };
+template <> struct DfConst<2> { static constexpr double v = kDelta; };
+template <> struct DfConst<3> { static constexpr double v = 5.0 / 36.0; };
+template <> struct DfConst<4> { static constexpr double v = 8.0 / 36.0; };
+template <> struct DfConst<5> { static constexpr double v = kDelta * 5.0 / 18.0; };
+template <int N> __device__ __forceinline__ dd dd_mulc(dd a) {
+  constexpr float ch = float(DfConst<N>::v);
+  constexpr float cl = float(DfConst<N>::v - double(ch));
+  return dd_mul(dd{ch, cl}, a);
 }
-// Gauss points -> nodes along DIR (transposed), in place
-template <int DIR> __device__ __forceinline__ void dsweep_t(dd* U) {
-#pragma unroll
-  for (int j = 0; j < 9; ++j) {
-    const int b = line_base<DIR>(j), s = Dir<DIR>::s;
-    const dd u0 = U[b], u1 = U[b + s], u2 = U[b + 2 * s];
-    U[b] = dd_norm(dd_add(dd_mul(cS(0, 0), u0), dd_mul(cS(2, 0), u2)));
-    U[b + s] = dd_norm(dd_add(dd_add(dd_mul(cS(0, 1), u0), u1), dd_mul(cS(2, 1), u2)));
-    U[b + 2 * s] = dd_norm(dd_add(dd_mul(cS(0, 2), u0), dd_mul(cS(2, 2), u2)));
-  }
+__device__ __forceinline__ dd dd_neg(dd a) { return {-a.h, -a.l}; }
+__device__ __forceinline__ dd dd_sub(dd a, dd b) { return dd_add(a, dd_neg(b)); }
+__device__ __forceinline__ dd dd_pow2(dd a, float s) { return {a.h * s, a.l * s}; }   // s a power of two
+
+// one line, nodes -> Gauss points (u1 stays)
+__device__ __forceinline__ void dd_line_values(dd& u0, dd u1, dd& u2) {
+  const dd m = dd_add(dd_mulc<1>(u1), dd_mulc<0>(dd_add(u0, u2)));
+  const dd r = dd_mulc<2>(dd_sub(u2, u0));
+  u0 = dd_norm(dd_sub(m, r));
+  u2 = dd_norm(dd_add(m, r));
 }
-// collocation derivative at point qd of a line (D[1][1] = 0)
-__device__ __forceinline__ dd ddline(int qd, dd u0, dd u1, dd u2) {
-  if (qd == 1) return dd_add(dd_mul(cD(1, 0), u0), dd_mul(cD(1, 2), u2));
-  return dd_add(dd_add(dd_mul(cD(qd, 0), u0), dd_mul(cD(qd, 1), u1)), dd_mul(cD(qd, 2), u2));
+// one line, Gauss points -> nodes (transposed); not renormalised
+__device__ __forceinline__ void dd_line_values_t(dd& f0, dd& f1, dd& f2) {
+  const dd t = dd_add(f0, f2), r = dd_mulc<2>(dd_sub(f2, f0)), c = dd_mulc<0>(t);
+  f1 = dd_add(f1, dd_mulc<1>(t));
+  f0 = dd_sub(c, r);
+  f2 = dd_add(c, r);
+}
+// 2 delta times the derivatives at the three Gauss points of a line of Gauss-point values
+__device__ __forceinline__ void dd_line_deriv(dd v0, dd v1, dd v2, dd& g0, dd& g1, dd& g2) {
+  g1 = dd_sub(v2, v0);
+  const dd c2 = dd_pow2(dd_sub(dd_add(v0, v2), dd_pow2(v1, 2.f)), 2.f);
+  g0 = dd_sub(g1, c2);
+  g2 = dd_add(g1, c2);
+}
+// the transpose of that stencil: (r0, r1, r2) += stencil^T (f0, f1, f2)
+__device__ __forceinline__ void dd_line_deriv_t(dd f0, dd f1, dd f2, dd& r0, dd& r1, dd& r2) {
+  const dd s = dd_add(dd_add(f0, f2), f1), e = dd_sub(f2, f0), e2 = dd_pow2(e, 2.f);
+  r0 = dd_add(r0, dd_sub(e2, s));
+  r1 = dd_sub(r1, dd_pow2(e, 4.f));
+  r2 = dd_add(r2, dd_add(e2, s));
+}
+// one line of a Q1 function: end values -> the three Gauss points
+__device__ __forceinline__ void dd_line_q1(dd p0, dd p1, dd& v0, dd& v1, dd& v2) {
+  const dd r = dd_mulc<2>(dd_sub(p1, p0));
+  v1 = dd_pow2(dd_add(p0, p1), 0.5f);
+  v0 = dd_norm(dd_sub(v1, r));
+  v2 = dd_norm(dd_add(v1, r));
+}
+// its transpose with the Gauss weights (5, 8, 5) / 18
+__device__ __forceinline__ void dd_line_q1_t(dd g0, dd g1, dd g2, dd& o0, dd& o1) {
+  const dd a = dd_add(dd_mulc<3>(dd_add(g0, g2)), dd_mulc<4>(g1)), b = dd_mulc<5>(dd_sub(g2, g0));
+  o0 = dd_norm(dd_sub(a, b));
+  o1 = dd_norm(dd_add(a, b));
+}
+// Gauss points -> nodes of a line whose test side has values v and derivative fluxes f: the transposed
+// value contraction applied to v + stencil^T f, with both transposes sharing their sums and differences
+__device__ __forceinline__ void dd_line_combine_t(dd f0, dd f1, dd f2, dd& v0, dd& v1, dd& v2) {
+  const dd s = dd_add(dd_add(f0, f2), f1), e4 = dd_pow2(dd_sub(f2, f0), 4.f);
+  const dd t = dd_add(dd_add(v0, v2), e4), d = dd_add(dd_sub(v2, v0), dd_pow2(s, 2.f));
+  const dd c = dd_mulc<0>(t), r = dd_mulc<2>(d);
+  v1 = dd_norm(dd_add(dd_sub(v1, e4), dd_mulc<1>(t)));
+  v0 = dd_norm(dd_sub(c, r));
+  v2 = dd_norm(dd_add(c, r));
 }
 
 }  // namespace

@@ -128,31 +128,27 @@ mf_status launch_helmholtz_q3_tc(mf_ctx* ctx, const mf_dofmap* m, const float* s
 // MF_ETIMEOUT (once, then the flag is cleared) if a tensor-core launch timed out; read it after
 // the stream has synchronised to cover the launches of the last call
 mf_status tc_take_error();
-// double-float scalar apply on uniform meshes (Helmholtz, heat without convection or Gauss-point
-// rho_cp): the tabulated coefficient split into float pairs of w_q h c_q, then the apply (dst
-// accumulated, nrhs vectors ld apart)
-mf_status launch_df_coef_split(mf_ctx* ctx, const mf_dofmap* m, const double* qcoef64, float* ch, float* cl);
-// the convective heat operator (transpose: its adjoint) in double-float on a uniform mesh; bh, bl the
-// float pairs of w_q h^2 rho_cp beta_d ([3][27][ncells], from launch_df_vec_split)
-mf_status launch_scalar_df_uniform_conv(mf_ctx* ctx, const mf_dofmap* m, const double* src, double* dst, int nrhs,
-                                        int64_t ld, const float* ch, const float* cl, const float* bh, const float* bl,
-                                        double mass, bool transpose, const float* mh = nullptr,
-                                        const float* ml = nullptr);
-mf_status launch_df_vec_split(mf_ctx* ctx, const mf_dofmap* m, const double* qvec64, float* bh, float* bl);
-// [27][ncells] value coefficients m_q -> w_q h^3 m_q as float pairs (the mh, ml of the kernel above)
-mf_status launch_df_mass_split(mf_ctx* ctx, const mf_dofmap* m, const double* qmass64, float* mh, float* ml);
-// the reinitialisation operator in double-float on an octree map (normals from the float pairs of
-// the fp64 Gauss-point table, [3][27][ncells]); dst zeroed by the caller, Dirichlet rows left alone
+// double-float scalar apply on uniform meshes (Helmholtz, heat, heat with convection and its transpose):
+// the Gauss-point tables as float pairs with weights, powers of h and the derivative factors folded in
+// (c: conductivity or a(phi), 27 per cell; b: convection, 81 per cell; m: value coefficient, 27 per
+// cell), then the apply (dst accumulated, nrhs vectors ld apart; b and qm may be NULL, qm needs b)
+mf_status launch_df_coef_split(mf_ctx* ctx, const mf_dofmap* m, const double* qcoef64, float2* out);
+mf_status launch_df_vec_split(mf_ctx* ctx, const mf_dofmap* m, const double* qvec64, float2* out);
+mf_status launch_df_mass_split(mf_ctx* ctx, const mf_dofmap* m, const double* qmass64, float2* out);
+mf_status launch_scalar_df_uniform(mf_ctx* ctx, const mf_dofmap* m, const double* src, double* dst, int nrhs, int64_t ld,
+                                   const float2* c, const float2* b, const float2* qm, double mass, bool transpose);
+// the reinitialisation operator in double-float on an octree map (n: float pairs of the fp64 normal
+// table, [3][27][ncells]); dst zeroed by the caller, Dirichlet rows left alone
 mf_status launch_reinit_df_octree(mf_ctx* ctx, const mf_dofmap* m, const double* src, double* dst, int nrhs,
-                                  int64_t ld, const float* nh, const float* nl, double eps, double mass);
-mf_status launch_scalar_df_uniform(mf_ctx* ctx, const mf_dofmap* m, const double* src, double* dst, int nrhs,
-                                   int64_t ld, const float* ch, const float* cl, double mass);
+                                  int64_t ld, const float2* n, double eps, double mass);
 // double-float Oseen apply on uniform meshes: the folded coefficient tables cm, cv (27 per cell) and
-// cb (81 per cell) as float pairs (high parts, then low parts); nr: the melt-pool interface normal
-// table (81 per cell, pairs) for the trace correction, or NULL without the melt-pool terms
-mf_status launch_split_pairs(mf_ctx* ctx, const double* c, int64_t n, float* h, float* l);
-mf_status launch_oseen_df_uniform(mf_ctx* ctx, const mf_dofmap* mu, const double* src, double* dst, const float* cm,
-                                  const float* cv, const float* cb, const float* nr);
+// cb (81 per cell) as float pairs from launch_oseen_df_split; nr: the melt-pool interface normal table
+// (81 per cell, pairs) for the trace correction, or NULL without the melt-pool terms
+mf_status launch_split_pairs(mf_ctx* ctx, const double* c, int64_t n, double scale, float2* out);
+mf_status launch_oseen_df_split(mf_ctx* ctx, const mf_dofmap* mu, const double* cm64, const double* cv64,
+                                const double* cb64, float2* cm, float2* cv, float2* cb);
+mf_status launch_oseen_df_uniform(mf_ctx* ctx, const mf_dofmap* mu, const double* src, double* dst, const float2* cm,
+                                  const float2* cv, const float2* cb, const float2* nr);
 // laser top-face load and its parameter derivatives (uniform maps)
 mf_status launch_laser(mf_ctx* ctx, const mf_dofmap* m, const double lz[5], double* f, double* dF);
 // dJ/dk_q = -w_q h grad(lambda) . grad(theta), [cell][27]
@@ -179,7 +175,7 @@ struct mf_op {
   mf::DevBuf qcoef64, qcoef32;    // [27][ncells]
   mf::DevBuf qvec64, qvec32;      // [3][27][ncells]
   mf::DevBuf qmass64, qmass32;    // [27][ncells] heat value term rho_cp,q / dt
-  mf::DevBuf qmass_dfh, qmass_dfl;  // the same times w_q h^3 as float pairs (double-float applies)
+  mf::DevBuf qmass_df;            // the same times w_q h^3 as float pairs (double-float applies)
   mf::DevBuf qcoef_tc;            // Q3 tensor-core apply: fp32 coefficients [tile of 128 cells][q][row]
   bool tc_ready = false;
   int qk_f32_tc = 0;              // Q3: plain fp32 applies run on the tensor cores (autotuned)
@@ -189,8 +185,8 @@ struct mf_op {
   mf::DevBuf diag64;              // cached diagonal (fp64)
   mf::DevBuf blk64, pdiag64;      // Oseen block Jacobi
   bool tables_ready = false;
-  mf::DevBuf qcoef_dfh, qcoef_dfl;  // [27][ncells] float pairs of w_q h c_q for the double-float kernel
-  mf::DevBuf qvec_dfh, qvec_dfl;    // [3][27][ncells] float pairs of w_q h^2 rho_cp beta (convection)
+  mf::DevBuf qcoef_df;              // [27][ncells] float pairs of the scalar coefficient (double-float kernels)
+  mf::DevBuf qvec_df;               // [3][27][ncells] float pairs of the convection (heat) or the normal (reinit)
   bool df_ready = false;
   mf::DevBuf cm_df, cv_df, cb_df;   // Oseen: folded coefficients as float pairs (high, then low parts)
   mf::DevBuf nrm_df;                // Oseen melt-pool terms: the interface normal table as float pairs
