@@ -36,6 +36,7 @@ BlockPool::BlockPool() {
 }
 BlockPool::~BlockPool() {
   trim();
+  if (call_pool) cudaMemPoolDestroy(call_pool);
   std::lock_guard<std::mutex> lk(g_pools_mu);
   g_pools.erase(std::remove(g_pools.begin(), g_pools.end(), this), g_pools.end());
 }
@@ -74,6 +75,36 @@ void BlockPool::trim() {
   for (auto& kv : keep) cudaFree(kv.second);
   keep.clear();
   kept = 0;
+  if (call_pool) {
+    cudaDeviceSynchronize();
+    cudaMemPoolTrimTo(call_pool, 0);
+  }
+}
+// Work memory of one call, in the order of its stream (hand back with cudaFreeAsync on that stream).  The
+// pool keeps what was handed back, at most the largest work areas that ran at once; NULL if there is none.
+mf_status BlockPool::call_get(size_t n, cudaStream_t s, void** out) {
+  *out = nullptr;
+  std::lock_guard<std::mutex> lk(mu);
+  if (!call_pool) {
+    cudaMemPoolProps p{};
+    p.allocType = cudaMemAllocationTypePinned;
+    p.location.type = cudaMemLocationTypeDevice;
+    int dev = 0;
+    MF_CUDA_TRY(cudaGetDevice(&dev));
+    p.location.id = dev;
+    if (cudaMemPoolCreate(&call_pool, &p) != cudaSuccess) {
+      cudaGetLastError();
+      call_pool = nullptr;
+      return MF_OK;
+    }
+    uint64_t keep_all = UINT64_MAX;
+    cudaMemPoolSetAttribute(call_pool, cudaMemPoolAttrReleaseThreshold, &keep_all);
+  }
+  if (cudaMallocFromPoolAsync(out, n, call_pool, s) != cudaSuccess) {
+    cudaGetLastError();
+    *out = nullptr;
+  }
+  return MF_OK;
 }
 void trim_block_pools() {
   std::lock_guard<std::mutex> lk(g_pools_mu);
@@ -490,6 +521,8 @@ mf_status mf_operator_set_field(mf_op* op, int field, const void* ptr, int dtype
   op->tables_ready = false;
   op->tc_ready = false;
   op->df_ready = false;
+  op->tiles_ready = false;
+  op->rhs_ready = false;
   op->diag_ready = false;
   op->lanczos_ready = false;
   op->h16_cnorm = 0.0f;
@@ -726,6 +759,85 @@ mf_status apply_h16(mf_op* op, const float* src, float* dst, int nrhs, int64_t l
   return MF_OK;
 }
 
+// Whether memory can be allocated now: not while the context's stream is being captured into a graph.
+static bool may_allocate(const mf_op* op) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(op->ctx->stream, &st) != cudaSuccess) cudaGetLastError();
+  return st == cudaStreamCaptureStatusNone;
+}
+
+// The fp32 marching kernel's tables of a uniform Q2 Helmholtz or heat operator.  *ok = false where the
+// operator has no such kernel, or where the tables are not built and cannot be now (a capture, no
+// memory): the apply then takes the general kernel.
+static mf_status ensure_tiles(mf_op* op, bool* ok) {
+  const int kind = scalar_kind(op);
+  *ok = op->map[0]->uniform && op->map[0]->degree == 2 && (kind == K_HELM || kind == K_HEAT);
+  if (!*ok || op->tiles_ready) return MF_OK;
+  if (!may_allocate(op)) {
+    *ok = false;
+    return MF_OK;
+  }
+  MF_TRY(ensure_tables(op));
+  const bool beta = heat_convection(op), qm = kind == K_HEAT && op->rhocp_user;
+  const struct {
+    bool used;
+    mf::DevBuf* buf;
+    int rows;
+    const double* table;
+  } parts[3] = {{true, &op->tile_c, 1, op->qcoef64.as<double>()},
+                {beta, &op->tile_b, 3, op->qvec64.as<double>()},
+                {qm, &op->tile_m, 1, op->qmass64.as<double>()}};
+  for (int w = 0; w < 3; ++w) {
+    if (!parts[w].used) continue;
+    const mf_status st = parts[w].buf->alloc(sizeof(float) * tile_table_floats(op->map[0], parts[w].rows));
+    if (st == MF_ENOMEM) {
+      *ok = false;
+      return MF_OK;
+    }
+    MF_TRY(st);
+    MF_TRY(launch_tile_table(op->ctx, op->map[0], w, parts[w].table, parts[w].buf->as<float>()));
+  }
+  op->tiles_ready = true;
+  return MF_OK;
+}
+
+// Lanes per leaf of the fp32 octree reinitialisation for several right-hand sides: the smallest of 2, 4, 8
+// that holds them (0: one right-hand side, or another operator, for which the general kernel serves).
+static int octree_rhs_lanes(const mf_op* op, int nrhs) {
+  if (op->p.kind != MF_OP_REINIT || op->map[0]->uniform || op->map[0]->degree != 2 || nrhs < 2) return 0;
+  return nrhs == 2 ? 2 : (nrhs <= 4 ? 4 : 8);
+}
+int64_t octree_rhs_work(const mf_op* op, int nrhs) {
+  if (op->f32_prec != PREC_F32) return 0;
+  return 2 * int64_t(octree_rhs_lanes(op, nrhs)) * op->n;
+}
+static mf_status ensure_octree_rhs(mf_op* op, bool* ok) {
+  *ok = true;
+  if (op->rhs_ready) return MF_OK;
+  *ok = may_allocate(op);
+  if (!*ok) return MF_OK;
+  MF_TRY(ensure_tables(op));
+  mf_status st = op->rhs_map.alloc(sizeof(int32_t) * 28 * op->ncells);
+  if (st == MF_OK) st = op->rhs_nrm.alloc(sizeof(float) * 84 * op->ncells);
+  if (st == MF_ENOMEM) {
+    *ok = false;
+    return MF_OK;
+  }
+  MF_TRY(st);
+  MF_TRY(launch_octree_rhs_tables(op->ctx, op->map[0], op->qvec64.as<double>(), op->rhs_map.as<int32_t>(),
+                                  op->rhs_nrm.as<float>()));
+  op->rhs_ready = true;
+  return MF_OK;
+}
+
+// Builds what the applies of a solve read before the solve records them into a graph.
+mf_status prepare_f32_applies(mf_op* op) {
+  bool ok;
+  if (op->f32_prec == PREC_F32 && octree_rhs_lanes(op, 2)) return ensure_octree_rhs(op, &ok);
+  if (op->f32_prec == PREC_F32 && (op->mode32 == 1 || heat_tabulated(op))) return ensure_tiles(op, &ok);
+  return MF_OK;
+}
+
 // dst = A src (or A^T src), nrhs vectors ld apart, precision T.
 // prec: PREC_F64 / PREC_DF64 for fp64 vectors (-1: the operator's fp64 arithmetic), PREC_F32 for fp32.
 template <typename T>
@@ -760,6 +872,33 @@ mf_status apply_impl(mf_op* op, const T* src, T* dst, int nrhs, int64_t ld, bool
   const int mode = df ? 1 : (f32 ? op->mode32 : op->mode64);
   const bool needs_tables = op->p.kind == MF_OP_OSEEN || mode == 1 || heat_tabulated(op);
   if (needs_tables) MF_TRY(ensure_tables(op));
+  if constexpr (sizeof(T) == 4) {
+    // fp32 reinitialisation of several right-hand sides on an octree: groups of eight, interleaved
+    if (prec == PREC_F32 && octree_rhs_lanes(op, nrhs)) {
+      bool ok;
+      MF_TRY(ensure_octree_rhs(op, &ok));
+      const int64_t floats = octree_rhs_work(op, std::min(nrhs, 8));
+      float* work = op->rhs_work && op->rhs_work_floats >= floats ? op->rhs_work : nullptr;
+      void* own = nullptr;
+      if (ok && !work && may_allocate(op)) {
+        MF_TRY(c->pool.call_get(sizeof(float) * floats, c->stream, &own));
+        work = static_cast<float*>(own);
+      }
+      if (ok && work) {
+        mf_status st = MF_OK;
+        int r = 0;
+        for (; r < nrhs - 1 && st == MF_OK; r += 8)
+          st = launch_reinit_f32_octree_rhs(c, op->map[0], src + r * ld, dst + r * ld, std::min(8, nrhs - r), ld,
+                                            op->rhs_map.as<int32_t>(), op->rhs_nrm.as<float>(), op->p.eps, value_coef(op),
+                                            work);
+        if (own) MF_CUDA_TRY(cudaFreeAsync(own, c->stream));
+        MF_TRY(st);
+        if (r < nrhs) MF_TRY(apply_impl<T>(op, src + r * ld, dst + r * ld, 1, ld, transpose, prec));
+        op->variant = "reinit/octree/f32/tabulated/interleaved" + std::to_string(octree_rhs_lanes(op, std::min(nrhs, 8)));
+        return MF_OK;
+      }
+    }
+  }
   if (ld == op->n) MF_CUDA_TRY(cudaMemsetAsync(dst, 0, sizeof(T) * op->n * nrhs, c->stream));
   else
     for (int r = 0; r < nrhs; ++r) MF_CUDA_TRY(cudaMemsetAsync(dst + r * ld, 0, sizeof(T) * op->n, c->stream));
@@ -867,6 +1006,20 @@ mf_status apply_impl(mf_op* op, const T* src, T* dst, int nrhs, int64_t ld, bool
     MF_TRY(launch_dirichlet_copy(c, op->map[0], src, dst, nrhs, ld, 0, f32));
     op->variant = std::string(kind == K_HELM ? "helmholtz" : "heat") + "/uniform" + pname + "/tabulated/line-per-thread";
     return MF_OK;
+  }
+  if constexpr (sizeof(T) == 4) {
+    // tabulated fp32 applies on uniform meshes: the marching kernel on its own coefficient tables
+    bool tiles = prec == PREC_F32 && m == 1 && nrhs <= 65535 && !op->general_f32;
+    if (tiles) MF_TRY(ensure_tiles(op, &tiles));
+    if (tiles) {
+      const bool qm = kind == K_HEAT && op->rhocp_user;
+      MF_TRY(launch_scalar_f32_uniform(c, op->map[0], src, dst, nrhs, ld, op->tile_c.as<float>(),
+                                       beta ? op->tile_b.as<float>() : nullptr, qm ? op->tile_m.as<float>() : nullptr,
+                                       value_coef(op), transpose));
+      op->variant = std::string(kind == K_HELM ? "helmholtz" : "heat") + "/uniform/f32/tabulated/march" +
+                    (beta ? (transpose ? "/conv-T" : "/conv") : "");
+      return MF_OK;
+    }
   }
   ScalarArgs<T> a = scalar_args<T>(op, src, dst, nrhs, ld);
   MF_TRY(launch_scalar_apply(c, op->map[0], kind, m, beta, transpose, prec, &a));

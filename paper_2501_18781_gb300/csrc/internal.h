@@ -84,6 +84,9 @@ struct BlockPool {
   ~BlockPool();
   BlockPool(const BlockPool&) = delete;
   BlockPool& operator=(const BlockPool&) = delete;
+  // stream-ordered memory of single calls (created on first use; trimmed with the kept blocks)
+  cudaMemPool_t call_pool = nullptr;
+  mf_status call_get(size_t n, cudaStream_t s, void** out);
   static size_t rounded(size_t n) {
     const size_t big = size_t(2) << 20, small = 512;
     return n >= (size_t(1) << 20) ? (n + big - 1) / big * big : (n + small - 1) / small * small;

@@ -128,6 +128,20 @@ mf_status launch_helmholtz_q3_tc(mf_ctx* ctx, const mf_dofmap* m, const float* s
 // MF_ETIMEOUT (once, then the flag is cleared) if a tensor-core launch timed out; read it after
 // the stream has synchronised to cover the launches of the last call
 mf_status tc_take_error();
+// fp32 scalar apply on uniform meshes (Helmholtz, heat, heat with convection and its transpose) from the
+// tables of launch_tile_table, tile_table_floats(m, rows) floats each (which 0: diffusion coefficient, 27
+// rows; 1: rho_cp beta, 81 rows; 2: value coefficient; from the fp64 [rows][ncells] tables); dst
+// accumulated, nrhs <= 65535 vectors ld apart, b and qm may be NULL
+int64_t tile_table_floats(const mf_dofmap* m, int rows);
+mf_status launch_tile_table(mf_ctx* ctx, const mf_dofmap* m, int which, const double* c, float* out);
+mf_status launch_scalar_f32_uniform(mf_ctx* ctx, const mf_dofmap* m, const float* src, float* dst, int nrhs, int64_t ld,
+                                    const float* c, const float* b, const float* qm, double mass, bool transpose);
+// fp32 reinitialisation apply to 2..8 right-hand sides on an octree map: per leaf in processing order its
+// node numbers and level (28 ints) and normals (84 floats), and 2 W n_dofs floats of work (W = 2, 4 or 8,
+// the smallest >= nr); writes every entry of dst (Dirichlet rows = src)
+mf_status launch_octree_rhs_tables(mf_ctx* ctx, const mf_dofmap* m, const double* qvec64, int32_t* map, float* nrm);
+mf_status launch_reinit_f32_octree_rhs(mf_ctx* ctx, const mf_dofmap* m, const float* src, float* dst, int nr, int64_t ld,
+                                       const int32_t* map, const float* nrm, double eps, double mass, float* work);
 // double-float scalar apply on uniform meshes (Helmholtz, heat, heat with convection and its transpose):
 // the Gauss-point tables as float pairs with weights, powers of h and the derivative factors folded in
 // (c: conductivity or a(phi), 27 per cell; b: convection, 81 per cell; m: value coefficient, 27 per
@@ -188,6 +202,13 @@ struct mf_op {
   mf::DevBuf qcoef_df;              // [27][ncells] float pairs of the scalar coefficient (double-float kernels)
   mf::DevBuf qvec_df;               // [3][27][ncells] float pairs of the convection (heat) or the normal (reinit)
   bool df_ready = false;
+  mf::DevBuf tile_c, tile_b, tile_m;   // fp32 uniform kernel: coefficient tables per tile of cells
+  bool tiles_ready = false;
+  bool general_f32 = false;            // mf_autotune: time the general kernel
+  mf::DevBuf rhs_map, rhs_nrm;         // fp32 octree kernel for several right-hand sides: per-leaf tables
+  bool rhs_ready = false;
+  float* rhs_work = nullptr;           // its work vectors while a solve lends them, else per call
+  int64_t rhs_work_floats = 0;
   mf::DevBuf cm_df, cv_df, cb_df;   // Oseen: folded coefficients as float pairs (high, then low parts)
   mf::DevBuf nrm_df;                // Oseen melt-pool terms: the interface normal table as float pairs
   bool diag_ready = false;

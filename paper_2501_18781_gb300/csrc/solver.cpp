@@ -23,6 +23,8 @@ bool heat_convection(const mf_op* op);
 int qk_degree(const mf_op* op);
 bool heat_tabulated(const mf_op* op);
 mf_status ensure_tables(mf_op* op);
+mf_status prepare_f32_applies(mf_op* op);
+int64_t octree_rhs_work(const mf_op* op, int nrhs);
 int scalar_kind(const mf_op* op);
 double value_coef(const mf_op* op);
 template <typename T> ScalarArgs<T> scalar_args(const mf_op* op, const T* src, T* dst, int nrhs, int64_t ld);
@@ -532,6 +534,7 @@ template <typename T> struct CG {
   Prec<T>* P;
   int nrhs;
   Vec<T> r, z, p, Ap;
+  Vec<float> work;   // interleaved vectors of batched fp32 octree applies (recorded into the step's graph)
   int check_every = 1;
   bool use_graph = false;
   cudaGraphExec_t exec = nullptr;
@@ -539,6 +542,7 @@ template <typename T> struct CG {
 
   ~CG() {
     if (exec) cudaGraphExecDestroy(exec);
+    if (work.p) op->rhs_work = nullptr;
   }
 
   mf_status setup(mf_op* o, Prec<T>* pr, int nr) {
@@ -546,6 +550,18 @@ template <typename T> struct CG {
     P = pr;
     nrhs = nr;
     const int64_t n = op->n * nrhs;
+    if (sizeof(T) == 4) {
+      MF_TRY(prepare_f32_applies(op));
+      const int64_t floats = octree_rhs_work(op, nrhs);
+      if (floats > 0) {
+        const mf_status st = work.alloc(floats);
+        if (st != MF_OK && st != MF_ENOMEM) return st;
+        if (st == MF_OK) {
+          op->rhs_work = work.p;
+          op->rhs_work_floats = floats;
+        }
+      }
+    }
     MF_TRY(r.alloc(n));
     MF_TRY(p.alloc(n));
     MF_TRY(Ap.alloc(n));
@@ -1221,9 +1237,10 @@ mf_status autotune_measure(mf_op* op) {
     MF_TRY(s32.alloc(sizeof(float) * n));
     MF_TRY(d32.alloc(sizeof(float) * n));
     MF_TRY(convert<double, float>(c, n, src.as<double>(), s32.as<float>()));
-    // the launch shape of octree operators is timed on a batch of eight right-hand sides (their
-    // batched reinitialisation; one and eight right-hand sides prefer different shapes)
-    const int shape_rhs = op->map[0]->uniform ? 1 : 8;
+    // the launch shape of octree operators is timed on a batch of eight right-hand sides (one and eight
+    // prefer different shapes); the reinitialisation, whose fp32 batches have their own kernel, on one
+    const bool batch = !op->map[0]->uniform && op->p.kind == MF_OP_REINIT;
+    const int shape_rhs = op->map[0]->uniform || batch ? 1 : 8;
     DevBuf sb, db;
     if (shape_rhs > 1) {
       MF_TRY(sb.alloc(sizeof(float) * n * shape_rhs));
@@ -1261,7 +1278,13 @@ mf_status autotune_measure(mf_op* op) {
       }
     op->mode64 = mode_ms[0][0] < mode_ms[0][1] ? 0 : 1;
     op->mode32 = (op->p.kind != MF_OP_REINIT && mode_ms[1][0] < mode_ms[1][1]) ? 0 : 1;
-    // 2) launch shape on the fp32 apply: cells per block (octree) and persistent grids
+    // 2) launch shape of the general kernel on the fp32 apply: cells per block (octree) and persistent grids
+    struct Shapes {
+      mf_op* op;
+      explicit Shapes(mf_op* o) : op(o) { op->general_f32 = true; }
+      ~Shapes() { op->general_f32 = false; }
+    };
+    std::unique_ptr<Shapes> general(new Shapes(op));
     const int shapes[5][2] = {{128, 0}, {64, 0}, {128, 2}, {128, 4}, {64, 8}};
     double shape_ms[5];
     int best_shape = 0;
@@ -1275,10 +1298,13 @@ mf_status autotune_measure(mf_op* op) {
     }
     op->block = shapes[best_shape][0];
     op->persistent_blocks = shapes[best_shape][1];
+    general.reset();
     // 3) fp64-accurate arithmetic: fp64 pipes vs double-float on the fp32 pipes; on uniform Q2
     //    Helmholtz / heat operators also the line-per-thread kernel in fp64 and fp32 (small meshes)
-    double f64_ms, df_ms, line64_ms = -1.0, line32_ms = -1.0;
+    double f64_ms, df_ms, f32_ms, line64_ms = -1.0, line32_ms = -1.0;
     op->q2_line64 = op->q2_line32 = 0;
+    MF_TRY(time_variant(PREC_F32, &f32_ms));
+    if (batch) MF_TRY(prepare_f32_applies(op));
     MF_TRY(time_variant(PREC_F64, &f64_ms));
     MF_TRY(time_variant(PREC_DF64, &df_ms));
     const int kind = scalar_kind(op);
@@ -1290,7 +1316,7 @@ mf_status autotune_measure(mf_op* op) {
       op->q2_line32 = 1;
       MF_TRY(time_variant(PREC_F32, &line32_ms));
       op->q2_line64 = line64_ms < f64_ms ? 1 : 0;
-      op->q2_line32 = line32_ms < shape_ms[best_shape] ? 1 : 0;
+      op->q2_line32 = line32_ms < f32_ms ? 1 : 0;
     }
     op->df64_faster = df_ms < (op->q2_line64 ? line64_ms : f64_ms);
     cudaEventDestroy(e0);
@@ -1302,7 +1328,7 @@ mf_status autotune_measure(mf_op* op) {
                   "\"f32_shape_ms\": %.6g, \"f64_ms\": %.6g, \"df64_ms\": %.6g, \"f64_line_ms\": %.6g, "
                   "\"f32_line_ms\": %.6g}",
                   op->p.kind, (long long)n, mode_ms[0][0], mode_ms[0][1], mode_ms[1][0], mode_ms[1][1], op->block,
-                  op->persistent_blocks, shape_ms[best_shape], f64_ms, df_ms, line64_ms, line32_ms);
+                  op->persistent_blocks, f32_ms, f64_ms, df_ms, line64_ms, line32_ms);
     op->tune_record = buf;
     return MF_OK;
   } catch (...) {
