@@ -164,9 +164,9 @@ mf_status mf_context_create(int device, void* cuda_stream, mf_ctx** out) {
   cudaDeviceGetAttribute(&c->sm_count, cudaDevAttrMultiProcessorCount, device);
   mf_status st = c->scratch.alloc(kScratchDoubles * sizeof(double));
   if (st == MF_OK) st = c->scalars.alloc(sizeof(double) * kScalarsTotal);
-  if (st == MF_OK) st = c->counters.alloc(sizeof(unsigned) * 64);
+  if (st == MF_OK) st = c->counters.alloc(sizeof(unsigned) * kCounters);
   // zeroed on the context's stream (a non-blocking stream is not ordered after the legacy one)
-  if (st == MF_OK && (cudaMemsetAsync(c->counters.p, 0, sizeof(unsigned) * 64, c->stream) != cudaSuccess ||
+  if (st == MF_OK && (cudaMemsetAsync(c->counters.p, 0, sizeof(unsigned) * kCounters, c->stream) != cudaSuccess ||
                       cudaStreamSynchronize(c->stream) != cudaSuccess))
     st = fail(MF_ECUDA, "zeroing the reduction counters failed");
   if (st == MF_OK && cudaMallocHost(&c->host_scalars, sizeof(double) * kScalarsTotal) != cudaSuccess)
@@ -830,9 +830,35 @@ static mf_status ensure_octree_rhs(mf_op* op, bool* ok) {
   return MF_OK;
 }
 
+// The fp32 Oseen kernel's tables per tile; *ok = false where they cannot be built now.
+static mf_status ensure_oseen_tiles(mf_op* op, bool* ok) {
+  *ok = true;
+  if (op->tiles_ready) return MF_OK;
+  *ok = may_allocate(op);
+  if (!*ok) return MF_OK;
+  MF_TRY(ensure_tables(op));
+  const bool ext = op->p.oseen_flags != 0;
+  const size_t one = sizeof(float) * tile_table_floats(op->map[0], 1);
+  mf_status st = op->tile_c.alloc(one);
+  if (st == MF_OK) st = op->tile_m.alloc(one);
+  if (st == MF_OK) st = op->tile_b.alloc(3 * one);
+  if (st == MF_OK && ext) st = op->tile_n.alloc(3 * one);
+  if (st == MF_ENOMEM) {
+    *ok = false;
+    return MF_OK;
+  }
+  MF_TRY(st);
+  MF_TRY(launch_oseen_f32_tables(op->ctx, op->map[0], op->cm64.as<double>(), op->cv64.as<double>(), op->cb64.as<double>(),
+                                 ext ? op->nrm64.as<double>() : nullptr, op->tile_c.as<float>(), op->tile_m.as<float>(),
+                                 op->tile_b.as<float>(), ext ? op->tile_n.as<float>() : nullptr));
+  op->tiles_ready = true;
+  return MF_OK;
+}
+
 // Builds what the applies of a solve read before the solve records them into a graph.
 mf_status prepare_f32_applies(mf_op* op) {
   bool ok;
+  if (op->p.kind == MF_OP_OSEEN) return ensure_oseen_tiles(op, &ok);
   if (op->f32_prec == PREC_F32 && octree_rhs_lanes(op, 2)) return ensure_octree_rhs(op, &ok);
   if (op->f32_prec == PREC_F32 && (op->mode32 == 1 || heat_tabulated(op))) return ensure_tiles(op, &ok);
   return MF_OK;
@@ -932,6 +958,18 @@ mf_status apply_impl(mf_op* op, const T* src, T* dst, int nrhs, int64_t ld, bool
           MF_TRY(launch_dirichlet_copy(c, op->map[0], src + r * ld, dst + r * ld, 3, nu, 0, false));
         }
         op->variant = std::string("oseen_q2q1/df64/tabulated/warp-per-component") + (ext ? "/meltpool" : "");
+        return MF_OK;
+      }
+    }
+    if constexpr (sizeof(T) == 4) {
+      bool ok;
+      MF_TRY(ensure_oseen_tiles(op, &ok));
+      if (ok) {
+        for (int r = 0; r < nrhs; ++r)
+          MF_TRY(launch_oseen_f32_uniform(c, op->map[0], src + r * ld, dst + r * ld, op->tile_c.as<float>(),
+                                          op->tile_m.as<float>(), op->tile_b.as<float>(),
+                                          op->p.oseen_flags ? op->tile_n.as<float>() : nullptr));
+        op->variant = std::string("oseen_q2q1/f32/tabulated/warp-per-component") + (op->p.oseen_flags ? "/meltpool" : "");
         return MF_OK;
       }
     }
@@ -1055,7 +1093,7 @@ template <typename T> mf_status oseen_coupling(mf_op* op, int which, const T* sr
       MF_TRY(pinv.alloc(sizeof(float) * size_t(np)));
       MF_TRY(oseen_blocks32(op, ua.as<float>(), pinv.as<float>()));
       MF_TRY(launch_schur_assemble_f32(op->ctx, op->map[0], ua.as<float>(), ub.p, sc.as<float>()));
-      MF_TRY(stencil125_apply(op->ctx, ub.p, sc.as<float>(), src, dst, gn[0], gn[1], gn[2], nullptr));
+      MF_TRY(stencil125_apply(op->ctx, ub.p, sc.as<float>(), src, dst, gn[0], gn[1], gn[2]));
       MF_CUDA_TRY(cudaStreamSynchronize(op->ctx->stream));  // before sc is freed
     } else {
       MF_TRY(diag64(op, nullptr));

@@ -207,7 +207,8 @@ __global__ void __launch_bounds__(kTileThreads, kTileBlocks) k_scalar_f32_march(
   store_plane(2 * k1, Rc);
 }
 
-// [rows][27][ncells] table -> [tile][27 rows][32] with w_q s folded in; lanes without a cell 0
+// [rows][27][ncells] table -> [tile][27 rows][32] times s (and w_q); lanes without a cell 0
+template <bool WEIGHTED>
 __global__ void k_tile_table(const double* __restrict__ c, int rows, double s, float* __restrict__ out, int ntx, int nty,
                              UniformGeom ug) {
   const int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
@@ -220,7 +221,7 @@ __global__ void k_tile_table(const double* __restrict__ c, int rows, double s, f
   const bool active = i < ug.nx && j < ug.ny;
   const int64_t cell = i + int64_t(ug.nx) * (j + int64_t(ug.ny) * k);
   for (int r = 0; r < 27 * rows; ++r)
-    out[(tile * (27 * rows) + r) * 32 + lane] = active ? float(c[r * nc + cell] * (cW364[r % 27] * s)) : 0.f;
+    out[(tile * (27 * rows) + r) * 32 + lane] = active ? float(c[r * nc + cell] * (WEIGHTED ? cW364[r % 27] * s : s)) : 0.f;
 }
 
 int64_t tile_count(const UniformGeom& ug) { return int64_t((ug.nx + 7) / 8) * ((ug.ny + 3) / 4) * ug.nz; }
@@ -235,8 +236,18 @@ mf_status launch_tile_table(mf_ctx* ctx, const mf_dofmap* m, int which, const do
   const UniformGeom ug = uniform_geom(m);
   const double h = ug.h, s = which == 0 ? h * (5.0 / 3.0) : (which == 1 ? h * h * kLineDerivScale : h * h * h);
   const int64_t n = tile_count(ug) * 32;
-  k_tile_table<<<unsigned((n + 255) / 256), 256, 0, ctx->stream>>>(c, which == 1 ? 3 : 1, s, out, (ug.nx + 7) / 8,
-                                                                   (ug.ny + 3) / 4, ug);
+  k_tile_table<true><<<unsigned((n + 255) / 256), 256, 0, ctx->stream>>>(c, which == 1 ? 3 : 1, s, out, (ug.nx + 7) / 8,
+                                                                         (ug.ny + 3) / 4, ug);
+  ctx->launches++;
+  MF_CUDA_TRY(cudaGetLastError());
+  return MF_OK;
+}
+
+mf_status launch_tile_table_plain(mf_ctx* ctx, const mf_dofmap* m, const double* c, int rows, double scale, float* out) {
+  const UniformGeom ug = uniform_geom(m);
+  const int64_t n = tile_count(ug) * 32;
+  k_tile_table<false><<<unsigned((n + 255) / 256), 256, 0, ctx->stream>>>(c, rows, scale, out, (ug.nx + 7) / 8,
+                                                                          (ug.ny + 3) / 4, ug);
   ctx->launches++;
   MF_CUDA_TRY(cudaGetLastError());
   return MF_OK;

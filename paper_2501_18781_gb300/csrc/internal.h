@@ -117,6 +117,8 @@ constexpr int kScalarsHeat = 2560;   // 8
 constexpr int kScalarsTri = 3072;    // Oseen block-triangular inner solves: 2 (k + 1) + 8 <= 512
 constexpr int kScalarsCGSteps = 3584;  // 64 step counters of the batched CG's on-device stopping test
 constexpr int kScalarsTotal = 4096;
+constexpr int kBarrierCounter = 64;    // counters: {arrived, generation, timed out} of the grid barrier
+constexpr int kCounters = 72;
 }  // namespace mf
 
 struct mf_ctx {
@@ -126,7 +128,7 @@ struct mf_ctx {
   int64_t launches = 0;
   int sm_count = 0;
   mf::DevBuf scratch;   // reduction partials (fixed size, allocated with the context)
-  mf::DevBuf counters;  // 64 arrival counters of the reductions (zero between launches)
+  mf::DevBuf counters;  // 64 arrival counters of the reductions (zero between launches), the grid barrier
   mf::DevBuf scalars;   // device scalars of the solvers
   double* host_scalars = nullptr;  // pinned
   // CUDA graphs are captured on a private stream (the legacy default stream cannot be

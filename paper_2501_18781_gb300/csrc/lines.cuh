@@ -42,6 +42,19 @@ template <typename T> __device__ __forceinline__ void line_deriv_t(const T& f0, 
   r1 = r1 - T(4) * e;
   r2 = (r2 + s) + T(2) * e;
 }
+// one line of a Q1 function: end values -> the three Gauss points
+template <typename T> __device__ __forceinline__ void line_q1(const T& p0, const T& p1, T& v0, T& v1, T& v2) {
+  const T d = p1 - p0;
+  v1 = T(0.5) * (p0 + p1);
+  v0 = v1 - T(kLineDelta) * d;
+  v2 = v1 + T(kLineDelta) * d;
+}
+// its transpose with the Gauss weights (5, 8, 5) / 18
+template <typename T> __device__ __forceinline__ void line_q1_t(const T& g0, const T& g1, const T& g2, T& o0, T& o1) {
+  const T a = T(5.0 / 36.0) * (g0 + g2) + T(8.0 / 36.0) * g1, b = T(kLineDelta * 5.0 / 18.0) * (g2 - g0);
+  o0 = a - b;
+  o1 = a + b;
+}
 // Gauss points -> nodes of a test side with values v and derivative fluxes f: the transposed values of
 // v + stencil^T f, both transposes sharing their sums and differences
 template <typename T>

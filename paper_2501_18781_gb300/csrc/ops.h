@@ -68,6 +68,12 @@ mf_status launch_oseen_coupling_f32(mf_ctx* ctx, const mf_dofmap* mu, int which,
 // inverses of the 3 x 3 nodal blocks, entry-major; S: stencil_halves(n_p) fp16 entries in the
 // scaled tiled layout of stencil_at, scale: n_p row factors; both overwritten)
 mf_status launch_schur_assemble_f32(mf_ctx* ctx, const mf_dofmap* mu, const float* blk, void* S, float* scale);
+// x = S~^-1 b by Jacobi-CG from 0 in one cooperative launch, zout = -x (fp64): at most maxit steps, to
+// |r|^2 <= tol2 |b|^2; work 4 n_p floats, w n_p floats, *steps += the steps taken.  A grid barrier that
+// waits for a second gives up and sets a flag: schur_cg_take_error, after the stream has synchronised.
+mf_status launch_schur_cg(mf_ctx* ctx, const void* S, const float* scale, const float* dinv, const double* b, float* x,
+                          float* work, float* w, double* zout, int nx, int ny, int nz, int maxit, double tol2, double* steps);
+mf_status schur_cg_take_error(mf_ctx* ctx);
 // Gauss-point tables from nodal fp64 fields (always evaluated in fp64, stored in both precisions)
 // (heat: rhocp_q / beta_q are the optional per-Gauss-point fields; qmass gets rhocp_q / dt)
 mf_status launch_scalar_qtables(mf_ctx* ctx, const mf_dofmap* m, int kind, const double* field, const double* kq_user,
@@ -134,6 +140,7 @@ mf_status tc_take_error();
 // accumulated, nrhs <= 65535 vectors ld apart, b and qm may be NULL
 int64_t tile_table_floats(const mf_dofmap* m, int rows);
 mf_status launch_tile_table(mf_ctx* ctx, const mf_dofmap* m, int which, const double* c, float* out);
+mf_status launch_tile_table_plain(mf_ctx* ctx, const mf_dofmap* m, const double* c, int rows, double scale, float* out);
 mf_status launch_scalar_f32_uniform(mf_ctx* ctx, const mf_dofmap* m, const float* src, float* dst, int nrhs, int64_t ld,
                                     const float* c, const float* b, const float* qm, double mass, bool transpose);
 // fp32 reinitialisation apply to 2..8 right-hand sides on an octree map: per leaf in processing order its
@@ -155,6 +162,12 @@ mf_status launch_scalar_df_uniform(mf_ctx* ctx, const mf_dofmap* m, const double
 // table, [3][27][ncells]); dst zeroed by the caller, Dirichlet rows left alone
 mf_status launch_reinit_df_octree(mf_ctx* ctx, const mf_dofmap* m, const double* src, double* dst, int nrhs,
                                   int64_t ld, const float2* n, double eps, double mass);
+// fp32 Oseen apply on uniform meshes from per-tile tables (launch_oseen_f32_tables from the folded fp64
+// tables; nr: the melt-pool interface normal, or NULL); dst accumulated, Dirichlet rows written
+mf_status launch_oseen_f32_tables(mf_ctx* ctx, const mf_dofmap* mu, const double* cm64, const double* cv64,
+                                  const double* cb64, const double* nr64, float* cm, float* cv, float* cb, float* nr);
+mf_status launch_oseen_f32_uniform(mf_ctx* ctx, const mf_dofmap* mu, const float* src, float* dst, const float* cm,
+                                   const float* cv, const float* cb, const float* nr);
 // double-float Oseen apply on uniform meshes: the folded coefficient tables cm, cv (27 per cell) and
 // cb (81 per cell) as float pairs from launch_oseen_df_split; nr: the melt-pool interface normal table
 // (81 per cell, pairs) for the trace correction, or NULL without the melt-pool terms
@@ -202,7 +215,8 @@ struct mf_op {
   mf::DevBuf qcoef_df;              // [27][ncells] float pairs of the scalar coefficient (double-float kernels)
   mf::DevBuf qvec_df;               // [3][27][ncells] float pairs of the convection (heat) or the normal (reinit)
   bool df_ready = false;
-  mf::DevBuf tile_c, tile_b, tile_m;   // fp32 uniform kernel: coefficient tables per tile of cells
+  mf::DevBuf tile_c, tile_b, tile_m;   // fp32 uniform kernels: coefficient tables per tile of cells (Oseen: cm, cb, cv)
+  mf::DevBuf tile_n;                   // Oseen melt-pool terms: the interface normal per tile
   bool tiles_ready = false;
   bool general_f32 = false;            // mf_autotune: time the general kernel
   mf::DevBuf rhs_map, rhs_nrm;         // fp32 octree kernel for several right-hand sides: per-leaf tables

@@ -7,17 +7,41 @@
 namespace mf {
 namespace {
 
-__device__ __forceinline__ double block_sum(double v) {
-  __shared__ double sh[kRedThreads / 32];
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
+// Sums over a block of kRedThreads threads.  GB300's fp64 pipe takes 16 cycles of an SM per warp
+// instruction, so a shuffle tree over every warp (five adds each) costs more than the data of a small
+// vector: the threads' values go to shared memory, and one warp per value adds eight of them per lane
+// before its shuffles (13 fp64 adds instead of 43; a 257 k element fp32 dot 14.7 -> 8.8 us with the grid cut
+// to the vector and 16-byte loads, the fp32 multidot of 5 vectors of 1.6 M 19.9 -> 12.1 us).  N values share the barrier; value k is summed by warp
+// k in a fixed order and given to put(k, sum) by its first lane.  Every thread of the block calls this.
+__device__ __forceinline__ double (*red_area1())[kRedThreads] {   // one area for every instance in a kernel
+  __shared__ double sh[1][kRedThreads];
+  return sh;
+}
+__device__ __forceinline__ double (*red_area())[kRedThreads] {
+  __shared__ double sh[kRedThreads / 32][kRedThreads];
+  return sh;
+}
+template <int N, typename F> __device__ __forceinline__ void block_sums(const double (&v)[N], F&& put) {
+  static_assert(N <= kRedThreads / 32, "one warp per value");
+  double(*sh)[kRedThreads] = N == 1 ? red_area1() : red_area();
+#pragma unroll
+  for (int k = 0; k < N; ++k) sh[k][threadIdx.x] = v[k];
   __syncthreads();
-  double s = 0.0;
-  if (threadIdx.x < 32) {
-    s = threadIdx.x < kRedThreads / 32 ? sh[threadIdx.x] : 0.0;
+  if (threadIdx.x < 32 * N) {
+    const int k = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    double s = sh[k][lane];
+#pragma unroll
+    for (int j = 1; j < kRedThreads / 32; ++j) s += sh[k][lane + 32 * j];
+#pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    if (lane == 0) put(k, s);
   }
   __syncthreads();
+}
+__device__ __forceinline__ double block_sum(double v) {
+  double s = 0.0;
+  const double a[1] = {v};
+  block_sums<1>(a, [&](int, double t) { s = t; });
   return s;  // valid in thread 0
 }
 
@@ -39,8 +63,42 @@ struct Dot2f {
     c += ((s - (t - z)) + (p - z)) + e;
     s = t;
   }
+  // the sum of both pairs
+  __device__ __forceinline__ void merge(float os, float oc) {
+    const float t = s + os;
+    const float z = t - s;
+    c += oc + ((s - (t - z)) + (os - z));
+    s = t;
+  }
+  __device__ __forceinline__ void merge(const Dot2f& o) { merge(o.s, o.c); }
+  // lane 0: the sum over the warp (pairs of floats: no fp64 instruction)
+  __device__ __forceinline__ void warp_sum() {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+      merge(__shfl_down_sync(0xffffffffu, s, o), __shfl_down_sync(0xffffffffu, c, o));
+  }
   __device__ __forceinline__ double value() const { return double(s) + double(c); }
 };
+
+// The same for pairs: summed over each warp as pairs, then the warps' sums in fp64.
+template <int N, typename F> __device__ __forceinline__ void block_sums(Dot2f (&v)[N], F&& put) {
+  static_assert(N <= kRedThreads / 32, "one warp per value");
+  __shared__ double sh[N][kRedThreads / 32];
+#pragma unroll
+  for (int k = 0; k < N; ++k) v[k].warp_sum();
+  if ((threadIdx.x & 31) == 0)
+#pragma unroll
+    for (int k = 0; k < N; ++k) sh[k][threadIdx.x >> 5] = v[k].value();
+  __syncthreads();
+  if (threadIdx.x < 32 * N) {
+    const int k = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    double s = lane < kRedThreads / 32 ? sh[k][lane] : 0.0;
+#pragma unroll
+    for (int o = kRedThreads / 64; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    if (lane == 0) put(k, s);
+  }
+  __syncthreads();
+}
 
 // What the sum of a row of g partials feeds (row r; mode 0: out[r] = sum; 1: pAp and alpha;
 // 2: rr, rz (second row), beta; 3: rz and beta; 4: rr and rz; 5: rr).  count: one arrival

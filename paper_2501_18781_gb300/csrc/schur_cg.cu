@@ -1,0 +1,324 @@
+// The Schur complement solve of the Oseen block-triangular preconditioner in one launch: Jacobi-
+// preconditioned CG on the assembled 125-point pressure stencil, fp32 vectors, fp64 scalars.
+//
+// Run as separate kernels, a step was four launches on vectors that fit in L2 (40^3 cells: 69 k rows, 33 us
+// per step in the launch list of a melt-pool step), and the steps after convergence still launched.  Here
+// one cooperative grid holds the whole iteration, one block of 1024 threads per SM, with two grid barriers
+// per step: the inner products of a step are gathered together (the single-reduction form of CG of
+// Chronopoulos and Gear, J. Comput. Appl. Math. 25, 1989: s = A p is updated with A z instead of
+// recomputed), and every block adds the per-block partial sums in the same order, so all blocks hold the
+// same scalars and the result does not depend on timing.  A barrier gives up after one second of
+// %globaltimer and sets a flag.
+// Bound: latency of the barriers and of the two dependent passes, 12 us per step at 40^3 (351 us per
+// call); the 40^3 step's Schur solves went from 30 to 10 ms.  The fp64 scalars are one thread's work:
+// divisions in all 32 warps took 8 us per step, the fp64 sums over all of them 5 us.
+#include <cuda_fp16.h>
+
+#include <cstring>
+
+#include "ops.h"
+#include "reduce.cuh"
+
+namespace mf {
+namespace {
+
+constexpr int kThreads = 1024;
+constexpr size_t kCoefBytes = size_t(200) << 10;   // coefficients a block may keep in shared memory
+
+// Barrier over the whole (co-resident) grid; bar = {arrived, generation, timed out}.  The release of the
+// arrival and the acquire of the new generation order the blocks' global memory accesses.
+__device__ __forceinline__ unsigned load_acquire(const unsigned* p) {
+  unsigned v;
+  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ bool grid_barrier(unsigned* bar, unsigned nblocks) {
+  __shared__ bool ok;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    ok = true;
+    const unsigned gen = load_acquire(bar + 1);
+    unsigned before;
+    asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], 1;" : "=r"(before) : "l"(bar) : "memory");
+    if (before == nblocks - 1) {
+      bar[0] = 0u;
+      asm volatile("red.add.release.gpu.global.u32 [%0], 1;" ::"l"(bar + 1) : "memory");
+    } else {
+      unsigned long long t0 = 0;
+      for (unsigned spins = 0; load_acquire(bar + 1) == gen; ++spins) {
+        if ((spins & 1023u) != 1023u) continue;
+        unsigned long long t;
+        asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+        if (!t0) t0 = t;
+        if (t - t0 > 1000000000ull || load_acquire(bar + 2)) {
+          atomicExch(bar + 2, 1u);
+          ok = false;
+          break;
+        }
+      }
+    }
+  }
+  __syncthreads();
+  return ok;
+}
+
+// Block sums of N values, value k to part[k * stride + blockIdx.x].  Pairs of floats down to one value per
+// warp: fp64 adds cost 16 cycles of the SM per warp instruction (a tree of them over the block's 32 warps
+// took longer than the step's stencil).
+template <int N> __device__ __forceinline__ void block_partials(Dot2f (&v)[N], double (*sh)[32], double* part, int64_t stride) {
+#pragma unroll
+  for (int k = 0; k < N; ++k) v[k].warp_sum();
+  if ((threadIdx.x & 31) == 0)
+#pragma unroll
+    for (int k = 0; k < N; ++k) sh[k][threadIdx.x >> 5] = v[k].value();
+  __syncthreads();
+  if (threadIdx.x < 32 * N) {
+    const int k = threadIdx.x >> 5;
+    double s = sh[k][threadIdx.x & 31];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    if ((threadIdx.x & 31) == 0) part[k * stride + blockIdx.x] = s;
+  }
+}
+
+struct SchurArgs {
+  const __half* S;      // scaled fp16 tiled layout of stencil_at
+  const float* scale;
+  const float* dinv;
+  const double* b;     // right-hand side
+  float *x, *r, *z, *p, *s, *w;
+  double* zout;        // -x in fp64
+  double* part;        // partial sums: [2][2][grid] (r.r, r.z by step parity), then [grid] (z.w)
+  double* steps;       // step counter over all solves
+  unsigned* bar;
+  double tol2;
+  int nx, ny, nz, maxit;
+};
+
+// Words K0 .. K0 + K - 1 (8 entries each) of stencil row i times v; w: the row's first word (words 32 apart, the
+// scaled fp16 tiled layout of stencil_at).  Entries toward nodes outside the grid are 0, and their loads
+// are clamped into it; v changes during the launch: plain loads.
+template <int K0, int K>
+__device__ __forceinline__ float stencil_words(const SchurArgs& A, const uint4* w, const float* v, int i) {
+  const int px = A.nx + 1, pxy = px * (A.ny + 1);
+  const int ix = i % px, iy = (i / px) % (A.ny + 1), iz = i / pxy;
+  int ox[5], oy[5], oz[5];
+#pragma unroll
+  for (int d = 0; d < 5; ++d) {
+    ox[d] = min(max(ix + d - 2, 0), A.nx);
+    oy[d] = px * min(max(iy + d - 2, 0), A.ny);
+    oz[d] = pxy * min(max(iz + d - 2, 0), A.nz);
+  }
+  float s0 = 0.f, s1 = 0.f;
+#pragma unroll
+  for (int c = 0; c < K / 4; ++c) {
+    uint4 q[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) q[k] = w[32 * (4 * c + k)];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const uint32_t pair[4] = {q[k].x, q[k].y, q[k].z, q[k].w};
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        __half2 h2;
+        memcpy(&h2, &pair[j], 4);
+        const float2 f = __half22float2(h2);
+        const int o = 8 * (K0 + 4 * c + k) + 2 * j;
+        if (o < 125) s0 = fmaf(f.x, v[ox[o % 5] + oy[(o / 5) % 5] + oz[o / 25]], s0);
+        if (o + 1 < 125) s1 = fmaf(f.y, v[ox[(o + 1) % 5] + oy[((o + 1) / 5) % 5] + oz[(o + 1) / 25]], s1);
+      }
+    }
+  }
+  return s0 + s1;
+}
+
+// PARTS threads share a row (warp by warp, so that every thread's entries are known at compile time).  CACHED:
+// the block's coefficients stay in shared memory for the whole solve.
+template <int PARTS, bool CACHED>
+__global__ void __launch_bounds__(kThreads, 1) k_schur_cg(const SchurArgs A) {
+  extern __shared__ uint4 coef[];
+  __shared__ double sh[2][32], tot[3];
+  __shared__ float coefs[2];
+  __shared__ bool done;
+  __shared__ float ssum[PARTS > 1 ? PARTS : 1][kThreads / PARTS];
+  constexpr int kRows = kThreads / PARTS, kWords = 16 / PARTS;   // rows of a block at a time, words of a thread
+  const int np = (A.nx + 1) * (A.ny + 1) * (A.nz + 1);
+  const int part = threadIdx.x / kRows, local = threadIdx.x % kRows;
+  const unsigned G = gridDim.x;
+  // rows of this block: consecutive runs of kRows
+  const int first = blockIdx.x * kRows, step = int(G) * kRows;
+  const int t0 = first + int(threadIdx.x);
+  const bool own = threadIdx.x < kRows;   // the thread that keeps the row's vectors
+  auto words = [&](int i) { return reinterpret_cast<const uint4*>(A.S + stencil_at(0, i)); };
+  if (CACHED) {
+    int run = 0;
+    for (int i0 = first; i0 < np; i0 += step, ++run) {
+      const uint4* const g = words(i0);   // kRows is a multiple of 32: the run's rows are consecutive tiles
+      const int n = (min(kRows, np - i0) + 31) / 32 * 512;
+      for (int q = threadIdx.x; q < n; q += kThreads) coef[run * (kRows * 16) + q] = __ldg(g + q);
+    }
+    __syncthreads();
+  }
+  // w = S~ z on the block's rows, and the thread's share of z . w
+  auto apply = [&](Dot2f& azw) {
+    int run = 0;
+    for (int i0 = first; i0 < np; i0 += step, ++run) {
+      const int i = i0 + local;
+      float s = 0.f;
+      if (i < np) {
+        const uint4* const q = (CACHED ? coef + run * (kRows * 16) + (local >> 5) * 512 + (local & 31) : words(i)) +
+                               32 * kWords * part;
+        if (PARTS == 1) s = stencil_words<0, kWords>(A, q, A.z, i);
+        else if (part == 0) s = stencil_words<0, kWords>(A, q, A.z, i);
+        else if (part == 1) s = stencil_words<kWords % 16, kWords>(A, q, A.z, i);
+        else if (part == 2) s = stencil_words<2 * kWords % 16, kWords>(A, q, A.z, i);
+        else s = stencil_words<3 * kWords % 16, kWords>(A, q, A.z, i);
+      }
+      if (PARTS > 1) {
+        ssum[part][local] = s;
+        __syncthreads();
+        if (own) {
+          s = ssum[0][local];
+#pragma unroll
+          for (int k = 1; k < PARTS; ++k) s += ssum[k][local];
+        }
+      }
+      if (own && i < np) {
+        const float w = A.scale[i] * s;
+        A.w[i] = w;
+        azw.add(A.z[i], w);
+      }
+      if (PARTS > 1) __syncthreads();
+    }
+  };
+  // fixed-order sums of the blocks' partials, the same in every block: warp k adds array k
+  auto totals = [&](int parity) {
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (w < 3) {
+      const double* q = w < 2 ? A.part + (2 * parity + w) * int64_t(G) : A.part + 4 * int64_t(G);
+      double s = 0.0;
+      for (unsigned k = lane; k < G; k += 32) s += __ldcg(q + k);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+      if (lane == 0) tot[w] = s;
+    }
+    __syncthreads();
+  };
+  Dot2f arr, arz;
+  if (own)
+    for (int i = t0; i < np; i += step) {
+      const float r = float(A.b[i]), z = A.dinv[i] * r;
+      A.r[i] = r;
+      A.z[i] = z;
+      A.x[i] = 0.f;
+      arr.add(r, r);
+      arz.add(r, z);
+    }
+  double rz_old = 1.0, alpha = 0.0, stop = 0.0;   // thread 0 of every block
+  int k = 0;
+  for (; k < A.maxit; ++k) {
+    Dot2f v2[2] = {arr, arz};
+    block_partials<2>(v2, sh, A.part + 2 * (k & 1) * int64_t(G), G);
+    if (!grid_barrier(A.bar, G)) return;
+    Dot2f v1[1];
+    apply(v1[0]);
+    block_partials<1>(v1, sh, A.part + 4 * int64_t(G), G);
+    if (!grid_barrier(A.bar, G)) return;
+    totals(k & 1);
+    if (threadIdx.x == 0) {   // fp64 divisions by one thread, not by 32 warps
+      const double rr = tot[0], rz = tot[1], zw = tot[2];
+      if (k == 0) stop = A.tol2 * rr;
+      const double beta = k ? rz / rz_old : 0.0;
+      const double pap = k ? zw - beta * rz / alpha : zw;   // p.A p of p = z + beta p
+      // converged (or a zero right-hand side), or a breakdown: x stays as it is
+      done = rr <= stop || !(pap > 0.0);
+      alpha = rz / pap;
+      rz_old = rz;
+      coefs[0] = float(alpha);
+      coefs[1] = float(beta);
+    }
+    __syncthreads();
+    if (done) break;
+    const float al = coefs[0], be = coefs[1];
+    arr = Dot2f();
+    arz = Dot2f();
+    if (own)
+      for (int i = t0; i < np; i += step) {
+        const float p = k ? A.z[i] + be * A.p[i] : A.z[i], s = k ? A.w[i] + be * A.s[i] : A.w[i];
+        const float r = A.r[i] - al * s, z = A.dinv[i] * r;
+        A.p[i] = p;
+        A.s[i] = s;
+        A.x[i] += al * p;
+        A.r[i] = r;
+        A.z[i] = z;
+        arr.add(r, r);
+        arz.add(r, z);
+      }
+  }
+  if (own)
+    for (int i = t0; i < np; i += step) A.zout[i] = -double(A.x[i]);
+  if (blockIdx.x == 0 && threadIdx.x == 0) *A.steps += double(k);
+}
+
+template <int PARTS> cudaError_t start(mf_ctx* ctx, SchurArgs& a, int64_t np) {
+  constexpr int rows = kThreads / PARTS;
+  const int64_t want = (np + rows - 1) / rows;
+  const unsigned grid = unsigned(want < ctx->sm_count ? want : ctx->sm_count);
+  const size_t runs = size_t((want + grid - 1) / grid), bytes = runs * rows * 256;
+  const bool cached = bytes <= kCoefBytes;
+  const void* const k = cached ? reinterpret_cast<const void*>(k_schur_cg<PARTS, true>)
+                               : reinterpret_cast<const void*>(k_schur_cg<PARTS, false>);
+  if (cached) {
+    const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kCoefBytes));
+    if (e != cudaSuccess) return e;
+  }
+  void* args[] = {&a};
+  return cudaLaunchCooperativeKernel(k, dim3(grid), dim3(kThreads), args, cached ? bytes : 0, ctx->stream);
+}
+
+}  // namespace
+
+// zout = -x and x = S~^-1 b by at most maxit steps from 0, to ||r|| <= sqrt(tol2) ||b||.  work: 4 n_p
+// floats (r, z, p, s).
+mf_status launch_schur_cg(mf_ctx* ctx, const void* S, const float* scale, const float* dinv, const double* b, float* x,
+                          float* work, float* w, double* zout, int nx, int ny, int nz, int maxit, double tol2, double* steps) {
+  const int64_t np = int64_t(nx + 1) * (ny + 1) * (nz + 1);
+  SchurArgs a{};
+  a.S = static_cast<const __half*>(S);
+  a.scale = scale;
+  a.dinv = dinv;
+  a.b = b;
+  a.x = x;
+  a.r = work;
+  a.z = work + np;
+  a.p = work + 2 * np;
+  a.s = work + 3 * np;
+  a.w = w;
+  a.zout = zout;
+  a.part = ctx->scratch.as<double>();
+  a.steps = steps;
+  a.bar = ctx->counters.as<unsigned>() + kBarrierCounter;
+  a.tol2 = tol2;
+  a.nx = nx;
+  a.ny = ny;
+  a.nz = nz;
+  a.maxit = maxit;
+  // as many threads per row as the grid has to spare
+  const int64_t threads = int64_t(ctx->sm_count) * kThreads;
+  MF_CUDA_TRY(4 * np <= threads ? start<4>(ctx, a, np) : (2 * np <= threads ? start<2>(ctx, a, np) : start<1>(ctx, a, np)));
+  ctx->launches++;
+  return MF_OK;
+}
+
+// MF_ETIMEOUT (once, then the barrier is reset) if a launch's barrier gave up
+mf_status schur_cg_take_error(mf_ctx* ctx) {
+  unsigned bar[3] = {0u, 0u, 0u};
+  unsigned* const d = ctx->counters.as<unsigned>() + kBarrierCounter;
+  MF_CUDA_TRY(cudaMemcpyAsync(bar, d, sizeof bar, cudaMemcpyDeviceToHost, ctx->stream));
+  MF_CUDA_TRY(cudaStreamSynchronize(ctx->stream));
+  if (!bar[2]) return MF_OK;
+  MF_CUDA_TRY(cudaMemsetAsync(d, 0, sizeof bar, ctx->stream));
+  return fail(MF_ETIMEOUT, "a grid barrier of the Schur complement solve timed out");
+}
+
+}  // namespace mf

@@ -30,8 +30,6 @@ double value_coef(const mf_op* op);
 template <typename T> ScalarArgs<T> scalar_args(const mf_op* op, const T* src, T* dst, int nrhs, int64_t ld);
 template <typename T> mf_status oseen_coupling(mf_op* op, int which, const T* src, T* dst);
 // device-side stopping test and Givens kernels of the inner solves (solver_kernels.cu)
-mf_status dev_cg_tol_init(mf_ctx* c, double* S, double tol2);
-mf_status dev_cg_tol_check(mf_ctx* c, double* S, double* steps);
 mf_status dev_cg_tol_init_batched(mf_ctx* c, double* S, double tol2, int nrhs);
 mf_status dev_cg_tol_check_batched(mf_ctx* c, double* S, double* steps, int nrhs);
 mf_status dev_gmres_begin(mf_ctx* c, const double* nrm2, double* G, int m);
@@ -197,7 +195,7 @@ struct OseenBlockTri {
   int64_t n = 0, nu = 0, nu3 = 0, np = 0;
   int ku = 10, smax = 30;
   double stol = 0.1;
-  Vec<float> blk32, ua, pinv32, xp, rp, zp, pp, sp, V, t, w;
+  Vec<float> blk32, ua, pinv32, xp, sp, cgw, V, t, w;
   DevBuf stil;        // S~ = B D^-1 B^T as a 125-point stencil on the pressure grid (fp16 entries)
   Vec<float> stscale;  // and its row factors
   int gn[3] = {0, 0, 0};  // cells per axis
@@ -229,7 +227,8 @@ struct OseenBlockTri {
     // fp32 3x3 block inverses and inverse pressure scaling, computed in fp32 (the preconditioner
     // applies them in fp32)
     MF_TRY(blk32.alloc(9 * nu));
-    for (Vec<float>* v : {&pinv32, &xp, &rp, &zp, &pp, &sp}) MF_TRY(v->alloc(np));
+    for (Vec<float>* v : {&pinv32, &xp, &sp}) MF_TRY(v->alloc(np));
+    MF_TRY(cgw.alloc(4 * np));
     MF_TRY(oseen_blocks32(op, blk32.p, pinv32.p));
     for (int d = 0; d < 3; ++d) gn[d] = op->map[0]->mesh->n[d];
     MF_TRY(stil.alloc(2 * size_t(stencil_halves(np))));
@@ -252,25 +251,11 @@ struct OseenBlockTri {
   // device counter of the Schur CG steps taken while still iterating, over all calls
   double* schur_steps() { return op->ctx->scalars.as<double>() + kScalarsTri + 144; }
 
-  // xp = S~^-1 r_p (r_p fp64): Jacobi-PCG from 0, smax steps; once ||r_k|| <= stol ||r_0|| (or
-  // p.S~p <= 0) the remaining steps' kernels return at once and x stays as it is.
-  mf_status schur_solve(const double* r) {
-    mf_ctx* c = op->ctx;
-    double* S = c->scalars.as<double>() + kScalarsTri + 128;
-    MF_CUDA_TRY(cudaMemsetAsync(xp.p, 0, sizeof(float) * np, c->stream));
-    MF_TRY((convert<double, float>(c, np, r, rp.p)));
-    MF_TRY(pointwise_mul<float>(c, np, pinv32.p, rp.p, zp.p));
-    MF_CUDA_TRY(cudaMemcpyAsync(pp.p, zp.p, sizeof(float) * np, cudaMemcpyDeviceToDevice, c->stream));
-    MF_TRY(cg_init_scalars<float>(c, rp.p, zp.p, np, np, 1, S));
-    MF_TRY(dev_cg_tol_init(c, S, stol * stol));
-    for (int k = 0; k < smax; ++k) {
-      // sp = S~ pp and alpha in one launch
-      MF_TRY(stencil125_apply(c, stil.p, stscale.p, pp.p, sp.p, gn[0], gn[1], gn[2], S));
-      MF_TRY(cg_update_xr<float>(c, np, np, 1, xp.p, rp.p, pp.p, sp.p, pinv32.p, zp.p, 1, S, true));
-      MF_TRY(dev_cg_tol_check(c, S, schur_steps()));
-      MF_TRY(cg_update_p<float>(c, np, np, 1, zp.p, pp.p, S, true));
-    }
-    return MF_OK;
+  // xp = S~^-1 r_p (r_p fp64) and z_p = -xp: Jacobi-PCG from 0 in one launch, at most smax steps; once
+  // ||r_k|| <= stol ||r_0|| (or p.S~p <= 0) x stays as it is.
+  mf_status schur_solve(const double* r, double* z) {
+    return launch_schur_cg(op->ctx, stil.p, stscale.p, pinv32.p, r, xp.p, cgw.p, sp.p, z, gn[0], gn[1], gn[2], smax,
+                           stol * stol, schur_steps());
   }
 
   // z_u = A^-1 rhs_u (z fp64) by ku steps of GMRES from 0, right-preconditioned by D^-1.  rhs
@@ -322,9 +307,8 @@ struct OseenBlockTri {
   // z = P^-1 r (fp64 vectors of length n)
   mf_status apply(const double* r, double* z) {
     mf_ctx* c = op->ctx;
-    MF_TRY(schur_solve(r + nu3));
-    // z_p = -x_p; velocity right-hand side r_u - B^T z_p = r_u + B^T x_p
-    MF_TRY((axpby<float, double>(c, np, -1.0, xp.p, 0.0, z + nu3)));
+    MF_TRY(schur_solve(r + nu3, z + nu3));
+    // velocity right-hand side r_u - B^T z_p = r_u + B^T x_p
     MF_TRY(oseen_coupling<float>(op, 0, xp.p, ua.p));
     MF_TRY((axpby<double, float>(c, nu3, 1.0, r, 0.0, w.p)));
     MF_TRY((axpby<float, float>(c, nu3, 1.0, ua.p, 1.0, w.p)));
@@ -891,6 +875,7 @@ mf_status solve_impl(mf_op* op, const mf_solver_params* sp, const double* b, dou
     }
     if (P.tri) {
       MF_TRY(sync_copy(c, c->host_scalars + kScalarsTri + 144, P.tri->schur_steps(), 1));
+      MF_TRY(schur_cg_take_error(c));
       inf.inner_steps = int(c->host_scalars[kScalarsTri + 144]);
     }
   } else if (sp->solver == MF_SOLVER_DEFECT_CORRECTION) {
@@ -1216,6 +1201,7 @@ mf_status autotune_measure(mf_op* op) {
         }
       }
       op->df64_faster = df_ms < std::min(ms[0], ms[1]);
+      MF_TRY(prepare_f32_applies(op));
       cudaEventDestroy(a0);
       cudaEventDestroy(a1);
       char buf[256];

@@ -39,19 +39,9 @@ __global__ void k_add_scaled(const float* d, double* x, const double* sc, int64_
     x[o + i] += s * double(d[o + i]);
 }
 
-// Inner solves of the Oseen block preconditioner without host round trips: the stopping test
-// of a CG and the Givens/back-substitution of a fixed-length GMRES run in one-thread kernels
-// on device scalars.
-__global__ void k_cg_tol_init(double* S, double tol2) {
-  S[S_ACTIVE] = S[S_RR] > 0.0 ? 1.0 : 0.0;
-  S[7] = tol2 * S[S_RR];
-}
-// steps: counts the steps that ran while the CG was still iterating (may be NULL)
-__global__ void k_cg_tol_check(double* S, double* steps) {
-  if (steps && S[S_ACTIVE] != 0.0) steps[0] += 1.0;
-  if (S[S_RR] <= S[7] || !(S[S_PAP] > 0.0)) S[S_ACTIVE] = 0.0;
-}
-// the same for the nrhs systems of the batched CG (one thread each; a system already stopped by the
+// The stopping test of a CG and the Givens/back-substitution of a fixed-length GMRES without host round
+// trips, in one-thread kernels on device scalars.
+// The nrhs systems of the batched CG (one thread each; a system already stopped by the
 // host stays stopped): the threshold tol2 ||r_0||^2 into slot 7, then per iteration the step count
 // and the stopping test
 __global__ void k_cg_tol_init_batched(double* S, double tol2, int nrhs) {
@@ -145,14 +135,6 @@ mf_status dev_add_scaled(mf_ctx* c, const float* d, double* x, const double* sca
   LAUNCHED();
 }
 
-mf_status dev_cg_tol_init(mf_ctx* c, double* S, double tol2) {
-  k_cg_tol_init<<<1, 1, 0, c->stream>>>(S, tol2);
-  LAUNCHED();
-}
-mf_status dev_cg_tol_check(mf_ctx* c, double* S, double* steps) {
-  k_cg_tol_check<<<1, 1, 0, c->stream>>>(S, steps);
-  LAUNCHED();
-}
 mf_status dev_cg_tol_init_batched(mf_ctx* c, double* S, double tol2, int nrhs) {
   k_cg_tol_init_batched<<<1, 64, 0, c->stream>>>(S, tol2, nrhs);
   LAUNCHED();

@@ -18,137 +18,163 @@ __global__ void __launch_bounds__(kRedThreads) k_finish(const double* part, int 
   finish_row(part, g, blockIdx.x, Finish{out, mode, S, nullptr});
 }
 
-// Per-block partial sums of x.y (and x2.y2).  Each thread keeps four independent
-// accumulators over elements one grid stride apart, so four loads per vector are in flight
-// per thread (enough bytes in flight to approach HBM bandwidth with one block per warp slot);
-// the partition and the summation order are fixed, so results are reproducible bit for bit.
-template <typename TX, typename TY>
-__global__ void __launch_bounds__(kRedThreads) k_dot2_partial(const TX* x, const TY* y, const TX* x2, const TY* y2,
-                                                             int64_t n, int64_t ld, double* part, Finish fin) {
+// A vector's 16-byte words (W elements), or its elements (W = 1).
+template <typename T, int W> struct alignas(sizeof(T) * W) Word {
+  T c[W];
+};
+template <typename T> struct DotAcc;
+template <> struct DotAcc<float> : Dot2f {};
+template <> struct DotAcc<double> {
+  double s = 0.0;
+  __device__ __forceinline__ void add(double a, double b) { s = fma(a, b, s); }
+  __device__ __forceinline__ void merge(const DotAcc<double>& o) { s += o.s; }
+  __device__ __forceinline__ double value() const { return s; }
+};
+template <int N, typename F> __device__ __forceinline__ void block_sums(DotAcc<float> (&v)[N], F&& put) {
+  Dot2f w[N];
+#pragma unroll
+  for (int k = 0; k < N; ++k) w[k] = v[k];
+  block_sums<N>(w, put);
+}
+template <int N, typename F> __device__ __forceinline__ void block_sums(DotAcc<double> (&v)[N], F&& put) {
+  double w[N];
+#pragma unroll
+  for (int k = 0; k < N; ++k) w[k] = v[k].s;
+  block_sums<N>(w, put);
+}
+
+// Per-block partial sums of x.y (and, TWO, x2.y2).  Each thread keeps an accumulator per element of a
+// 16-byte word (every vector aligned), and two words of each vector in flight; W = 1 where a vector is
+// not aligned, with four elements in flight.  The partition and the summation order are fixed, so results are reproducible
+// bit for bit.
+template <typename T, int W, bool TWO>
+__global__ void __launch_bounds__(kRedThreads) k_dot2_partial(const T* x, const T* y, const T* x2, const T* y2, int64_t n,
+                                                             int64_t ld, double* part, Finish fin) {
+  using V = Word<T, W>;
   const int r = blockIdx.y;
   x += r * ld; y += r * ld;
-  if (x2) { x2 += r * ld; y2 += r * ld; }
-  const int64_t st = int64_t(gridDim.x) * blockDim.x;
-  int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  if constexpr (std::is_same<TX, float>::value && std::is_same<TY, float>::value) {
-    Dot2f a0, a1, a2, a3, b0, b1, b2, b3;
-    for (; i + 3 * st < n; i += 4 * st) {
-      const float p0 = x[i], p1 = x[i + st], p2 = x[i + 2 * st], p3 = x[i + 3 * st];
-      const float q0 = y[i], q1 = y[i + st], q2 = y[i + 2 * st], q3 = y[i + 3 * st];
-      a0.add(p0, q0); a1.add(p1, q1); a2.add(p2, q2); a3.add(p3, q3);
-      if (x2) {
-        b0.add(x2[i], y2[i]); b1.add(x2[i + st], y2[i + st]);
-        b2.add(x2[i + 2 * st], y2[i + 2 * st]); b3.add(x2[i + 3 * st], y2[i + 3 * st]);
+  if (TWO) { x2 += r * ld; y2 += r * ld; }
+  const int64_t st = int64_t(gridDim.x) * blockDim.x, t0 = int64_t(blockIdx.x) * blockDim.x + threadIdx.x, nw = n / W;
+  const V *xw = reinterpret_cast<const V*>(x), *yw = reinterpret_cast<const V*>(y);
+  const V *xw2 = reinterpret_cast<const V*>(x2), *yw2 = reinterpret_cast<const V*>(y2);
+  // words in flight per vector, and accumulators: one per element of a word, or per word of one element
+  constexpr int UN = W == 1 ? 4 : 2, NA = W == 1 ? UN : W;
+  DotAcc<T> a[NA], b[NA];
+  int64_t i = t0;
+  for (; i + (UN - 1) * st < nw; i += UN * st) {
+    V p[UN], q[UN];
+#pragma unroll
+    for (int u = 0; u < UN; ++u) {
+      p[u] = xw[i + u * st];
+      q[u] = yw[i + u * st];
+    }
+#pragma unroll
+    for (int u = 0; u < UN; ++u)
+#pragma unroll
+      for (int c = 0; c < W; ++c) a[W == 1 ? u : c].add(p[u].c[c], q[u].c[c]);
+    if (TWO) {
+#pragma unroll
+      for (int u = 0; u < UN; ++u) {
+        p[u] = xw2[i + u * st];
+        q[u] = yw2[i + u * st];
       }
+#pragma unroll
+      for (int u = 0; u < UN; ++u)
+#pragma unroll
+        for (int c = 0; c < W; ++c) b[W == 1 ? u : c].add(p[u].c[c], q[u].c[c]);
     }
-    for (; i < n; i += st) {
-      a0.add(x[i], y[i]);
-      if (x2) b0.add(x2[i], y2[i]);
-    }
-    const double s = block_sum((a0.value() + a1.value()) + (a2.value() + a3.value()));
-    const double s2 = x2 ? block_sum((b0.value() + b1.value()) + (b2.value() + b3.value())) : 0.0;
-    if (threadIdx.x == 0) {
-      part[int64_t(r) * 2 * gridDim.x + blockIdx.x] = s;
-      part[int64_t(r) * 2 * gridDim.x + gridDim.x + blockIdx.x] = s2;
-    }
-    finish_if_last(part, fin);
-    return;
   }
-  double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0, b0 = 0.0, b1 = 0.0, b2 = 0.0, b3 = 0.0;
-  if (x2) {
-    for (; i + 3 * st < n; i += 4 * st) {
-      const double p0 = double(x[i]), p1 = double(x[i + st]), p2 = double(x[i + 2 * st]), p3 = double(x[i + 3 * st]);
-      const double q0 = double(y[i]), q1 = double(y[i + st]), q2 = double(y[i + 2 * st]), q3 = double(y[i + 3 * st]);
-      const double u0 = double(x2[i]), u1 = double(x2[i + st]), u2 = double(x2[i + 2 * st]), u3 = double(x2[i + 3 * st]);
-      const double v0 = double(y2[i]), v1 = double(y2[i + st]), v2 = double(y2[i + 2 * st]), v3 = double(y2[i + 3 * st]);
-      a0 += p0 * q0; a1 += p1 * q1; a2 += p2 * q2; a3 += p3 * q3;
-      b0 += u0 * v0; b1 += u1 * v1; b2 += u2 * v2; b3 += u3 * v3;
+  for (; i < nw; i += st) {
+    const V p0 = xw[i], q0 = yw[i];
+#pragma unroll
+    for (int c = 0; c < W; ++c) a[c].add(p0.c[c], q0.c[c]);
+    if (TWO) {
+      const V u0 = xw2[i], v0 = yw2[i];
+#pragma unroll
+      for (int c = 0; c < W; ++c) b[c].add(u0.c[c], v0.c[c]);
     }
-    for (; i < n; i += st) {
-      a0 += double(x[i]) * double(y[i]);
-      b0 += double(x2[i]) * double(y2[i]);
-    }
-  } else {
-    for (; i + 3 * st < n; i += 4 * st) {
-      const double p0 = double(x[i]), p1 = double(x[i + st]), p2 = double(x[i + 2 * st]), p3 = double(x[i + 3 * st]);
-      const double q0 = double(y[i]), q1 = double(y[i + st]), q2 = double(y[i + 2 * st]), q3 = double(y[i + 3 * st]);
-      a0 += p0 * q0; a1 += p1 * q1; a2 += p2 * q2; a3 += p3 * q3;
-    }
-    for (; i < n; i += st) a0 += double(x[i]) * double(y[i]);
   }
-  double s = block_sum((a0 + a1) + (a2 + a3));
-  double s2 = x2 ? block_sum((b0 + b1) + (b2 + b3)) : 0.0;
-  if (threadIdx.x == 0) {
-    part[int64_t(r) * 2 * gridDim.x + blockIdx.x] = s;
-    part[int64_t(r) * 2 * gridDim.x + gridDim.x + blockIdx.x] = s2;
+  for (int64_t k = nw * W + t0; k < n; k += st) {   // the last n mod W elements
+    a[0].add(x[k], y[k]);
+    if (TWO) b[0].add(x2[k], y2[k]);
   }
+#pragma unroll
+  for (int c = 1; c < NA; ++c) {
+    a[0].merge(a[c]);
+    if (TWO) b[0].merge(b[c]);
+  }
+  double* const pr = part + int64_t(r) * 2 * gridDim.x + blockIdx.x;
+  const int64_t g = gridDim.x;
+  DotAcc<T> v[TWO ? 2 : 1];
+  v[0] = a[0];
+  if (TWO) v[TWO ? 1 : 0] = b[0];
+  block_sums<TWO ? 2 : 1>(v, [&](int k, double t) { pr[k * g] = t; });
   finish_if_last(part, fin);
 }
 
-template <typename T>
+// ZMODE 1: z = dinv .* r and r.z; 0: r.z = r.r; 2: r.r only
+template <typename T, int W, int ZMODE>
 __global__ void __launch_bounds__(kRedThreads) k_cg_xr(int64_t n, int64_t ld, T* x, T* r, const T* p, const T* Ap,
-                                                       const T* dinv, T* z, int zmode, const double* S, double* part,
-                                                       Finish fin, bool skip_inactive) {
+                                                       const T* dinv, T* z, const double* S, double* part, Finish fin,
+                                                       bool skip_inactive) {
+  using V = Word<T, W>;
   const int rh = blockIdx.y;
   if (skip_inactive && S[rh * S_NSCAL + S_ACTIVE] == 0.0) return;  // this system has stopped
-  const double alpha = S[rh * S_NSCAL + S_ALPHA];
-  const int64_t o = rh * ld;
-  double rr = 0.0, rz = 0.0;
-  if constexpr (std::is_same<T, float>::value) {
-    Dot2f crr, crz;
-    for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x) {
-      const float xi = x[o + i] + float(alpha) * p[o + i];
-      const float ri = r[o + i] - float(alpha) * Ap[o + i];
-      x[o + i] = xi;
-      r[o + i] = ri;
-      crr.add(ri, ri);
-      if (zmode == 1) {
-        const float zi = dinv[i] * ri;
-        z[o + i] = zi;
-        crz.add(ri, zi);
-      } else if (zmode == 0) {
-        crz.add(ri, ri);
-      }
+  const T alpha = T(S[rh * S_NSCAL + S_ALPHA]);
+  const int64_t o = rh * ld, st = int64_t(gridDim.x) * blockDim.x, t0 = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+  x += o; r += o; p += o; Ap += o;
+  if (ZMODE == 1) z += o;
+  DotAcc<T> a[W], b[W];
+  auto elem = [&](T& xi, T& ri, T pi, T ai, T di, T& zi, int c) {
+    xi = xi + alpha * pi;
+    ri = ri - alpha * ai;
+    a[c].add(ri, ri);
+    if (ZMODE == 1) {
+      zi = di * ri;
+      b[c].add(ri, zi);
     }
-    rr = crr.value();
-    rz = crz.value();
-  } else {
-    for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x) {
-      T xi = x[o + i] + T(alpha) * p[o + i];
-      T ri = r[o + i] - T(alpha) * Ap[o + i];
-      x[o + i] = xi;
-      r[o + i] = ri;
-      rr += double(ri) * double(ri);
-      if (zmode == 1) {
-        T zi = dinv[i] * ri;
-        z[o + i] = zi;
-        rz += double(ri) * double(zi);
-      } else if (zmode == 0) {
-        rz += double(ri) * double(ri);
-      }
-    }
+  };
+  const int64_t nw = n / W;
+  for (int64_t i = t0; i < nw; i += st) {
+    V xv = reinterpret_cast<V*>(x)[i], rv = reinterpret_cast<V*>(r)[i], zv, dv{};
+    const V pv = reinterpret_cast<const V*>(p)[i], av = reinterpret_cast<const V*>(Ap)[i];
+    if (ZMODE == 1) dv = reinterpret_cast<const V*>(dinv)[i];
+#pragma unroll
+    for (int c = 0; c < W; ++c) elem(xv.c[c], rv.c[c], pv.c[c], av.c[c], dv.c[c], zv.c[c], c);
+    reinterpret_cast<V*>(x)[i] = xv;
+    reinterpret_cast<V*>(r)[i] = rv;
+    if (ZMODE == 1) reinterpret_cast<V*>(z)[i] = zv;
   }
-  rr = block_sum(rr);
-  rz = block_sum(rz);
-  if (threadIdx.x == 0) {
-    part[int64_t(rh) * 2 * gridDim.x + blockIdx.x] = rr;
-    part[int64_t(rh) * 2 * gridDim.x + gridDim.x + blockIdx.x] = rz;
+  for (int64_t k = nw * W + t0; k < n; k += st) {
+    T zi{};
+    elem(x[k], r[k], p[k], Ap[k], ZMODE == 1 ? dinv[k] : T(0), zi, 0);
+    if (ZMODE == 1) z[k] = zi;
   }
+#pragma unroll
+  for (int c = 1; c < W; ++c) {
+    a[0].merge(a[c]);
+    if (ZMODE == 1) b[0].merge(b[c]);
+  }
+  double* const pr = part + int64_t(rh) * 2 * gridDim.x + blockIdx.x;
+  const int64_t g = gridDim.x;
+  DotAcc<T> v[ZMODE == 1 ? 2 : 1];
+  v[0] = a[0];
+  if (ZMODE == 1) v[ZMODE == 1 ? 1 : 0] = b[0];
+  block_sums<ZMODE == 1 ? 2 : 1>(v, [&](int k, double t) {
+    pr[k * g] = t;
+    if (ZMODE == 0) pr[g] = t;
+  });
   finish_if_last(part, fin);
 }
 
 // y = S p for a 125-point stencil on an (nx + 1) x (ny + 1) x (nz + 1) grid (the scaled fp16
 // tiled layout of stencil_at; entries toward nodes outside the grid are 0, and their loads are
-// clamped into it).  All sixteen 16-byte words of a row are loaded before the first is used.  DOT: also p.y, reduced like cg_alpha (Finish mode 1), so one launch
-// is a CG step's operator application and its alpha.  Fixed grid of at most kRedBlocks blocks.
-template <bool DOT>
+// clamped into it).  All sixteen 16-byte words of a row are loaded before the first is used.
 __global__ void __launch_bounds__(kRedThreads) k_stencil125(const __half* __restrict__ S,
                                                             const float* __restrict__ scale,
                                                             const float* __restrict__ p, float* __restrict__ y,
-                                                            int nx, int ny, int nz, double* part, Finish fin) {
-  if (DOT && fin.S[S_ACTIVE] == 0.0) return;  // the CG this step belongs to has stopped
+                                                            int nx, int ny, int nz) {
   const int px = nx + 1, pxy = px * (ny + 1), np = pxy * (nz + 1);
-  Dot2f acc;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < np; i += gridDim.x * blockDim.x) {
     const int ix = i % px, iy = (i / px) % (ny + 1), iz = i / pxy;
     int ox[5], oy[5], oz[5];
@@ -182,14 +208,7 @@ __global__ void __launch_bounds__(kRedThreads) k_stencil125(const __half* __rest
         }
       }
     }
-    const float s = scale[i] * (((sz[0] + sz[1]) + (sz[2] + sz[3])) + sz[4]);
-    y[i] = s;
-    if (DOT) acc.add(p[i], s);
-  }
-  if constexpr (DOT) {
-    const double t = block_sum(acc.value());
-    if (threadIdx.x == 0) part[blockIdx.x] = t;
-    finish_if_last(part, fin);
+    y[i] = scale[i] * (((sz[0] + sz[1]) + (sz[2] + sz[3])) + sz[4]);
   }
 }
 
@@ -202,20 +221,34 @@ __global__ void k_stencil_diag_inverse(const __half* __restrict__ S, const float
   if (d > 0.0f) pinv[i] = 1.0f / d;
 }
 
-template <typename T>
+template <typename T, int W>
 __global__ void k_cg_p(int64_t n, int64_t ld, const T* z, T* p, const double* S, bool skip_inactive) {
+  using V = Word<T, W>;
   const int rh = blockIdx.y;
   if (skip_inactive && S[rh * S_NSCAL + S_ACTIVE] == 0.0) return;
   const T beta = T(S[rh * S_NSCAL + S_BETA]);
-  const int64_t o = rh * ld;
-  for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x)
-    p[o + i] = z[o + i] + beta * p[o + i];
+  z += rh * ld;
+  p += rh * ld;
+  const int64_t st = int64_t(gridDim.x) * blockDim.x, t0 = int64_t(blockIdx.x) * blockDim.x + threadIdx.x, nw = n / W;
+  for (int64_t i = t0; i < nw; i += st) {
+    const V zv = reinterpret_cast<const V*>(z)[i];
+    V pv = reinterpret_cast<V*>(p)[i];
+#pragma unroll
+    for (int c = 0; c < W; ++c) pv.c[c] = zv.c[c] + beta * pv.c[c];
+    reinterpret_cast<V*>(p)[i] = pv;
+  }
+  for (int64_t i = nw * W + t0; i < n; i += st) p[i] = z[i] + beta * p[i];
 }
 
 template <typename TX, typename TY>
 __global__ void k_axpby(int64_t n, double a, const TX* x, double b, TY* y) {
   for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x)
     y[i] = TY(a * double(x[i]) + (b == 0.0 ? 0.0 : b * double(y[i])));
+}
+// y += a x in fp32 with one rounding per element
+__global__ void k_axpy32(int64_t n, float a, const float* x, float* y) {
+  for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x)
+    y[i] = fmaf(a, x[i], y[i]);
 }
 
 template <typename T> __global__ void k_pmul(int64_t n, const T* d, const T* r, T* z) {
@@ -337,18 +370,6 @@ __global__ void k_cheb_step(int64_t n, int64_t ld, T* z, const T* res_in, T* res
 // 16-byte boundaries and ld * sizeof(T) is a multiple of 16 (the solvers pad their bases so),
 // every thread moves 16-byte words (four floats or two doubles), so each step of a thread has
 // KG + 1 independent 16-byte loads in flight; otherwise the same code runs on single elements.
-template <typename T, int W> struct alignas(sizeof(T) * W) Word {
-  T c[W];
-};
-
-template <typename T> struct DotAcc;
-template <> struct DotAcc<float> : Dot2f {};
-template <> struct DotAcc<double> {
-  double s = 0.0;
-  __device__ __forceinline__ void add(double a, double b) { s = fma(a, b, s); }
-  __device__ __forceinline__ double value() const { return s; }
-};
-
 // part[(j0 + g) * gridDim.x + block] = the block's share of V_g . w for g < KG (V already offset
 // to vector j0): one sweep over w for KG vectors.
 template <typename T, int KG, int W>
@@ -375,11 +396,7 @@ __device__ __forceinline__ void multidot_group(const T* V, int64_t ld, const T* 
 #pragma unroll
       for (int g = 0; g < KG; ++g) acc[g].add(V[g * ld + i], y);
     }
-#pragma unroll
-  for (int g = 0; g < KG; ++g) {
-    const double sg = block_sum(acc[g].value());
-    if (threadIdx.x == 0) part[int64_t(j0 + g) * gridDim.x + blockIdx.x] = sg;
-  }
+  block_sums<KG>(acc, [&](int g, double t) { part[int64_t(j0 + g) * gridDim.x + blockIdx.x] = t; });
 }
 
 // h_j partials of V_j . w for j < k: groups of eight vectors, then one group of the rest
@@ -440,11 +457,7 @@ __global__ void __launch_bounds__(kRedThreads, 4) k_axpy_multidot(const T* V, in
 #pragma unroll
       for (int g = 0; g < KG; ++g) acc[g].add(V[g * ld + i], y);
     }
-#pragma unroll
-  for (int g = 0; g < KG; ++g) {
-    const double sg = block_sum(acc[g].value());
-    if (threadIdx.x == 0) part[int64_t(g) * gridDim.x + blockIdx.x] = sg;
-  }
+  block_sums<KG>(acc, [&](int g, double t) { part[int64_t(g) * gridDim.x + blockIdx.x] = t; });
 }
 
 __global__ void __launch_bounds__(kRedThreads) k_multidot_finish(const double* part, int g, double* h) {
@@ -469,7 +482,7 @@ __global__ void __launch_bounds__(256) k_multiaxpy(const T* V, int64_t ld, int k
   const int64_t nw = n / W, ldw = ld / W;
   const Wd* Vw = reinterpret_cast<const Wd*>(V);
   Wd* ww = reinterpret_cast<Wd*>(w);
-  DotAcc<T> nrm;
+  DotAcc<T> nrm[1];
   for (int64_t i = t0; i < nw; i += st) {
     Wd acc = ww[i];
     int j = 0;
@@ -490,18 +503,17 @@ __global__ void __launch_bounds__(256) k_multiaxpy(const T* V, int64_t ld, int k
     ww[i] = acc;
     if (NORM)
 #pragma unroll
-      for (int c = 0; c < W; ++c) nrm.add(acc.c[c], acc.c[c]);
+      for (int c = 0; c < W; ++c) nrm[0].add(acc.c[c], acc.c[c]);
   }
   if (W > 1)
     for (int64_t i = nw * W + t0; i < n; i += st) {
       T acc = w[i];
       for (int j = 0; j < k; ++j) acc = fma(hs[j], V[j * ld + i], acc);
       w[i] = acc;
-      if (NORM) nrm.add(acc, acc);
+      if (NORM) nrm[0].add(acc, acc);
     }
   if constexpr (NORM) {
-    const double s = block_sum(nrm.value());
-    if (threadIdx.x == 0) part[blockIdx.x] = s;
+    block_sums<1>(nrm, [&](int, double t) { part[blockIdx.x] = t; });
     finish_if_last(part, fin);
   }
 }
@@ -547,11 +559,35 @@ mf_status scratch(mf_ctx* ctx, size_t doubles, double** p) {
 #define LAUNCH_CHECK() \
   do { ctx->launches++; MF_CUDA_TRY(cudaGetLastError()); } while (0)
 
+// Blocks of a reduction over n elements: one element per thread up to four resident blocks per SM.  It
+// depends on n alone, so results are reproducible; a small vector pays for few block sums and partials.
+inline int red_blocks(int64_t n) {
+  return int(std::max<int64_t>(1, std::min<int64_t>(kRedBlocks, (n + kRedThreads - 1) / kRedThreads)));
+}
+// p starts on a 16-byte boundary and so does every vector ld elements further on
+template <typename T> bool words16(const T* p, int64_t ld) {
+  return reinterpret_cast<uintptr_t>(p) % 16 == 0 && (ld * int64_t(sizeof(T))) % 16 == 0;
+}
+
+// partial sums of x.y (and x2.y2 with x2 non-NULL) of nvec vectors ld apart
+template <typename T>
+static void launch_dot2(cudaStream_t s, const T* x, const T* y, const T* x2, const T* y2, int64_t n, int64_t ld, int nvec,
+                        double* part, const Finish& fin) {
+  constexpr int W = 16 / sizeof(T);
+  const int64_t l = nvec > 1 ? ld : 0;
+  const bool words = words16(x, l) && words16(y, l) && (!x2 || (words16(x2, l) && words16(y2, l)));
+  const dim3 g(red_blocks(n), nvec);
+  if (x2 && words) k_dot2_partial<T, W, true><<<g, kRedThreads, 0, s>>>(x, y, x2, y2, n, ld, part, fin);
+  else if (x2) k_dot2_partial<T, 1, true><<<g, kRedThreads, 0, s>>>(x, y, x2, y2, n, ld, part, fin);
+  else if (words) k_dot2_partial<T, W, false><<<g, kRedThreads, 0, s>>>(x, y, x2, y2, n, ld, part, fin);
+  else k_dot2_partial<T, 1, false><<<g, kRedThreads, 0, s>>>(x, y, x2, y2, n, ld, part, fin);
+}
+
 template <typename TX, typename TY> mf_status dot(mf_ctx* ctx, const TX* x, const TY* y, int64_t n, double* out) {
+  static_assert(std::is_same<TX, TY>::value, "one element type");
   double* part;
   MF_TRY(scratch(ctx, 2 * kRedBlocks, &part));
-  k_dot2_partial<TX, TY><<<dim3(kRedBlocks, 1), kRedThreads, 0, ctx->stream>>>(x, y, nullptr, nullptr, n, 0, part,
-                                                                                Finish{out, 0, nullptr, counters(ctx)});
+  launch_dot2<TX>(ctx->stream, x, y, nullptr, nullptr, n, 0, 1, part, Finish{out, 0, nullptr, counters(ctx)});
   LAUNCH_CHECK();
   return MF_OK;
 }
@@ -562,8 +598,7 @@ template <typename T>
 mf_status dot_batched(mf_ctx* ctx, const T* x, const T* y, int64_t n, int64_t ld, int nvec, double* out) {
   double* part;
   MF_TRY(scratch(ctx, 2 * kRedBlocks * size_t(nvec), &part));
-  k_dot2_partial<T, T><<<dim3(kRedBlocks, nvec), kRedThreads, 0, ctx->stream>>>(x, y, nullptr, nullptr, n, ld, part,
-                                                                                 Finish{out, 0, nullptr, counters(ctx)});
+  launch_dot2<T>(ctx->stream, x, y, nullptr, nullptr, n, ld, nvec, part, Finish{out, 0, nullptr, counters(ctx)});
   LAUNCH_CHECK();
   return MF_OK;
 }
@@ -573,6 +608,13 @@ template mf_status dot_batched<float>(mf_ctx*, const float*, const float*, int64
 mf_status norm2_sq(mf_ctx* ctx, const double* x, int64_t n, double* out) { return dot<double, double>(ctx, x, x, n, out); }
 
 template <typename TX, typename TY> mf_status axpby(mf_ctx* ctx, int64_t n, double a, const TX* x, double b, TY* y) {
+  if constexpr (std::is_same<TX, float>::value && std::is_same<TY, float>::value) {
+    if (b == 1.0 && double(float(a)) == a) {   // the fp64 form converts three times per element at the fp64 rate
+      k_axpy32<<<grid_for(n), 256, 0, ctx->stream>>>(n, float(a), x, y);
+      LAUNCH_CHECK();
+      return MF_OK;
+    }
+  }
   k_axpby<TX, TY><<<grid_for(n), 256, 0, ctx->stream>>>(n, a, x, b, y);
   LAUNCH_CHECK();
   return MF_OK;
@@ -621,8 +663,7 @@ template mf_status convert<float, double>(mf_ctx*, int64_t, const float*, double
 template <typename T> mf_status cg_alpha(mf_ctx* ctx, const T* p, const T* Ap, int64_t n, int64_t ld, int nrhs, double* S) {
   double* part;
   MF_TRY(scratch(ctx, 2 * kRedBlocks * size_t(nrhs), &part));
-  k_dot2_partial<T, T><<<dim3(kRedBlocks, nrhs), kRedThreads, 0, ctx->stream>>>(p, Ap, nullptr, nullptr, n, ld, part,
-                                                                                 Finish{nullptr, 1, S, counters(ctx)});
+  launch_dot2<T>(ctx->stream, p, Ap, nullptr, nullptr, n, ld, nrhs, part, Finish{nullptr, 1, S, counters(ctx)});
   LAUNCH_CHECK();
   return MF_OK;
 }
@@ -634,9 +675,17 @@ mf_status cg_update_xr(mf_ctx* ctx, int64_t n, int64_t ld, int nrhs, T* x, T* r,
                        const T* dinv, T* z, int zmode, double* S, bool skip_inactive) {
   double* part;
   MF_TRY(scratch(ctx, 2 * kRedBlocks * size_t(nrhs), &part));
-  k_cg_xr<T><<<dim3(kRedBlocks, nrhs), kRedThreads, 0, ctx->stream>>>(
-      n, ld, x, r, p, Ap, dinv, z, zmode, S, part, Finish{nullptr, zmode == 2 ? 5 : 2, S, counters(ctx)},
-      skip_inactive);
+  constexpr int W = 16 / sizeof(T);
+  const int64_t l = nrhs > 1 ? ld : 0;
+  const bool words = words16(x, l) && words16(r, l) && words16(p, l) && words16(Ap, l) &&
+                     (zmode != 1 || (words16(dinv, 0) && words16(z, l)));
+  const dim3 g(red_blocks(n), nrhs);
+  const Finish fin{nullptr, zmode == 2 ? 5 : 2, S, counters(ctx)};
+  auto start = [&](auto kernel) {
+    kernel<<<g, kRedThreads, 0, ctx->stream>>>(n, ld, x, r, p, Ap, dinv, z, S, part, fin, skip_inactive);
+  };
+  if (words) zmode == 1 ? start(k_cg_xr<T, W, 1>) : (zmode == 0 ? start(k_cg_xr<T, W, 0>) : start(k_cg_xr<T, W, 2>));
+  else zmode == 1 ? start(k_cg_xr<T, 1, 1>) : (zmode == 0 ? start(k_cg_xr<T, 1, 0>) : start(k_cg_xr<T, 1, 2>));
   LAUNCH_CHECK();
   return MF_OK;
 }
@@ -648,8 +697,7 @@ template mf_status cg_update_xr<float>(mf_ctx*, int64_t, int64_t, int, float*, f
 template <typename T> mf_status cg_rz(mf_ctx* ctx, const T* r, const T* z, int64_t n, int64_t ld, int nrhs, double* S) {
   double* part;
   MF_TRY(scratch(ctx, 2 * kRedBlocks * size_t(nrhs), &part));
-  k_dot2_partial<T, T><<<dim3(kRedBlocks, nrhs), kRedThreads, 0, ctx->stream>>>(r, z, nullptr, nullptr, n, ld, part,
-                                                                                 Finish{nullptr, 3, S, counters(ctx)});
+  launch_dot2<T>(ctx->stream, r, z, nullptr, nullptr, n, ld, nrhs, part, Finish{nullptr, 3, S, counters(ctx)});
   LAUNCH_CHECK();
   return MF_OK;
 }
@@ -660,8 +708,7 @@ template <typename T>
 mf_status cg_init_scalars(mf_ctx* ctx, const T* r, const T* z, int64_t n, int64_t ld, int nrhs, double* S) {
   double* part;
   MF_TRY(scratch(ctx, 2 * kRedBlocks * size_t(nrhs), &part));
-  k_dot2_partial<T, T><<<dim3(kRedBlocks, nrhs), kRedThreads, 0, ctx->stream>>>(r, r, r, z, n, ld, part,
-                                                                                 Finish{nullptr, 4, S, counters(ctx)});
+  launch_dot2<T>(ctx->stream, r, r, r, z, n, ld, nrhs, part, Finish{nullptr, 4, S, counters(ctx)});
   LAUNCH_CHECK();
   return MF_OK;
 }
@@ -669,19 +716,12 @@ template mf_status cg_init_scalars<double>(mf_ctx*, const double*, const double*
 template mf_status cg_init_scalars<float>(mf_ctx*, const float*, const float*, int64_t, int64_t, int, double*);
 
 mf_status stencil125_apply(mf_ctx* ctx, const void* Sv, const float* scale, const float* p, float* y, int nx, int ny,
-                           int nz, double* Scg) {
+                           int nz) {
   const __half* S = static_cast<const __half*>(Sv);
   const int64_t np = int64_t(nx + 1) * (ny + 1) * (nz + 1);
   if (np >= (int64_t(1) << 30)) return fail(MF_EUNSUPPORTED, "stencil grid too large for 32-bit indices");
   const int g = int(std::min<int64_t>((np + kRedThreads - 1) / kRedThreads, kRedBlocks));
-  if (Scg) {
-    double* part;
-    MF_TRY(scratch(ctx, 2 * kRedBlocks, &part));
-    k_stencil125<true><<<g, kRedThreads, 0, ctx->stream>>>(S, scale, p, y, nx, ny, nz, part,
-                                                         Finish{nullptr, 1, Scg, counters(ctx)});
-  } else {
-    k_stencil125<false><<<g, kRedThreads, 0, ctx->stream>>>(S, scale, p, y, nx, ny, nz, nullptr, Finish{});
-  }
+  k_stencil125<<<g, kRedThreads, 0, ctx->stream>>>(S, scale, p, y, nx, ny, nz);
   LAUNCH_CHECK();
   return MF_OK;
 }
@@ -695,7 +735,12 @@ mf_status stencil_diag_inverse(mf_ctx* ctx, const void* S, const float* scale, i
 
 template <typename T>
 mf_status cg_update_p(mf_ctx* ctx, int64_t n, int64_t ld, int nrhs, const T* z, T* p, double* S, bool skip_inactive) {
-  k_cg_p<T><<<dim3(grid_for(n), nrhs), 256, 0, ctx->stream>>>(n, ld, z, p, S, skip_inactive);
+  const int64_t l = nrhs > 1 ? ld : 0;
+  constexpr int W = 16 / sizeof(T);
+  if (words16(z, l) && words16(p, l))
+    k_cg_p<T, W><<<dim3(grid_for((n + W - 1) / W), nrhs), 256, 0, ctx->stream>>>(n, ld, z, p, S, skip_inactive);
+  else
+    k_cg_p<T, 1><<<dim3(grid_for(n), nrhs), 256, 0, ctx->stream>>>(n, ld, z, p, S, skip_inactive);
   LAUNCH_CHECK();
   return MF_OK;
 }
@@ -743,14 +788,9 @@ template mf_status cheb_step<double>(mf_ctx*, int64_t, int64_t, int, double*, co
 template mf_status cheb_step<float>(mf_ctx*, int64_t, int64_t, int, float*, const float*, float*, const float*, float*,
                                     const float*, double, double, bool, bool);
 
-// p starts on a 16-byte boundary and so does every vector ld elements further on
-template <typename T> bool words16(const T* p, int64_t ld) {
-  return reinterpret_cast<uintptr_t>(p) % 16 == 0 && (ld * int64_t(sizeof(T))) % 16 == 0;
-}
-
 template <typename T> mf_status multidot(mf_ctx* ctx, const T* V, int64_t ld, int k, const T* w, int64_t n, double* h) {
   if (k > 64) return fail(MF_EINVAL, "multidot: at most 64 vectors");
-  const int g = kRedBlocks;
+  const int g = red_blocks(n);
   double* part;
   MF_TRY(scratch(ctx, size_t(g) * (k + 1) + 64, &part));
   if (words16(V, ld) && words16(w, 0))
@@ -772,7 +812,7 @@ template <typename T> constexpr int kAxpyDotMax = sizeof(T) == 4 ? 6 : 2;
 template <typename T, int W>
 static void launch_axpy_multidot(mf_ctx* ctx, const T* V, int64_t ld, int k, const double* h, double sign, T* w,
                                  int64_t n, double* part) {
-  const int g = kRedBlocks;
+  const int g = red_blocks(n);
   switch (k) {
     case 1: k_axpy_multidot<T, 1, W><<<g, kRedThreads, 0, ctx->stream>>>(V, ld, h, sign, w, n, part); break;
     case 2: k_axpy_multidot<T, 2, W><<<g, kRedThreads, 0, ctx->stream>>>(V, ld, h, sign, w, n, part); break;
@@ -803,7 +843,7 @@ mf_status axpy_multidot(mf_ctx* ctx, const T* V, int64_t ld, int k, const double
     return multidot<T>(ctx, V, ld, k, w, n, h2);
   }
   if (k < 1) return MF_OK;
-  const int g = kRedBlocks;
+  const int g = red_blocks(n);
   double* part;
   MF_TRY(scratch(ctx, size_t(g) * (k + 1) + 64, &part));
   if (words16(V, ld) && words16(w, 0))
@@ -914,10 +954,9 @@ template <typename T>
 static mf_status dot_noalloc(const T* x, const T* y, int64_t n, int64_t ld, int nvec, double* out, cudaStream_t s) {
   double* part = nullptr;
   MF_TRY(noalloc_workspace(&part));
-  k_dot2_partial<T, T><<<dim3(kRedBlocks, nvec), kRedThreads, 0, s>>>(x, y, nullptr, nullptr, n, ld, part,
-                                                                       Finish{nullptr, 0, nullptr, nullptr});
+  launch_dot2<T>(s, x, y, nullptr, nullptr, n, ld, nvec, part, Finish{nullptr, 0, nullptr, nullptr});
   MF_CUDA_TRY(cudaGetLastError());
-  k_finish<<<nvec, kRedThreads, 0, s>>>(part, kRedBlocks, out, 0, nullptr);
+  k_finish<<<nvec, kRedThreads, 0, s>>>(part, red_blocks(n), out, 0, nullptr);
   MF_CUDA_TRY(cudaGetLastError());
   return MF_OK;
 }

@@ -60,10 +60,9 @@ __host__ __device__ inline int64_t stencil_at(int o, int64_t i) {
 }
 inline int64_t stencil_halves(int64_t n) { return (n + 31) / 32 * (128 * 32); }
 // y = S p for a 125-point stencil on the (nx + 1) x (ny + 1) x (nz + 1) grid (S: the fp16 entries,
-// scale: the row factors); with Scg non-NULL also Scg[pAp] = p.y and Scg[alpha] as cg_alpha sets
-// them, in the same launch, and nothing at all once Scg's active flag is 0
+// scale: the row factors)
 mf_status stencil125_apply(mf_ctx* ctx, const void* S, const float* scale, const float* p, float* y, int nx, int ny,
-                           int nz, double* Scg);
+                           int nz);
 // pinv[i] = 1 / (the stencil's diagonal entry of row i) where that is positive, else unchanged
 mf_status stencil_diag_inverse(mf_ctx* ctx, const void* S, const float* scale, int64_t n, float* pinv);
 // p = z + beta p (z = r when z is NULL); skip_inactive as for cg_update_xr
