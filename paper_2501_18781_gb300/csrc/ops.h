@@ -69,11 +69,11 @@ mf_status launch_oseen_coupling_f32(mf_ctx* ctx, const mf_dofmap* mu, int which,
 // scaled tiled layout of stencil_at, scale: n_p row factors; both overwritten)
 mf_status launch_schur_assemble_f32(mf_ctx* ctx, const mf_dofmap* mu, const float* blk, void* S, float* scale);
 // x = S~^-1 b by Jacobi-CG from 0 in one cooperative launch, zout = -x (fp64): at most maxit steps, to
-// |r|^2 <= tol2 |b|^2; work 4 n_p floats, w n_p floats, *steps += the steps taken.  A grid barrier that
-// waits for a second gives up and sets a flag: schur_cg_take_error, after the stream has synchronised.
+// |r|^2 <= tol2 |b|^2; work 4 n_p floats, *steps += the steps taken.  A grid barrier that
+// waits for a second gives up and sets a flag: grid_barrier_take_error, after the stream has synchronised.
 mf_status launch_schur_cg(mf_ctx* ctx, const void* S, const float* scale, const float* dinv, const double* b, float* x,
-                          float* work, float* w, double* zout, int nx, int ny, int nz, int maxit, double tol2, double* steps);
-mf_status schur_cg_take_error(mf_ctx* ctx);
+                          float* work, double* zout, int nx, int ny, int nz, int maxit, double tol2, double* steps);
+mf_status grid_barrier_take_error(mf_ctx* ctx);
 // Gauss-point tables from nodal fp64 fields (always evaluated in fp64, stored in both precisions)
 // (heat: rhocp_q / beta_q are the optional per-Gauss-point fields; qmass gets rhocp_q / dt)
 mf_status launch_scalar_qtables(mf_ctx* ctx, const mf_dofmap* m, int kind, const double* field, const double* kq_user,

@@ -4,11 +4,12 @@
 // Run as separate kernels, a step was four launches on vectors that fit in L2 (40^3 cells: 69 k rows, 33 us
 // per step in the launch list of a melt-pool step), and the steps after convergence still launched.  Here
 // one cooperative grid holds the whole iteration, one block of 1024 threads per SM, with two grid barriers
-// per step: the inner products of a step are gathered together (the single-reduction form of CG of
-// Chronopoulos and Gear, J. Comput. Appl. Math. 25, 1989: s = A p is updated with A z instead of
-// recomputed), and every block adds the per-block partial sums in the same order, so all blocks hold the
-// same scalars and the result does not depend on timing.  A barrier gives up after one second of
-// %globaltimer and sets a flag.
+// per step: the stencil is applied to z, which the barrier after the vector update has just made visible, and
+// s = S~ p follows from s = S~ z + beta s, so the direction needs no barrier of its own.  p . s is summed as
+// it stands: formed from z . S~ z as in the single-reduction CG it loses digits, which moved the
+// outer iteration's count.  Every block adds the per-block partial sums in the same order, so all blocks
+// hold the same scalars and the result does not depend on timing.  A barrier gives up after one second
+// of %globaltimer and sets a flag.
 // Bound: latency of the barriers and of the two dependent passes, 12 us per step at 40^3 (351 us per
 // call); the 40^3 step's Schur solves went from 30 to 10 ms.  The fp64 scalars are one thread's work:
 // divisions in all 32 warps took 8 us per step, the fp64 sums over all of them 5 us.
@@ -16,79 +17,22 @@
 
 #include <cstring>
 
+#include "grid_barrier.cuh"
 #include "ops.h"
-#include "reduce.cuh"
 
 namespace mf {
 namespace {
 
 constexpr int kThreads = 1024;
-constexpr size_t kCoefBytes = size_t(200) << 10;   // coefficients a block may keep in shared memory
-
-// Barrier over the whole (co-resident) grid; bar = {arrived, generation, timed out}.  The release of the
-// arrival and the acquire of the new generation order the blocks' global memory accesses.
-__device__ __forceinline__ unsigned load_acquire(const unsigned* p) {
-  unsigned v;
-  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-  return v;
-}
-__device__ __forceinline__ bool grid_barrier(unsigned* bar, unsigned nblocks) {
-  __shared__ bool ok;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    ok = true;
-    const unsigned gen = load_acquire(bar + 1);
-    unsigned before;
-    asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], 1;" : "=r"(before) : "l"(bar) : "memory");
-    if (before == nblocks - 1) {
-      bar[0] = 0u;
-      asm volatile("red.add.release.gpu.global.u32 [%0], 1;" ::"l"(bar + 1) : "memory");
-    } else {
-      unsigned long long t0 = 0;
-      for (unsigned spins = 0; load_acquire(bar + 1) == gen; ++spins) {
-        if ((spins & 1023u) != 1023u) continue;
-        unsigned long long t;
-        asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-        if (!t0) t0 = t;
-        if (t - t0 > 1000000000ull || load_acquire(bar + 2)) {
-          atomicExch(bar + 2, 1u);
-          ok = false;
-          break;
-        }
-      }
-    }
-  }
-  __syncthreads();
-  return ok;
-}
-
-// Block sums of N values, value k to part[k * stride + blockIdx.x].  Pairs of floats down to one value per
-// warp: fp64 adds cost 16 cycles of the SM per warp instruction (a tree of them over the block's 32 warps
-// took longer than the step's stencil).
-template <int N> __device__ __forceinline__ void block_partials(Dot2f (&v)[N], double (*sh)[32], double* part, int64_t stride) {
-#pragma unroll
-  for (int k = 0; k < N; ++k) v[k].warp_sum();
-  if ((threadIdx.x & 31) == 0)
-#pragma unroll
-    for (int k = 0; k < N; ++k) sh[k][threadIdx.x >> 5] = v[k].value();
-  __syncthreads();
-  if (threadIdx.x < 32 * N) {
-    const int k = threadIdx.x >> 5;
-    double s = sh[k][threadIdx.x & 31];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-    if ((threadIdx.x & 31) == 0) part[k * stride + blockIdx.x] = s;
-  }
-}
 
 struct SchurArgs {
   const __half* S;      // scaled fp16 tiled layout of stencil_at
   const float* scale;
   const float* dinv;
   const double* b;     // right-hand side
-  float *x, *r, *z, *p, *s, *w;
+  float *x, *r, *z, *p, *s;
   double* zout;        // -x in fp64
-  double* part;        // partial sums: [2][2][grid] (r.r, r.z by step parity), then [grid] (z.w)
+  double* part;        // partial sums: [2][grid] (r.r, r.z), then [grid] (p.s)
   double* steps;       // step counter over all solves
   unsigned* bar;
   double tol2;
@@ -132,16 +76,17 @@ __device__ __forceinline__ float stencil_words(const SchurArgs& A, const uint4* 
   return s0 + s1;
 }
 
-// PARTS threads share a row (warp by warp, so that every thread's entries are known at compile time).  CACHED:
-// the block's coefficients stay in shared memory for the whole solve.
-template <int PARTS, bool CACHED>
+// PARTS threads share a row (warp by warp, so that every thread's entries are known at compile time).  With two
+// or four a block has one run of rows (start()), whose coefficients stay in shared memory for the whole solve.
+template <int PARTS>
 __global__ void __launch_bounds__(kThreads, 1) k_schur_cg(const SchurArgs A) {
   extern __shared__ uint4 coef[];
-  __shared__ double sh[2][32], tot[3];
-  __shared__ float coefs[2];
+  __shared__ double sh[2][32], tot[2];
+  __shared__ float coef_s;   // beta, then alpha
   __shared__ bool done;
   __shared__ float ssum[PARTS > 1 ? PARTS : 1][kThreads / PARTS];
   constexpr int kRows = kThreads / PARTS, kWords = 16 / PARTS;   // rows of a block at a time, words of a thread
+  constexpr bool CACHED = PARTS > 1;
   const int np = (A.nx + 1) * (A.ny + 1) * (A.nz + 1);
   const int part = threadIdx.x / kRows, local = threadIdx.x % kRows;
   const unsigned G = gridDim.x;
@@ -151,53 +96,49 @@ __global__ void __launch_bounds__(kThreads, 1) k_schur_cg(const SchurArgs A) {
   const bool own = threadIdx.x < kRows;   // the thread that keeps the row's vectors
   auto words = [&](int i) { return reinterpret_cast<const uint4*>(A.S + stencil_at(0, i)); };
   if (CACHED) {
-    int run = 0;
-    for (int i0 = first; i0 < np; i0 += step, ++run) {
-      const uint4* const g = words(i0);   // kRows is a multiple of 32: the run's rows are consecutive tiles
-      const int n = (min(kRows, np - i0) + 31) / 32 * 512;
-      for (int q = threadIdx.x; q < n; q += kThreads) coef[run * (kRows * 16) + q] = __ldg(g + q);
-    }
+    const uint4* const g = words(first);   // kRows is a multiple of 32: the rows are consecutive tiles
+    const int n = (min(kRows, np - first) + 31) / 32 * 512;
+    for (int q = threadIdx.x; q < n; q += kThreads) coef[q] = __ldg(g + q);
     __syncthreads();
   }
-  // w = S~ z on the block's rows, and the thread's share of z . w
-  auto apply = [&](Dot2f& azw) {
-    int run = 0;
-    for (int i0 = first; i0 < np; i0 += step, ++run) {
+  // p = z + beta p, s = S~ z + beta s (so s = S~ p) on the block's rows, and the thread's share of p . s
+  auto apply = [&](int k, float be, Dot2f& aps) {
+    for (int i0 = first; i0 < np; i0 += step) {
       const int i = i0 + local;
-      float s = 0.f;
+      float w = 0.f;
       if (i < np) {
-        const uint4* const q = (CACHED ? coef + run * (kRows * 16) + (local >> 5) * 512 + (local & 31) : words(i)) +
-                               32 * kWords * part;
-        if (PARTS == 1) s = stencil_words<0, kWords>(A, q, A.z, i);
-        else if (part == 0) s = stencil_words<0, kWords>(A, q, A.z, i);
-        else if (part == 1) s = stencil_words<kWords % 16, kWords>(A, q, A.z, i);
-        else if (part == 2) s = stencil_words<2 * kWords % 16, kWords>(A, q, A.z, i);
-        else s = stencil_words<3 * kWords % 16, kWords>(A, q, A.z, i);
+        const uint4* const q = (CACHED ? coef + (local >> 5) * 512 + (local & 31) : words(i)) + 32 * kWords * part;
+        if (PARTS == 1) w = stencil_words<0, kWords>(A, q, A.z, i);
+        else if (part == 0) w = stencil_words<0, kWords>(A, q, A.z, i);
+        else if (part == 1) w = stencil_words<kWords % 16, kWords>(A, q, A.z, i);
+        else if (part == 2) w = stencil_words<2 * kWords % 16, kWords>(A, q, A.z, i);
+        else w = stencil_words<3 * kWords % 16, kWords>(A, q, A.z, i);
       }
       if (PARTS > 1) {
-        ssum[part][local] = s;
+        ssum[part][local] = w;
         __syncthreads();
         if (own) {
-          s = ssum[0][local];
+          w = ssum[0][local];
 #pragma unroll
-          for (int k = 1; k < PARTS; ++k) s += ssum[k][local];
+          for (int j = 1; j < PARTS; ++j) w += ssum[j][local];
         }
       }
       if (own && i < np) {
-        const float w = A.scale[i] * s;
-        A.w[i] = w;
-        azw.add(A.z[i], w);
+        w *= A.scale[i];
+        const float p = k ? A.z[i] + be * A.p[i] : A.z[i], t = k ? w + be * A.s[i] : w;
+        A.p[i] = p;
+        A.s[i] = t;
+        aps.add(p, t);
       }
       if (PARTS > 1) __syncthreads();
     }
   };
-  // fixed-order sums of the blocks' partials, the same in every block: warp k adds array k
-  auto totals = [&](int parity) {
+  // fixed-order sums of N arrays of the blocks' partials, the same in every block: warp k adds array k
+  auto totals = [&](const double* q, int n) {
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (w < 3) {
-      const double* q = w < 2 ? A.part + (2 * parity + w) * int64_t(G) : A.part + 4 * int64_t(G);
+    if (w < n) {
       double s = 0.0;
-      for (unsigned k = lane; k < G; k += 32) s += __ldcg(q + k);
+      for (unsigned k = lane; k < G; k += 32) s += __ldcg(q + w * int64_t(G) + k);
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
       if (lane == 0) tot[w] = s;
@@ -214,41 +155,39 @@ __global__ void __launch_bounds__(kThreads, 1) k_schur_cg(const SchurArgs A) {
       arr.add(r, r);
       arz.add(r, z);
     }
-  double rz_old = 1.0, alpha = 0.0, stop = 0.0;   // thread 0 of every block
+  double rz = 1.0, stop = 0.0;   // thread 0 of every block: fp64 divisions by one thread, not by 32 warps
   int k = 0;
   for (; k < A.maxit; ++k) {
     Dot2f v2[2] = {arr, arz};
-    block_partials<2>(v2, sh, A.part + 2 * (k & 1) * int64_t(G), G);
+    block_partials<2>(v2, sh, A.part, G);
     if (!grid_barrier(A.bar, G)) return;
-    Dot2f v1[1];
-    apply(v1[0]);
-    block_partials<1>(v1, sh, A.part + 4 * int64_t(G), G);
-    if (!grid_barrier(A.bar, G)) return;
-    totals(k & 1);
-    if (threadIdx.x == 0) {   // fp64 divisions by one thread, not by 32 warps
-      const double rr = tot[0], rz = tot[1], zw = tot[2];
-      if (k == 0) stop = A.tol2 * rr;
-      const double beta = k ? rz / rz_old : 0.0;
-      const double pap = k ? zw - beta * rz / alpha : zw;   // p.A p of p = z + beta p
-      // converged (or a zero right-hand side), or a breakdown: x stays as it is
-      done = rr <= stop || !(pap > 0.0);
-      alpha = rz / pap;
-      rz_old = rz;
-      coefs[0] = float(alpha);
-      coefs[1] = float(beta);
+    totals(A.part, 2);
+    if (threadIdx.x == 0) {
+      if (k == 0) stop = A.tol2 * tot[0];
+      done = tot[0] <= stop;   // converged, or a zero right-hand side
+      coef_s = float(k ? tot[1] / rz : 0.0);
+      rz = tot[1];
     }
     __syncthreads();
     if (done) break;
-    const float al = coefs[0], be = coefs[1];
+    Dot2f v1[1];
+    apply(k, coef_s, v1[0]);
+    block_partials<1>(v1, sh, A.part + 2 * int64_t(G), G);
+    if (!grid_barrier(A.bar, G)) return;
+    totals(A.part + 2 * int64_t(G), 1);
+    if (threadIdx.x == 0) {
+      done = !(tot[0] > 0.0);   // a breakdown: x stays as it is
+      coef_s = float(rz / tot[0]);
+    }
+    __syncthreads();
+    if (done) break;
+    const float al = coef_s;
     arr = Dot2f();
     arz = Dot2f();
     if (own)
       for (int i = t0; i < np; i += step) {
-        const float p = k ? A.z[i] + be * A.p[i] : A.z[i], s = k ? A.w[i] + be * A.s[i] : A.w[i];
-        const float r = A.r[i] - al * s, z = A.dinv[i] * r;
-        A.p[i] = p;
-        A.s[i] = s;
-        A.x[i] += al * p;
+        const float r = A.r[i] - al * A.s[i], z = A.dinv[i] * r;
+        A.x[i] += al * A.p[i];
         A.r[i] = r;
         A.z[i] = z;
         arr.add(r, r);
@@ -260,20 +199,19 @@ __global__ void __launch_bounds__(kThreads, 1) k_schur_cg(const SchurArgs A) {
   if (blockIdx.x == 0 && threadIdx.x == 0) *A.steps += double(k);
 }
 
+// PARTS > 1 only where the grid holds all rows at once
 template <int PARTS> cudaError_t start(mf_ctx* ctx, SchurArgs& a, int64_t np) {
   constexpr int rows = kThreads / PARTS;
   const int64_t want = (np + rows - 1) / rows;
   const unsigned grid = unsigned(want < ctx->sm_count ? want : ctx->sm_count);
-  const size_t runs = size_t((want + grid - 1) / grid), bytes = runs * rows * 256;
-  const bool cached = bytes <= kCoefBytes;
-  const void* const k = cached ? reinterpret_cast<const void*>(k_schur_cg<PARTS, true>)
-                               : reinterpret_cast<const void*>(k_schur_cg<PARTS, false>);
-  if (cached) {
-    const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kCoefBytes));
+  const size_t bytes = PARTS > 1 ? size_t(rows) * 256 : 0;   // 128 or 64 KB
+  const void* const k = reinterpret_cast<const void*>(k_schur_cg<PARTS>);
+  if (bytes) {
+    const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(bytes));
     if (e != cudaSuccess) return e;
   }
   void* args[] = {&a};
-  return cudaLaunchCooperativeKernel(k, dim3(grid), dim3(kThreads), args, cached ? bytes : 0, ctx->stream);
+  return cudaLaunchCooperativeKernel(k, dim3(grid), dim3(kThreads), args, bytes, ctx->stream);
 }
 
 }  // namespace
@@ -281,7 +219,7 @@ template <int PARTS> cudaError_t start(mf_ctx* ctx, SchurArgs& a, int64_t np) {
 // zout = -x and x = S~^-1 b by at most maxit steps from 0, to ||r|| <= sqrt(tol2) ||b||.  work: 4 n_p
 // floats (r, z, p, s).
 mf_status launch_schur_cg(mf_ctx* ctx, const void* S, const float* scale, const float* dinv, const double* b, float* x,
-                          float* work, float* w, double* zout, int nx, int ny, int nz, int maxit, double tol2, double* steps) {
+                          float* work, double* zout, int nx, int ny, int nz, int maxit, double tol2, double* steps) {
   const int64_t np = int64_t(nx + 1) * (ny + 1) * (nz + 1);
   SchurArgs a{};
   a.S = static_cast<const __half*>(S);
@@ -293,7 +231,6 @@ mf_status launch_schur_cg(mf_ctx* ctx, const void* S, const float* scale, const 
   a.z = work + np;
   a.p = work + 2 * np;
   a.s = work + 3 * np;
-  a.w = w;
   a.zout = zout;
   a.part = ctx->scratch.as<double>();
   a.steps = steps;
@@ -310,15 +247,15 @@ mf_status launch_schur_cg(mf_ctx* ctx, const void* S, const float* scale, const 
   return MF_OK;
 }
 
-// MF_ETIMEOUT (once, then the barrier is reset) if a launch's barrier gave up
-mf_status schur_cg_take_error(mf_ctx* ctx) {
+// MF_ETIMEOUT (once, then the barrier is reset) if the barrier of a cooperative launch gave up
+mf_status grid_barrier_take_error(mf_ctx* ctx) {
   unsigned bar[3] = {0u, 0u, 0u};
   unsigned* const d = ctx->counters.as<unsigned>() + kBarrierCounter;
   MF_CUDA_TRY(cudaMemcpyAsync(bar, d, sizeof bar, cudaMemcpyDeviceToHost, ctx->stream));
   MF_CUDA_TRY(cudaStreamSynchronize(ctx->stream));
   if (!bar[2]) return MF_OK;
   MF_CUDA_TRY(cudaMemsetAsync(d, 0, sizeof bar, ctx->stream));
-  return fail(MF_ETIMEOUT, "a grid barrier of the Schur complement solve timed out");
+  return fail(MF_ETIMEOUT, "a grid barrier of a solver kernel timed out");
 }
 
 }  // namespace mf

@@ -195,7 +195,7 @@ struct OseenBlockTri {
   int64_t n = 0, nu = 0, nu3 = 0, np = 0;
   int ku = 10, smax = 30;
   double stol = 0.1;
-  Vec<float> blk32, ua, pinv32, xp, sp, cgw, V, t, w;
+  Vec<float> blk32, ua, pinv32, xp, cgw, V, t, w;
   DevBuf stil;        // S~ = B D^-1 B^T as a 125-point stencil on the pressure grid (fp16 entries)
   Vec<float> stscale;  // and its row factors
   int gn[3] = {0, 0, 0};  // cells per axis
@@ -227,7 +227,7 @@ struct OseenBlockTri {
     // fp32 3x3 block inverses and inverse pressure scaling, computed in fp32 (the preconditioner
     // applies them in fp32)
     MF_TRY(blk32.alloc(9 * nu));
-    for (Vec<float>* v : {&pinv32, &xp, &sp}) MF_TRY(v->alloc(np));
+    for (Vec<float>* v : {&pinv32, &xp}) MF_TRY(v->alloc(np));
     MF_TRY(cgw.alloc(4 * np));
     MF_TRY(oseen_blocks32(op, blk32.p, pinv32.p));
     for (int d = 0; d < 3; ++d) gn[d] = op->map[0]->mesh->n[d];
@@ -254,7 +254,7 @@ struct OseenBlockTri {
   // xp = S~^-1 r_p (r_p fp64) and z_p = -xp: Jacobi-PCG from 0 in one launch, at most smax steps; once
   // ||r_k|| <= stol ||r_0|| (or p.S~p <= 0) x stays as it is.
   mf_status schur_solve(const double* r, double* z) {
-    return launch_schur_cg(op->ctx, stil.p, stscale.p, pinv32.p, r, xp.p, cgw.p, sp.p, z, gn[0], gn[1], gn[2], smax,
+    return launch_schur_cg(op->ctx, stil.p, stscale.p, pinv32.p, r, xp.p, cgw.p, z, gn[0], gn[1], gn[2], smax,
                            stol * stol, schur_steps());
   }
 
@@ -875,7 +875,7 @@ mf_status solve_impl(mf_op* op, const mf_solver_params* sp, const double* b, dou
     }
     if (P.tri) {
       MF_TRY(sync_copy(c, c->host_scalars + kScalarsTri + 144, P.tri->schur_steps(), 1));
-      MF_TRY(schur_cg_take_error(c));
+      MF_TRY(grid_barrier_take_error(c));
       inf.inner_steps = int(c->host_scalars[kScalarsTri + 144]);
     }
   } else if (sp->solver == MF_SOLVER_DEFECT_CORRECTION) {
