@@ -21,7 +21,7 @@ COMMON = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-Xcompiler",
 SOURCES = ["mesh.cpp", "cellops_host.cpp", "api.cpp", "solver.cpp",
            "apply.cu", "apply_f64.cu", "apply_f32.cu", "apply_df64.cu", "apply_df64_uniform.cu", "apply_df64_octree.cu",
            "apply_f32_uniform.cu", "apply_f32_octree_rhs.cu", "apply_f32_oseen.cu", "aux.cu", "vec.cu",
-           "solver_kernels.cu", "sources.cu", "apply_h16.cu", "step.cu", "step.cpp", "apply_qk.cu", "apply_qk_tc.cu", "schur_cg.cu"]
+           "solver_kernels.cu", "sources.cu", "apply_h16.cu", "step.cu", "step.cpp", "apply_qk.cu", "apply_qk_tc.cu", "schur_cg.cu", "q2_line.cu"]
 
 
 def _digest():

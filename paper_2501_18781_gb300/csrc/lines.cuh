@@ -66,4 +66,28 @@ __device__ __forceinline__ void line_combine_t(const T& f0, const T& f1, const T
   v2 = c + T(kLineDelta) * d;
 }
 
+// The transposes with the Gauss weights folded into them, for test sides kept without weights: the stencil
+// becomes W^-1 stencil^T W (weights (5, 8, 5) / 18), the value transpose S^T W times a factor given by the
+// caller's constants k = {0.3 w0, w1, 0.4 w0, delta w0} f.
+template <typename T> __device__ __forceinline__ void line_deriv_tw(const T& f0, const T& f1, const T& f2, T& r0, T& r1, T& r2) {
+  const T s = (f0 + f2) + T(1.6) * f1, e = f2 - f0;
+  r0 = (r0 - s) + T(2) * e;
+  r1 = r1 - T(2.5) * e;
+  r2 = (r2 + s) + T(2) * e;
+}
+template <typename T> __device__ __forceinline__ void line_values_tw(const T (&k)[4], T& f0, T& f1, T& f2) {
+  const T t = f0 + f2, d = k[3] * (f2 - f0), c = k[0] * t;
+  f1 = k[1] * f1 + k[2] * t;
+  f0 = c - d;
+  f2 = c + d;
+}
+template <typename T>
+__device__ __forceinline__ void line_combine_tw(const T (&k)[4], const T& f0, const T& f1, const T& f2, T& v0, T& v1, T& v2) {
+  const T s = (f0 + f2) + T(1.6) * f1, e = f2 - f0;
+  const T t = (v0 + v2) + T(4) * e, d = k[3] * ((v2 - v0) + T(2) * s), c = k[0] * t;
+  v1 = k[1] * (v1 - T(2.5) * e) + k[2] * t;
+  v0 = c - d;
+  v2 = c + d;
+}
+
 }  // namespace mf

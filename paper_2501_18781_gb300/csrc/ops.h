@@ -124,6 +124,12 @@ mf_status launch_helmholtz_qk(mf_ctx* ctx, const mf_dofmap* m, const T* src, T* 
 // accumulated (zero it first); Dirichlet rows receive nothing
 template <typename T>
 mf_status launch_q2_line(mf_ctx* ctx, const mf_dofmap* m, const T* src, T* dst, const T* coef, double mass);
+// Jacobi-CG on such an operator in one cooperative launch, from the r, z = dinv r, p = z and scalars S of
+// cg_init_scalars; p2 a second direction buffer; stops at r.r <= tol^2 r0.r0, after maxit steps and, with
+// stop_indefinite, at p.Ap <= 0: S[rr], S[active] (0: stopped by itself) and steps[0] are set
+mf_status launch_q2_line_cg(mf_ctx* ctx, const mf_dofmap* m, const double* coef, double mass, const double* dinv, double* x,
+                            double* r, double* z, double* p, double* p2, double* Ap, double tol, int maxit,
+                            bool stop_indefinite, double* S, double* steps);
 mf_status launch_qk_diag(mf_ctx* ctx, const mf_dofmap* m, const double* coef, double mass, double* diag);
 // Q3 Helmholtz on the tensor cores (fp32 vectors, dst accumulated; coef per tile of 128 cells,
 // [tile][q][row], from launch_tc_coef_layout).  A launch returns MF_ETIMEOUT when an earlier one

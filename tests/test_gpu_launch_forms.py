@@ -1,4 +1,5 @@
-"""Launch forms that only larger inputs reach: the row splits of the Schur complement solve."""
+"""Launch forms that only larger inputs reach: the Jacobi-CG that runs as one launch (one cell per group of
+nine threads, or several), and the row splits of the Schur complement solve."""
 import numpy as np
 import pytest
 
@@ -20,6 +21,44 @@ def ctx():
 
 def _cuda(a):
     return torch.tensor(np.ascontiguousarray(a), device="cuda")
+
+
+def _map(ctx, n, faces, degree=2, h=0.125):
+    from paper_2501_18781_gb300 import DofMap, Mesh
+    return DofMap(Mesh.uniform(ctx, list(n), (0.0, 0.0, 0.0), tuple(h * m for m in n)), degree, faces)
+
+
+# The one-launch CG takes single systems, two systems run step by step.  Both stop at ||r|| <= 1e-11 ||b||;
+# with value and stiffness terms of one size the Jacobi-scaled operator has a condition number below 1e3, so the
+# solutions agree to 2 x 1e-11 x 1e3.  The iteration counts differ by roundoff only: at most one step.
+@pytest.mark.parametrize("box", [(1, 1, 1), (9, 5, 3), (17, 14, 13), (19, 16, 15)])
+@pytest.mark.parametrize("use_graph", [False, True])
+@pytest.mark.parametrize("kind", ["helmholtz", "heat"])
+def test_one_launch_cg_matches_steps(ctx, box, use_graph, kind):
+    from paper_2501_18781_gb300 import Operator
+    m = _map(ctx, box, 0b011010 if kind == "heat" else 0)
+    rng = syn.uniform_pm1(3, m.n_dofs)
+    rho = 2.0 * 8 ** 3
+    if kind == "heat":
+        op = Operator(ctx, "heat", [m], rhocp=rho, dt=1.0, k0=8.0, t_boil=1.0, coef_mode=1)
+        op.set_field("t_prev", _cuda(1.0 + 0.5 * rng))
+    else:
+        op = Operator(ctx, "helmholtz", [m], mass_coef=rho, a_liquid=80.0, a_gas=8.0, coef_mode=1)
+        op.set_field("phi", _cuda(np.tanh(4.0 * (m.coords()[:, 2] - 0.3) + 0.2 * rng)))
+    op.set_variant("q2_line", 1)
+    b = _cuda(syn.uniform_pm1(7, m.n_dofs))
+    kw = dict(solver="cg", precond="jacobi", tol=1e-11, maxit=2000, use_graph=use_graph)
+    x1, one = op.solve(b, **kw)
+    x2, two = op.solve(torch.cat([b, b]), nrhs=2, **kw)
+    assert one["status"] == two["status"] == 0
+    assert abs(one["iterations"] - two["iterations"]) <= 1, (one, two)
+    assert float((x1 - x2[:m.n_dofs]).norm() / x1.norm()) <= 2e-8
+    # a cap below the count: both stop there and say so
+    cap = max(1, one["iterations"] // 2)
+    for rhs, nrhs in ((b, 1), (torch.cat([b, b]), 2)):
+        _, info = op.solve(rhs, nrhs=nrhs, **{**kw, "maxit": cap})
+        if cap < one["iterations"]:
+            assert info["status"] != 0 and info["iterations"] == cap, info
 
 
 # 33^3 cells: two threads per pressure row on 152 SMs, 42^3: one (the smaller meshes that are held to the oracle
