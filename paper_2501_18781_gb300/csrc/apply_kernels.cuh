@@ -120,14 +120,12 @@ __device__ __forceinline__ void scalar_cell(const ScalarArgs<typename Store<T>::
 
 // One launch sweeps all nwork work units; with fewer blocks than units (the persistent
 // variant, grid = a few blocks per SM) each block strides over them.  All right-hand sides of
-// a cell are applied while its coefficients sit in registers.  Two fp32 instances are held to five
-// blocks of 128 per SM (96 registers): the octree reinitialisation (no spills; its indirect gathers are
-// latency-bound, and 20 warps per SM instead of 16 measured 2.41 -> 2.32 ms for the 8-RHS base-32
-// octree apply) and the uniform heat operator without convection (48 bytes of spills; 128^3 apply
-// 0.168 -> 0.161 ms).  The other instances would spill more at that bound.
+// a cell are applied while its coefficients sit in registers.  Two fp32 instances are held to four
+// blocks of 128 per SM: the octree reinitialisation, whose indirect gathers are latency-bound, and the
+// uniform heat operator without convection (five blocks spill in the difference form).
 template <typename T, int KIND, int MODE, bool BETA, bool TR, bool OCT>
 __global__ void __launch_bounds__(128, (sizeof(T) == 4 && ((OCT && KIND == K_REINIT) ||
-                                                           (!OCT && KIND == K_HEAT && !BETA))) ? 5 : 1)
+                                                           (!OCT && KIND == K_HEAT && !BETA))) ? 4 : 1)
     k_scalar(ScalarArgs<typename Store<T>::type> A, UniformGeom ug, OctGeom og,
                                                 int64_t nwork) {
   for (int64_t w = blockIdx.x; w < nwork; w += gridDim.x) {
@@ -256,10 +254,20 @@ __global__ void __launch_bounds__(128, 1) k_oseen(OseenArgs<typename Store<T>::t
 template <typename T, bool EXT = false>
 __global__ void __launch_bounds__(128) k_oseen_qouter(OseenArgs<typename Store<T>::type> A, UniformGeom ug) {
   using St = typename Store<T>::type;
-  int i, j, k;
-  if (!brick_cell(ug, i, j, k)) return;
-  const int64_t cell = i + int64_t(ug.nx) * (j + int64_t(ug.ny) * k);
   const int64_t nc = int64_t(ug.nx) * ug.ny * ug.nz;
+  int i, j, k;
+  if constexpr (sizeof(T) == 8) {
+    // cells in lexicographic order: the fp64 pipe bounds this kernel, so no lane may idle where the box is
+    // not a multiple of the bricks (33 x 40 x 27: bricks leave 20 % of the lanes without a cell)
+    const int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+    if (t >= nc) return;
+    i = int(t % ug.nx);
+    j = int((t / ug.nx) % ug.ny);
+    k = int(t / (int64_t(ug.nx) * ug.ny));
+  } else if (!brick_cell(ug, i, j, k)) {
+    return;
+  }
+  const int64_t cell = i + int64_t(ug.nx) * (j + int64_t(ug.ny) * k);
   const int64_t base = 2 * int64_t(i) + ug.sx * (2 * int64_t(j)) + ug.sy * (2 * int64_t(k));
   const uint32_t dmask = dirichlet_mask(ug, i, j, k);
   const int64_t px = ug.nx + 1, pxy = px * (ug.ny + 1);
