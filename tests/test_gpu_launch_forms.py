@@ -1,5 +1,6 @@
-"""Launch forms that only larger inputs reach: the Jacobi-CG that runs as one launch (one cell per group of
-nine threads, or several), and the row splits of the Schur complement solve."""
+"""Launch forms that only larger inputs reach: marches of several layers in the fp32 kernel of uniform
+meshes, the Jacobi-CG that runs as one launch (one cell per group of nine threads, or several), and the
+row splits of the Schur complement solve."""
 import numpy as np
 import pytest
 
@@ -26,6 +27,31 @@ def _cuda(a):
 def _map(ctx, n, faces, degree=2, h=0.125):
     from paper_2501_18781_gb300 import DofMap, Mesh
     return DofMap(Mesh.uniform(ctx, list(n), (0.0, 0.0, 0.0), tuple(h * m for m in n)), degree, faces)
+
+
+# 45 columns of 13 layers: 2 layers per march with 17 right-hand sides on 152 SMs, 6 with 60, so the last
+# march of a column has one layer.  fp32 against the fp64 apply, held to the fp32 bar 2e-5 of the largest
+# entry (unit roundoff 6e-8, a few hundred operations per row).
+@pytest.mark.parametrize("nrhs", [17, 60])
+@pytest.mark.parametrize("faces", [0, 0b110101])
+def test_fp32_marches_of_several_layers(ctx, nrhs, faces):
+    from paper_2501_18781_gb300 import Operator
+    m = _map(ctx, (39, 35, 13), faces)
+    rng = syn.uniform_pm1(3, m.n_dofs)
+    rho = 2.0 * 8 ** 3
+    op = Operator(ctx, "heat", [m], rhocp=rho, dt=1.0, k0=8.0, t_boil=1.0, coef_mode=1)
+    op.set_field("t_prev", _cuda(1.0 + 0.5 * rng))
+    u = _cuda(syn.uniform_pm1(11, m.n_dofs * nrhs))
+    for beta, qmass in ((False, False), (True, False), (True, True)):
+        if beta:
+            op.set_field("beta", _cuda(syn.uniform_pm1(5, 3 * m.n_dofs) / 8))
+        if qmass:
+            op.set_field("rhocp_qpoint", _cuda(rho * (1.5 + 0.5 * syn.uniform_pm1(6, 27 * m.n_cells))))
+        for transpose in (False, True) if beta else (False,):
+            ref = op.apply(u, nrhs=nrhs, transpose=transpose)
+            v = op.apply(u.float(), nrhs=nrhs, transpose=transpose).double()
+            worst = float((v - ref).abs().max() / ref.abs().max())
+            assert worst <= 2e-5, (beta, qmass, transpose, op.variant, worst)
 
 
 # The one-launch CG takes single systems, two systems run step by step.  Both stop at ||r|| <= 1e-11 ||b||;
