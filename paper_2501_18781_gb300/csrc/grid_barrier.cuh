@@ -1,5 +1,5 @@
 // Device-side pieces of the cooperative solver kernels (internal): a bounded barrier over the grid and the
-// reduction of a value over it.
+// reduction of values over it.
 #pragma once
 
 #include "reduce.cuh"
@@ -7,41 +7,60 @@
 namespace mf {
 namespace {
 
-// Barrier over the whole (co-resident) grid; bar = {arrived, generation, timed out}.  The release of the
-// arrival and the acquire of the new generation order the blocks' global memory accesses.
+// Barrier over the whole (co-resident) grid; bar = {arrivals, timed out}, the arrivals zeroed before the launch
+// and never reset in it, so an arrival needs no answer and the blocks wait for the count itself.  (A last
+// block that resets the count and publishes a generation adds a round trip to L2: with that and the sums
+// below read one after another, the 16^3 Jacobi-CG took 5.5 ms instead of 4.4, the Schur solve of a 40^3
+// step 362 us instead of 303.  Polling every block's sum in place of a count is slower still: 5.7 ms,
+// 437 us.)  nth counts the launch's barriers from 1.  The release of the
+// arrivals and the acquire of the count order the blocks' global memory accesses.  A block that waits for
+// one second of %globaltimer sets the flag and gives up.
 __device__ __forceinline__ unsigned load_acquire(const unsigned* p) {
   unsigned v;
   asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
   return v;
 }
-__device__ __forceinline__ bool grid_barrier(unsigned* bar, unsigned nblocks) {
+__device__ __forceinline__ bool grid_barrier(unsigned* bar, unsigned nblocks, unsigned nth) {
   __shared__ bool ok;
   __syncthreads();
   if (threadIdx.x == 0) {
     ok = true;
-    const unsigned gen = load_acquire(bar + 1);
-    unsigned before;
-    asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], 1;" : "=r"(before) : "l"(bar) : "memory");
-    if (before == nblocks - 1) {
-      bar[0] = 0u;
-      asm volatile("red.add.release.gpu.global.u32 [%0], 1;" ::"l"(bar + 1) : "memory");
-    } else {
-      unsigned long long t0 = 0;
-      for (unsigned spins = 0; load_acquire(bar + 1) == gen; ++spins) {
-        if ((spins & 1023u) != 1023u) continue;
-        unsigned long long t;
-        asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-        if (!t0) t0 = t;
-        if (t - t0 > 1000000000ull || load_acquire(bar + 2)) {
-          atomicExch(bar + 2, 1u);
-          ok = false;
-          break;
-        }
+    const unsigned target = nblocks * nth;
+    asm volatile("red.add.release.gpu.global.u32 [%0], 1;" ::"l"(bar) : "memory");
+    unsigned long long t0 = 0;
+    for (unsigned spins = 0; int(load_acquire(bar) - target) < 0; ++spins) {
+      if ((spins & 1023u) != 1023u) continue;
+      unsigned long long t;
+      asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+      if (!t0) t0 = t;
+      if (t - t0 > 1000000000ull || load_acquire(bar + 1)) {
+        atomicExch(bar + 1, 1u);
+        ok = false;
+        break;
       }
     }
   }
   __syncthreads();
   return ok;
+}
+
+// Fixed-order sums of N arrays of the blocks' partial sums, value w to tot[w], the same in every block: one warp
+// per array, with the loads of up to 160 blocks in flight together.  Every thread of the block calls this.
+__device__ __forceinline__ void grid_totals(const double* part, int n, unsigned nblocks, double* tot) {
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (w < n) {
+    const double* const q = part + w * int64_t(nblocks);
+    double v[5], s = 0.0;
+#pragma unroll
+    for (int j = 0; j < 5; ++j) v[j] = lane + 32u * j < nblocks ? __ldcg(q + lane + 32 * j) : 0.0;
+#pragma unroll
+    for (int j = 0; j < 5; ++j) s += v[j];
+    for (unsigned k = lane + 160; k < nblocks; k += 32) s += __ldcg(q + k);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    if (lane == 0) tot[w] = s;
+  }
+  __syncthreads();
 }
 
 // Block sums of N values, value k to part[k * stride + blockIdx.x].  Pairs of floats down to one value per

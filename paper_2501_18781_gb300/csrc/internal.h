@@ -117,7 +117,7 @@ constexpr int kScalarsHeat = 2560;   // 8
 constexpr int kScalarsTri = 3072;    // Oseen block-triangular inner solves: 2 (k + 1) + 8 <= 512
 constexpr int kScalarsCGSteps = 3584;  // 64 step counters of the batched CG's on-device stopping test
 constexpr int kScalarsTotal = 4096;
-constexpr int kBarrierCounter = 64;    // counters: {arrived, generation, timed out} of the grid barrier
+constexpr int kBarrierCounter = 64;    // counters: {arrived, timed out} of the grid barrier
 constexpr int kCounters = 72;
 }  // namespace mf
 

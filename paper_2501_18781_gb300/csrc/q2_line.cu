@@ -3,7 +3,7 @@
 // Where one thread per cell would leave most SMs idle, nine threads work on a cell: each takes one line of
 // three values per direction, in difference form (lines.cuh), and the lines of the next direction are read
 // from shared memory.  The test side is kept without Gauss weights, which the transposes carry in their
-// constants, so a point costs one product per flux.  86 fp64 operations per thread instead of 123 with the
+// constants, so a point costs one product per flux.  88 fp64 operations per thread instead of 123 with the
 // dense 3 x 3 contractions; the fp64 pipe (16 cycles of an SM per warp instruction) bounds it together with
 // the latency of the seven phases.  16^3 cells in fp64, with the launch that zeroes the result: 18.4 -> 14.3 us.
 #include <algorithm>
@@ -190,7 +190,7 @@ __global__ void __launch_bounds__(line_threads<kCells>()) k_q2_line(const __grid
 // other of two buffers), and p . A p is summed over the cells, so a step is
 //   cells: Ap += A_cell p, p . A_cell p          barrier
 //   rows:  p, x, r, z, r . r, r . z, Ap = 0      barrier
-// 16^3 cells, 256 steps: 11.0 -> 5.5 ms; each of the five kernels of a step had paid a launch and a drained grid.
+// 16^3 cells, 256 steps: 11.0 -> 4.4 ms; each of the five kernels of a step had paid a launch and a drained grid.
 constexpr int kCgCells = 28, kCgThreads = kRedThreads;   // 252 of 256 threads work on cells
 
 struct LineCgArgs {
@@ -218,30 +218,17 @@ __global__ void __launch_bounds__(kCgThreads, 1) k_q2_line_cg(const __grid_const
   const int slot = threadIdx.x / 9, t9 = threadIdx.x % 9, i = t9 % 3, j = t9 / 3;
   const bool in_block = slot < kCgCells;
   const int64_t t0 = int64_t(blockIdx.x) * kCgThreads + threadIdx.x, st = int64_t(G) * kCgThreads;
-  // fixed-order sum of the blocks' partials, one warp per value, the same in every block
-  auto totals = [&](const double* q, int n) {
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (w < n) {
-      double s = 0.0;
-      for (unsigned k = lane; k < G; k += 32) s += __ldcg(q + w * int64_t(G) + k);
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-      if (lane == 0) tot[w] = s;
-    }
-    __syncthreads();
-  };
   const int ncells = int(A.line.ncells), cell0 = int(blockIdx.x) * kCgCells + slot;
   const bool on0 = in_block && cell0 < ncells;
   const LineCell first = line_cell(g, on0 ? cell0 : 0, i, j);
   const LineCoef<double> coef0 = line_coef(A.line, cell0, on0, i, j);
-  for (int64_t k = t0; k < A.n; k += st) A.Ap[k] = 0.0;
   const double rr0 = A.S[S_RR];
   double rz = A.S[S_RZ], rr = rr0;   // thread 0
   if (threadIdx.x == 0) {
     sbeta = 0.0;
     done = false;
   }
-  if (!grid_barrier(A.bar, G)) return;
+  __syncthreads();
   int k = 0;
   for (; k < A.maxit; ++k) {
     // p = z + beta p_old, except the first direction, which is there already
@@ -283,8 +270,8 @@ __global__ void __launch_bounds__(kCgThreads, 1) k_q2_line_cg(const __grid_const
       const double v1[1] = {acc};
       block_sums<1>(v1, [&](int, double s) { A.part[blockIdx.x] = s; });
     }
-    if (!grid_barrier(A.bar, G)) return;
-    totals(A.part, 1);
+    if (!grid_barrier(A.bar, G, 2 * k + 1)) return;
+    grid_totals(A.part, 1, G, tot);
     if (threadIdx.x == 0) salpha = tot[0] != 0.0 ? rz / tot[0] : 0.0;
     __syncthreads();
     const double alpha = salpha;
@@ -306,8 +293,8 @@ __global__ void __launch_bounds__(kCgThreads, 1) k_q2_line_cg(const __grid_const
     double* const pr = A.part + (1 + 2 * (k & 1)) * int64_t(G);
     block_sums<2>(v2, [&](int w, double s) { pr[w * int64_t(G) + blockIdx.x] = s; });
     const double pap = tot[0];
-    if (!grid_barrier(A.bar, G)) return;
-    totals(pr, 2);
+    if (!grid_barrier(A.bar, G, 2 * k + 2)) return;
+    grid_totals(pr, 2, G, tot);
     if (threadIdx.x == 0) {
       rr = tot[0];
       sbeta = rz != 0.0 ? tot[1] / rz : 0.0;
@@ -368,6 +355,8 @@ mf_status launch_q2_line_cg(mf_ctx* ctx, const mf_dofmap* m, const double* coef,
   UniformGeom g = uniform_geom(m);
   const int64_t want = std::max<int64_t>((m->n_cells + kCgCells - 1) / kCgCells, 1);
   const unsigned grid = unsigned(std::min<int64_t>(want, ctx->sm_count));
+  MF_CUDA_TRY(cudaMemsetAsync(a.bar, 0, sizeof(unsigned), ctx->stream));
+  MF_CUDA_TRY(cudaMemsetAsync(Ap, 0, sizeof(double) * a.n, ctx->stream));
   void* args[] = {&a, &g};
   const void* const k = want <= grid ? reinterpret_cast<const void*>(k_q2_line_cg<true>)
                                      : reinterpret_cast<const void*>(k_q2_line_cg<false>);

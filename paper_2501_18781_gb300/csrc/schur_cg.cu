@@ -10,8 +10,8 @@
 // outer iteration's count.  Every block adds the per-block partial sums in the same order, so all blocks
 // hold the same scalars and the result does not depend on timing.  A barrier gives up after one second
 // of %globaltimer and sets a flag.
-// Bound: latency of the barriers and of the two dependent passes, 12 us per step at 40^3 (351 us per
-// call); the 40^3 step's Schur solves went from 30 to 10 ms.  The fp64 scalars are one thread's work:
+// Bound: latency of the barriers and of the two dependent passes, 15 us per step at 40^3 (303 us per
+// call); the 40^3 step's Schur solves went from 30 to 8.8 ms.  The fp64 scalars are one thread's work:
 // divisions in all 32 warps took 8 us per step, the fp64 sums over all of them 5 us.
 #include <cuda_fp16.h>
 
@@ -133,18 +133,6 @@ __global__ void __launch_bounds__(kThreads, 1) k_schur_cg(const SchurArgs A) {
       if (PARTS > 1) __syncthreads();
     }
   };
-  // fixed-order sums of N arrays of the blocks' partials, the same in every block: warp k adds array k
-  auto totals = [&](const double* q, int n) {
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (w < n) {
-      double s = 0.0;
-      for (unsigned k = lane; k < G; k += 32) s += __ldcg(q + w * int64_t(G) + k);
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-      if (lane == 0) tot[w] = s;
-    }
-    __syncthreads();
-  };
   Dot2f arr, arz;
   if (own)
     for (int i = t0; i < np; i += step) {
@@ -160,8 +148,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_schur_cg(const SchurArgs A) {
   for (; k < A.maxit; ++k) {
     Dot2f v2[2] = {arr, arz};
     block_partials<2>(v2, sh, A.part, G);
-    if (!grid_barrier(A.bar, G)) return;
-    totals(A.part, 2);
+    if (!grid_barrier(A.bar, G, 2 * k + 1)) return;
+    grid_totals(A.part, 2, G, tot);
     if (threadIdx.x == 0) {
       if (k == 0) stop = A.tol2 * tot[0];
       done = tot[0] <= stop;   // converged, or a zero right-hand side
@@ -173,8 +161,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_schur_cg(const SchurArgs A) {
     Dot2f v1[1];
     apply(k, coef_s, v1[0]);
     block_partials<1>(v1, sh, A.part + 2 * int64_t(G), G);
-    if (!grid_barrier(A.bar, G)) return;
-    totals(A.part + 2 * int64_t(G), 1);
+    if (!grid_barrier(A.bar, G, 2 * k + 2)) return;
+    grid_totals(A.part + 2 * int64_t(G), 1, G, tot);
     if (threadIdx.x == 0) {
       done = !(tot[0] > 0.0);   // a breakdown: x stays as it is
       coef_s = float(rz / tot[0]);
@@ -210,6 +198,8 @@ template <int PARTS> cudaError_t start(mf_ctx* ctx, SchurArgs& a, int64_t np) {
     const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(bytes));
     if (e != cudaSuccess) return e;
   }
+  const cudaError_t e = cudaMemsetAsync(a.bar, 0, sizeof(unsigned), ctx->stream);
+  if (e != cudaSuccess) return e;
   void* args[] = {&a};
   return cudaLaunchCooperativeKernel(k, dim3(grid), dim3(kThreads), args, bytes, ctx->stream);
 }
@@ -247,14 +237,14 @@ mf_status launch_schur_cg(mf_ctx* ctx, const void* S, const float* scale, const 
   return MF_OK;
 }
 
-// MF_ETIMEOUT (once, then the barrier is reset) if the barrier of a cooperative launch gave up
+// MF_ETIMEOUT (once) if the barrier of a cooperative launch gave up
 mf_status grid_barrier_take_error(mf_ctx* ctx) {
-  unsigned bar[3] = {0u, 0u, 0u};
-  unsigned* const d = ctx->counters.as<unsigned>() + kBarrierCounter;
-  MF_CUDA_TRY(cudaMemcpyAsync(bar, d, sizeof bar, cudaMemcpyDeviceToHost, ctx->stream));
+  unsigned timed_out = 0u;
+  unsigned* const d = ctx->counters.as<unsigned>() + kBarrierCounter + 1;
+  MF_CUDA_TRY(cudaMemcpyAsync(&timed_out, d, sizeof timed_out, cudaMemcpyDeviceToHost, ctx->stream));
   MF_CUDA_TRY(cudaStreamSynchronize(ctx->stream));
-  if (!bar[2]) return MF_OK;
-  MF_CUDA_TRY(cudaMemsetAsync(d, 0, sizeof bar, ctx->stream));
+  if (!timed_out) return MF_OK;
+  MF_CUDA_TRY(cudaMemsetAsync(d, 0, sizeof timed_out, ctx->stream));
   return fail(MF_ETIMEOUT, "a grid barrier of a solver kernel timed out");
 }
 
