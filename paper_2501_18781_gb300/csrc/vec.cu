@@ -366,6 +366,31 @@ __global__ void k_cheb_step(int64_t n, int64_t ld, T* z, const T* res_in, T* res
   }
 }
 
+// Up to this many products are added up by the last block of the launch that formed their partial sums: one
+// warp per product.  k_multidot_finish took 4.7 us beside the 12 us of five products of 1.6 M fp32 elements;
+// with more products the one block's fp64 adds (16 cycles of its SM per warp instruction) take longer than that.
+constexpr int kFusedDots = kRedThreads / 32;
+__device__ __forceinline__ void finish_dots_if_last(const double* part, int k, double* h, unsigned* count) {
+  if (!count) return;
+  __shared__ unsigned last;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicAdd(count, 1u) == gridDim.x - 1 ? 1u : 0u;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  const int j = threadIdx.x >> 5, lane = threadIdx.x & 31, g = int(gridDim.x);
+  if (j < k) {
+    double s = 0.0;
+#pragma unroll 4
+    for (int i = lane; i < g; i += 32) s += __ldcg(part + int64_t(j) * g + i);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    if (lane == 0) h[j] = s;
+  }
+  if (threadIdx.x == 0) *count = 0u;
+}
+
 // CGS2 pieces of the GMRES solvers.  V holds k basis vectors ld apart.  Where V and w start on
 // 16-byte boundaries and ld * sizeof(T) is a multiple of 16 (the solvers pad their bases so),
 // every thread moves 16-byte words (four floats or two doubles), so each step of a thread has
@@ -402,7 +427,7 @@ __device__ __forceinline__ void multidot_group(const T* V, int64_t ld, const T* 
 // h_j partials of V_j . w for j < k: groups of eight vectors, then one group of the rest
 template <typename T, int W>
 __global__ void __launch_bounds__(kRedThreads, 4) k_multidot(const T* V, int64_t ld, int k, const T* w, int64_t n,
-                                                             double* part) {
+                                                             double* part, double* h, unsigned* count) {
   int j0 = 0;
   for (; j0 + 8 <= k; j0 += 8) multidot_group<T, 8, W>(V + j0 * ld, ld, w, n, part, j0);
   const T* Vr = V + j0 * ld;
@@ -416,6 +441,7 @@ __global__ void __launch_bounds__(kRedThreads, 4) k_multidot(const T* V, int64_t
     case 7: multidot_group<T, 7, W>(Vr, ld, w, n, part, j0); break;
     default: break;
   }
+  finish_dots_if_last(part, k, h, count);
 }
 // The first pass's update and the second pass's products of classical Gram-Schmidt in one sweep,
 // for KG <= 8 vectors: w <- w + sign V h (T arithmetic, as k_multiaxpy), then part[g] = the
@@ -423,7 +449,8 @@ __global__ void __launch_bounds__(kRedThreads, 4) k_multidot(const T* V, int64_t
 // the two separate launches bit for bit).
 template <typename T, int KG, int W>
 __global__ void __launch_bounds__(kRedThreads, 4) k_axpy_multidot(const T* V, int64_t ld, const double* h, double sign,
-                                                                  T* w, int64_t n, double* part) {
+                                                                  T* w, int64_t n, double* part, double* h2,
+                                                                  unsigned* count) {
   using Wd = Word<T, W>;
   __shared__ T hs[KG];
   if (threadIdx.x < KG) hs[threadIdx.x] = T(sign * h[threadIdx.x]);
@@ -458,6 +485,7 @@ __global__ void __launch_bounds__(kRedThreads, 4) k_axpy_multidot(const T* V, in
       for (int g = 0; g < KG; ++g) acc[g].add(V[g * ld + i], y);
     }
   block_sums<KG>(acc, [&](int g, double t) { part[int64_t(g) * gridDim.x + blockIdx.x] = t; });
+  finish_dots_if_last(part, KG, h2, count);
 }
 
 __global__ void __launch_bounds__(kRedThreads) k_multidot_finish(const double* part, int g, double* h) {
@@ -793,13 +821,16 @@ template <typename T> mf_status multidot(mf_ctx* ctx, const T* V, int64_t ld, in
   const int g = red_blocks(n);
   double* part;
   MF_TRY(scratch(ctx, size_t(g) * (k + 1) + 64, &part));
+  unsigned* const count = k <= kFusedDots ? counters(ctx) : nullptr;
   if (words16(V, ld) && words16(w, 0))
-    k_multidot<T, 16 / sizeof(T)><<<g, kRedThreads, 0, ctx->stream>>>(V, ld, k, w, n, part);
+    k_multidot<T, 16 / sizeof(T)><<<g, kRedThreads, 0, ctx->stream>>>(V, ld, k, w, n, part, h, count);
   else
-    k_multidot<T, 1><<<g, kRedThreads, 0, ctx->stream>>>(V, ld, k, w, n, part);
+    k_multidot<T, 1><<<g, kRedThreads, 0, ctx->stream>>>(V, ld, k, w, n, part, h, count);
   LAUNCH_CHECK();
-  k_multidot_finish<<<k, kRedThreads, 0, ctx->stream>>>(part, g, h);
-  LAUNCH_CHECK();
+  if (!count) {
+    k_multidot_finish<<<k, kRedThreads, 0, ctx->stream>>>(part, g, h);
+    LAUNCH_CHECK();
+  }
   return MF_OK;
 }
 template mf_status multidot<double>(mf_ctx*, const double*, int64_t, int, const double*, int64_t, double*);
@@ -811,26 +842,26 @@ template <typename T> constexpr int kAxpyDotMax = sizeof(T) == 4 ? 6 : 2;
 
 template <typename T, int W>
 static void launch_axpy_multidot(mf_ctx* ctx, const T* V, int64_t ld, int k, const double* h, double sign, T* w,
-                                 int64_t n, double* part) {
+                                 int64_t n, double* part, double* h2, unsigned* count) {
   const int g = red_blocks(n);
   switch (k) {
-    case 1: k_axpy_multidot<T, 1, W><<<g, kRedThreads, 0, ctx->stream>>>(V, ld, h, sign, w, n, part); break;
-    case 2: k_axpy_multidot<T, 2, W><<<g, kRedThreads, 0, ctx->stream>>>(V, ld, h, sign, w, n, part); break;
+    case 1: k_axpy_multidot<T, 1, W><<<g, kRedThreads, 0, ctx->stream>>>(V, ld, h, sign, w, n, part, h2, count); break;
+    case 2: k_axpy_multidot<T, 2, W><<<g, kRedThreads, 0, ctx->stream>>>(V, ld, h, sign, w, n, part, h2, count); break;
     case 3:
       if constexpr (kAxpyDotMax<T> >= 3)
-        k_axpy_multidot<T, 3, W><<<g, kRedThreads, 0, ctx->stream>>>(V, ld, h, sign, w, n, part);
+        k_axpy_multidot<T, 3, W><<<g, kRedThreads, 0, ctx->stream>>>(V, ld, h, sign, w, n, part, h2, count);
       break;
     case 4:
       if constexpr (kAxpyDotMax<T> >= 4)
-        k_axpy_multidot<T, 4, W><<<g, kRedThreads, 0, ctx->stream>>>(V, ld, h, sign, w, n, part);
+        k_axpy_multidot<T, 4, W><<<g, kRedThreads, 0, ctx->stream>>>(V, ld, h, sign, w, n, part, h2, count);
       break;
     case 5:
       if constexpr (kAxpyDotMax<T> >= 5)
-        k_axpy_multidot<T, 5, W><<<g, kRedThreads, 0, ctx->stream>>>(V, ld, h, sign, w, n, part);
+        k_axpy_multidot<T, 5, W><<<g, kRedThreads, 0, ctx->stream>>>(V, ld, h, sign, w, n, part, h2, count);
       break;
     default:
       if constexpr (kAxpyDotMax<T> >= 6)
-        k_axpy_multidot<T, 6, W><<<g, kRedThreads, 0, ctx->stream>>>(V, ld, h, sign, w, n, part);
+        k_axpy_multidot<T, 6, W><<<g, kRedThreads, 0, ctx->stream>>>(V, ld, h, sign, w, n, part, h2, count);
       break;
   }
 }
@@ -847,11 +878,9 @@ mf_status axpy_multidot(mf_ctx* ctx, const T* V, int64_t ld, int k, const double
   double* part;
   MF_TRY(scratch(ctx, size_t(g) * (k + 1) + 64, &part));
   if (words16(V, ld) && words16(w, 0))
-    launch_axpy_multidot<T, 16 / sizeof(T)>(ctx, V, ld, k, h, sign, w, n, part);
+    launch_axpy_multidot<T, 16 / sizeof(T)>(ctx, V, ld, k, h, sign, w, n, part, h2, counters(ctx));
   else
-    launch_axpy_multidot<T, 1>(ctx, V, ld, k, h, sign, w, n, part);
-  LAUNCH_CHECK();
-  k_multidot_finish<<<k, kRedThreads, 0, ctx->stream>>>(part, g, h2);
+    launch_axpy_multidot<T, 1>(ctx, V, ld, k, h, sign, w, n, part, h2, counters(ctx));
   LAUNCH_CHECK();
   return MF_OK;
 }
@@ -862,7 +891,8 @@ mf_status multiaxpy(mf_ctx* ctx, const T* V, int64_t ld, int k, const double* h,
   if (k > 64) return fail(MF_EINVAL, "multiaxpy: at most 64 vectors");
   if (k < 1 && !norm2) return MF_OK;
   const bool words = words16(V, ld) && words16(w, 0);
-  const int g = grid_for(n);
+  // with the norm, as many blocks as the reductions: their partial sums are added by one block
+  const int g = norm2 ? red_blocks(n) : grid_for(n);
   if (norm2) {
     double* part;
     MF_TRY(scratch(ctx, size_t(g), &part));
