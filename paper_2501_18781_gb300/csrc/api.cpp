@@ -936,20 +936,26 @@ mf_status apply_impl(mf_op* op, const T* src, T* dst, int nrhs, int64_t ld, bool
       if (df) {
         // double-float: one warp per velocity component over a brick of 32 cells (the Darcy term is
         // folded into cm; the trace correction reads the interface normal pairs)
-        const int64_t nc = op->ncells;
         const bool ext = op->p.oseen_flags != 0;
+        bool ok = true;
         if (!op->df_ready) {
-          MF_TRY(op->cm_df.alloc(sizeof(float2) * 27 * nc));
-          MF_TRY(op->cv_df.alloc(sizeof(float2) * 27 * nc));
-          MF_TRY(op->cb_df.alloc(sizeof(float2) * 81 * nc));
-          MF_TRY(launch_oseen_df_split(c, op->map[0], op->cm64.as<double>(), op->cv64.as<double>(), op->cb64.as<double>(),
-                                       op->cm_df.as<float2>(), op->cv_df.as<float2>(), op->cb_df.as<float2>()));
-          if (ext) {
-            MF_TRY(op->nrm_df.alloc(sizeof(float2) * 81 * nc));
-            MF_TRY(launch_split_pairs(c, op->nrm64.as<double>(), 81 * nc, 1.0, op->nrm_df.as<float2>()));
+          // tables per tile of 32 cells, padded to whole tiles; without the memory the fp64 pipes do it
+          const size_t one = sizeof(float2) * tile_table_floats(op->map[0], 1);
+          mf_status st = op->cm_df.alloc(one);
+          if (st == MF_OK) st = op->cv_df.alloc(one);
+          if (st == MF_OK) st = op->cb_df.alloc(3 * one);
+          if (st == MF_OK && ext) st = op->nrm_df.alloc(3 * one);
+          ok = st != MF_ENOMEM;
+          if (ok) {
+            MF_TRY(st);
+            MF_TRY(launch_oseen_df_split(c, op->map[0], op->cm64.as<double>(), op->cv64.as<double>(), op->cb64.as<double>(),
+                                         ext ? op->nrm64.as<double>() : nullptr, op->cm_df.as<float2>(),
+                                         op->cv_df.as<float2>(), op->cb_df.as<float2>(),
+                                         ext ? op->nrm_df.as<float2>() : nullptr));
+            op->df_ready = true;
           }
-          op->df_ready = true;
         }
+        if (!ok) return apply_impl<T>(op, src, dst, nrhs, ld, transpose, PREC_F64);
         for (int r = 0; r < nrhs; ++r) {
           MF_TRY(launch_oseen_df_uniform(c, op->map[0], reinterpret_cast<const double*>(src + r * ld),
                                          reinterpret_cast<double*>(dst + r * ld), op->cm_df.as<float2>(),

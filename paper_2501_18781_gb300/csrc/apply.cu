@@ -9,7 +9,6 @@ mf_status launch_scalar_apply_f32(mf_ctx*, const mf_dofmap*, int, int, bool, boo
 mf_status launch_scalar_apply_df64(mf_ctx*, const mf_dofmap*, int, int, bool, bool, const ScalarArgs<double>&);
 mf_status launch_oseen_apply_f64(mf_ctx*, const mf_dofmap*, const OseenArgs<double>&);
 mf_status launch_oseen_apply_f32(mf_ctx*, const mf_dofmap*, const OseenArgs<float>&);
-mf_status launch_oseen_apply_df64(mf_ctx*, const mf_dofmap*, const OseenArgs<double>&);
 
 namespace {
 
@@ -67,7 +66,6 @@ mf_status launch_scalar_apply(mf_ctx* ctx, const mf_dofmap* m, int kind, int mod
 
 mf_status launch_oseen_apply(mf_ctx* ctx, const mf_dofmap* mu, int prec, const void* args) {
   if (prec == PREC_F32) return launch_oseen_apply_f32(ctx, mu, *static_cast<const OseenArgs<float>*>(args));
-  if (prec == PREC_DF64) return launch_oseen_apply_df64(ctx, mu, *static_cast<const OseenArgs<double>*>(args));
   return launch_oseen_apply_f64(ctx, mu, *static_cast<const OseenArgs<double>*>(args));
 }
 

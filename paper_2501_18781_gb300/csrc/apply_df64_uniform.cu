@@ -274,21 +274,27 @@ __global__ void __launch_bounds__(kThreads, 4) k_scalar_df_uniform(const __grid_
 // d_a u_a.  Then planes (a, c): the flux along c with its half d_a u_c, the transpose along c of the
 // whole test side, and the value transpose along a.  So each derivative is taken by whole lines, and the
 // rolled loops over planes keep the three warps inside a short instruction body.
-// Bound: fp32 instruction issue at 12 warps per SM (48 KB of shared memory per block).  46.8k instead of
-// 72.9k instructions per 32 cells at 60 % instead of 46 % of the issue slots: 64^3 1105 -> 539 us.
+// Bound: fp32 instruction issue at 12 warps per SM (48 KB of shared memory per block).  45.9k instead of
+// 72.9k instructions per 32 cells at 63 % instead of 46 % of the issue slots: 64^3 1105 -> 505 us (539 with
+// tables over cells, whose rows took 64-bit address arithmetic; per tile they share the offsets of the
+// shared arrays, and one instruction per table fetches a tile into L2).
 
 struct DfOseenArgs {
   const double* src;
   double* dst;
   int64_t nu;              // velocity DoFs per component (pressure block starts at 3 nu)
-  const float2* cm;        // [27][ncells] w h^3 sigma rho (+ Darcy)
-  const float2* cv;        // [27][ncells] (5/3) w h mu
-  const float2* cb;        // [3][27][ncells] w h^2 rho beta / (2 delta)
-  const float2* nr;        // melt-pool trace correction: interface normal per Gauss point, [3][27][ncells]
-  int64_t ncells;
+  // per tile of 8 x 4 x 1 cells as [q][lane]; lanes without a cell 0
+  const float2* cm;        // [tile][27][32] w h^3 sigma rho (+ Darcy)
+  const float2* cv;        // [tile][27][32] (5/3) w h mu
+  const float2* cb;        // [tile][81][32] w h^2 rho beta / (2 delta)
+  const float2* nr;        // melt-pool trace correction: interface normal per Gauss point, [tile][81][32]
   float2 pw[27];           // -h^2 w_q / (2 delta): pressure term of the gradient test
   float2 mh2;              // -h^2 / (2 delta): continuity rows
 };
+
+__device__ __forceinline__ void prefetch_l2(const float2* p, unsigned bytes) {
+  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
+}
 
 __device__ __forceinline__ float pow2f(int e) {  // 2^e for e in [-126, 127]; 0 below
   return e < -126 ? 0.f : __uint_as_float(unsigned(min(e, 127) + 127) << 23);
@@ -314,21 +320,25 @@ __global__ void __launch_bounds__(96, 4) k_oseen_df_uniform(const __grid_constan
   const int blk = blockIdx.x;
   const int i = (blk % nbx) * 8 + (lane & 7), j = ((blk / nbx) % nby) * 4 + (lane >> 3), k = blk / (nbx * nby);
   const bool active = i < ug.nx && j < ug.ny;
-  const int64_t cell = active ? i + int64_t(ug.nx) * (j + int64_t(ug.ny) * k) : 0;
   const int64_t base = active ? 2 * int64_t(i) + ug.sx * (2 * int64_t(j)) + ug.sy * (2 * int64_t(k)) : 0;
   const uint32_t dmask = active ? dirichlet_mask(ug, i, j, k) : 0u;
   const int64_t px = ug.nx + 1, pxy = px * (ug.ny + 1);
   const int64_t pbase = active ? i + px * (j + (ug.ny + 1) * int64_t(k)) : 0;
-  const int64_t nc = A.ncells;
-  // L2 prefetch of the coefficient tables while the inputs load and the sweeps run: a brick row's 8
-  // cells share 64 bytes of every table row, fetched by the brick row's 24 lanes as 32-byte halves
-  if (j < ug.ny) {
-    const int64_t row_cell = int64_t(i - (lane & 7)) + int64_t(ug.nx) * (j + int64_t(ug.ny) * k);
-#pragma unroll 1
-    for (int r = w * 8 + (lane & 7); r < 270; r += 24) {
-      const int rr = r >> 1;
-      const float2* t = rr < 27 ? A.cv + rr * nc : rr < 54 ? A.cm + (rr - 27) * nc : A.cb + (rr - 54) * nc;
-      if (!(r & 1) || i - (lane & 7) + 4 < ug.nx) asm volatile("prefetch.global.L2 [%0];" ::"l"(t + row_cell + 4 * (r & 1)));
+  // the tile's coefficients, addressed by the offsets of the shared arrays
+  const float2* __restrict__ const tm = A.cm + int64_t(blk) * (27 * 32) + lane;
+  const float2* __restrict__ const tv = A.cv + int64_t(blk) * (27 * 32) + lane;
+  const float2* __restrict__ const tb = A.cb + int64_t(blk) * (81 * 32) + lane;
+  const float2* __restrict__ const tn = A.nr + int64_t(blk) * (81 * 32) + lane;
+  // into L2 while the inputs load and the sweeps run
+  if (lane == 0) {
+    constexpr unsigned kRow = 32 * sizeof(float2);
+    if (w == 0) {
+      prefetch_l2(tv, 27 * kRow);
+      prefetch_l2(tm, 27 * kRow);
+    } else if (w == 1) {
+      prefetch_l2(tb, 81 * kRow);
+    } else if (EXT) {
+      prefetch_l2(tn, 81 * kRow);
     }
   }
   // raw inputs: this warp's velocity component (Dirichlet nodes and lanes without a cell read as 0)
@@ -440,7 +450,7 @@ __global__ void __launch_bounds__(96, 4) k_oseen_df_uniform(const __grid_constan
       const dd v0 = ld2(z), v1 = ld2(z + 9 * 32), v2 = ld2(z + 18 * 32);
       const dd cc = dd_sub(dd_add(v0, v2), dd_pow2(v1, 2.f));
       const dd div = dd_norm(dd_add(D[p], dd_add(dd_sub(v2, v0), dd_pow2(cc, sg))));
-      const dd cv = ldg2(A.cv + (p + 9 * w) * nc + cell);
+      const dd cv = ldg2(tv + (p + 9 * w) * 32);
       st2(sT + (p + 9 * w) * 32, dd_norm(dd_pow2(dd_mul(cv, div), -2.f)));
     }
     __syncthreads();
@@ -448,7 +458,7 @@ __global__ void __launch_bounds__(96, 4) k_oseen_df_uniform(const __grid_constan
   // permuted axes: a = own direction, b and c the others (strides in the 27-array)
   const int sa = w == 0 ? 1 : (w == 1 ? 3 : 9), sb = w == 1 ? 1 : 3, sc = w == 2 ? 1 : 9;
   const int eb = w == 1 ? 0 : 1, ec = w == 2 ? 0 : 2;
-  const int64_t na = sa * nc, nb = sb * nc, ncc = sc * nc;
+  const int na = sa * 32, nb = sb * 32, ncc = sc * 32;
   const float2* const uC = sU + 27 * w * 32;
   dd Rp[8];
 #pragma unroll
@@ -456,11 +466,10 @@ __global__ void __launch_bounds__(96, 4) k_oseen_df_uniform(const __grid_constan
 #pragma unroll 1
   for (int ic = 0; ic < 3; ++ic) {
     const int o = ic * sc * 32;
-    const int64_t og = ic * ncc + cell;
-    const float2* __restrict__ gm = A.cm + og;
-    const float2* __restrict__ gv = A.cv + og;
-    const float2* __restrict__ ga = A.cb + 27 * w * nc + og;
-    const float2* __restrict__ gb = A.cb + 27 * eb * nc + og;
+    const float2* __restrict__ gm = tm + o;
+    const float2* __restrict__ gv = tv + o;
+    const float2* __restrict__ ga = tb + 27 * 32 * w + o;
+    const float2* __restrict__ gb = tb + 27 * 32 * eb + o;
     dd U[9], R[9], cv[9];
 #pragma unroll
     for (int p = 0; p < 9; ++p) {
@@ -522,11 +531,11 @@ __global__ void __launch_bounds__(96, 4) k_oseen_df_uniform(const __grid_constan
     if (EXT) {
 #pragma unroll
       for (int p = 0; p < 9; ++p) {
-        const int64_t on = og + (p % 3) * na + (p / 3) * nb;
-        const dd nA = ldg2(A.nr + 27 * w * nc + on), nB = ldg2(A.nr + 27 * eb * nc + on);
-        const dd tn = dd_mul(dd_pow2(ld2(sT + o + ((p % 3) * sa + (p / 3) * sb) * 32), su), nA);
-        fa[p] = dd_fma(fa[p], tn, nA);
-        fb[p] = dd_fma(fb[p], tn, nB);
+        const int on = o + (p % 3) * na + (p / 3) * nb;
+        const dd nA = ldg2(tn + 27 * 32 * w + on), nB = ldg2(tn + 27 * 32 * eb + on);
+        const dd tA = dd_mul(dd_pow2(ld2(sT + o + ((p % 3) * sa + (p / 3) * sb) * 32), su), nA);
+        fa[p] = dd_fma(fa[p], tA, nA);
+        fb[p] = dd_fma(fb[p], tA, nB);
       }
     }
 #pragma unroll
@@ -553,7 +562,6 @@ __global__ void __launch_bounds__(96, 4) k_oseen_df_uniform(const __grid_constan
 #pragma unroll 1
   for (int ib = 0; ib < 3; ++ib) {
     const int o = ib * sb * 32;
-    const int64_t og = ib * nb + cell;
     dd X[9], V[9];   // index ia + 3 ic
     const float2* const uc = sU + 27 * ec * 32 + o;
 #pragma unroll
@@ -564,16 +572,15 @@ __global__ void __launch_bounds__(96, 4) k_oseen_df_uniform(const __grid_constan
 #pragma unroll
     for (int m = 0; m < 3; ++m) {
       const int om = o + m * sa * 32;
-      const int64_t gm = og + m * na;
       dd g[3], f[3];
       dd_line_deriv(ld2(uC + om), ld2(uC + om + sc * 32), ld2(uC + om + 2 * sc * 32), g[0], g[1], g[2]);
 #pragma unroll
       for (int n = 0; n < 3; ++n) {
         const int p = m + 3 * n;
-        f[n] = dd_pow2(dd_mul(ldg2(A.cv + gm + n * ncc), dd_add(g[n], X[p])), su);
-        V[p] = dd_add(ld2(sV + om + n * sc * 32), dd_pow2(dd_mul(ldg2(A.cb + 27 * ec * nc + gm + n * ncc), g[n]), su));
+        f[n] = dd_pow2(dd_mul(ldg2(tv + om + n * ncc), dd_add(g[n], X[p])), su);
+        V[p] = dd_add(ld2(sV + om + n * sc * 32), dd_pow2(dd_mul(ldg2(tb + 27 * 32 * ec + om + n * ncc), g[n]), su));
         if (EXT) {
-          const dd nA = ldg2(A.nr + 27 * w * nc + gm + n * ncc), nC = ldg2(A.nr + 27 * ec * nc + gm + n * ncc);
+          const dd nA = ldg2(tn + 27 * 32 * w + om + n * ncc), nC = ldg2(tn + 27 * 32 * ec + om + n * ncc);
           f[n] = dd_fma(f[n], dd_mul(dd_pow2(ld2(sT + om + n * sc * 32), su), nA), nC);
         }
       }
@@ -614,6 +621,25 @@ __global__ void k_split_plain(const double* __restrict__ c, int64_t n, double s,
   const double v = c[t] * s;
   const float hi = __double2float_rn(v);
   out[t] = make_float2(hi, __double2float_rn(v - double(hi)));
+}
+
+// s c of a [rows][ncells] table as float pairs, per tile of 8 x 4 x 1 cells: [tile][rows][32]
+__global__ void k_split_tiles(const double* __restrict__ c, int rows, double s, float2* __restrict__ out, int ntx, int nty,
+                              UniformGeom ug) {
+  const int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+  const int64_t nc = int64_t(ug.nx) * ug.ny * ug.nz;
+  if (t >= int64_t(ntx) * nty * ug.nz * 32) return;
+  const int lane = int(t & 31);
+  const int64_t tile = t >> 5;
+  const int col = int(tile % (ntx * nty)), k = int(tile / (ntx * nty));
+  const int i = (col % ntx) * 8 + (lane & 7), j = (col / ntx) * 4 + (lane >> 3);
+  const bool active = i < ug.nx && j < ug.ny;
+  const int64_t cell = i + int64_t(ug.nx) * (j + int64_t(ug.ny) * k);
+  for (int r = 0; r < rows; ++r) {
+    const double v = active ? c[r * nc + cell] * s : 0.0;
+    const float hi = __double2float_rn(v);
+    out[(tile * rows + r) * 32 + lane] = make_float2(hi, __double2float_rn(v - double(hi)));
+  }
 }
 
 // w_q s c_q of a Gauss-point table ([27][ncells] or [3][27][ncells]) as float pairs
@@ -703,13 +729,24 @@ mf_status launch_split_pairs(mf_ctx* ctx, const double* c, int64_t n, double sca
   return MF_OK;
 }
 
-// cv carries both derivative factors 1 / (2 delta) of the viscous term, cb the one of the convection
+static mf_status launch_split_tiles(mf_ctx* ctx, const mf_dofmap* m, const double* c, int rows, double scale, float2* out) {
+  const UniformGeom ug = uniform_geom(m);
+  const int ntx = (ug.nx + 7) / 8, nty = (ug.ny + 3) / 4;
+  const int64_t n = int64_t(ntx) * nty * ug.nz * 32;
+  k_split_tiles<<<unsigned((n + 127) / 128), 128, 0, ctx->stream>>>(c, rows, scale, out, ntx, nty, ug);
+  ctx->launches++;
+  MF_CUDA_TRY(cudaGetLastError());
+  return MF_OK;
+}
+
+// cv carries both derivative factors 1 / (2 delta) of the viscous term, cb the one of the convection; nr64, nr:
+// the interface normals, or NULL
 mf_status launch_oseen_df_split(mf_ctx* ctx, const mf_dofmap* mu, const double* cm64, const double* cv64,
-                                const double* cb64, float2* cm, float2* cv, float2* cb) {
-  const int64_t nc = mu->n_cells;
-  MF_TRY(launch_split_pairs(ctx, cm64, 27 * nc, 1.0, cm));
-  MF_TRY(launch_split_pairs(ctx, cv64, 27 * nc, 5.0 / 3.0, cv));
-  return launch_split_pairs(ctx, cb64, 81 * nc, kDerivScale, cb);
+                                const double* cb64, const double* nr64, float2* cm, float2* cv, float2* cb, float2* nr) {
+  MF_TRY(launch_split_tiles(ctx, mu, cm64, 27, 1.0, cm));
+  MF_TRY(launch_split_tiles(ctx, mu, cv64, 27, 5.0 / 3.0, cv));
+  MF_TRY(launch_split_tiles(ctx, mu, cb64, 81, kDerivScale, cb));
+  return nr64 ? launch_split_tiles(ctx, mu, nr64, 81, 1.0, nr) : MF_OK;
 }
 
 mf_status launch_oseen_df_uniform(mf_ctx* ctx, const mf_dofmap* mu, const double* src, double* dst, const float2* cm,
@@ -728,7 +765,6 @@ mf_status launch_oseen_df_uniform(mf_ctx* ctx, const mf_dofmap* mu, const double
   a.src = src;
   a.dst = dst;
   a.nu = mu->n_dofs;
-  a.ncells = mu->n_cells;
   a.cm = cm;
   a.cv = cv;
   a.cb = cb;

@@ -179,7 +179,7 @@ mf_status launch_oseen_f32_uniform(mf_ctx* ctx, const mf_dofmap* mu, const float
 // (81 per cell, pairs) for the trace correction, or NULL without the melt-pool terms
 mf_status launch_split_pairs(mf_ctx* ctx, const double* c, int64_t n, double scale, float2* out);
 mf_status launch_oseen_df_split(mf_ctx* ctx, const mf_dofmap* mu, const double* cm64, const double* cv64,
-                                const double* cb64, float2* cm, float2* cv, float2* cb);
+                                const double* cb64, const double* nr64, float2* cm, float2* cv, float2* cb, float2* nr);
 mf_status launch_oseen_df_uniform(mf_ctx* ctx, const mf_dofmap* mu, const double* src, double* dst, const float2* cm,
                                   const float2* cv, const float2* cb, const float2* nr);
 // laser top-face load and its parameter derivatives (uniform maps)
