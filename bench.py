@@ -36,24 +36,22 @@ METRIC = "GDoF/s of matrix-free operator apply & %HBM roofline; CG solve time FP
 WORKLOAD = "heat_laser_q2_128"
 HBM_FALLBACK_GBS = 6800.0
 FP64_PEAK_TFLOPS = 1.25      # GB300 FP64 (vector and tensor) rate of the profiling recipe's table
-# Algorithmic flops of one scalar Q2 heat-cell apply as the kernel performs it (FMA = 2).  The 1D
-# sweeps skip the exact zeros and ones of the 3-point tables (the middle Gauss point is the middle
-# node; D[1][1] = 0): a value sweep costs 9 lines x 2 points x 5 = 90 (three sweeps 270), an
-# integration sweep 9 x 10 = 90 (three sweeps 270); the reference gradient at the 27 points costs
-# 3 x (9 x 3 + 18 x 5) = 351 and its transposed test accumulation 3 x (9 x 4 + 18 x 6) = 432; per
-# point the mass term w (m h^2) u (2), the conductivity factor w k and its three products (4) and the
-# value accumulation (1) make 27 x 7 = 189; the final h scaling 27: 1539 with k tabulated per Gauss
-# point.  With k evaluated in the kernel, the nodal T^n is swept to the Gauss points (270) and
-# k0 + s T applied (27 x 2): 1863.
-HEAT_FLOPS_PER_CELL = {"tabulated": 1539, "inkernel": 1863}
+# Algorithmic flops of one scalar Q2 heat-cell apply as the kernel performs it (FMA = 2), lines in
+# difference form and Gauss weights inside the transposes.  Value lines 27 x 9 = 243, the mass term
+# 27, derivative lines 27 x 8 = 216, the products with the coefficient 81, derivative transposes in x
+# and y 18 x 12 = 216, the combined z transposes 9 x 19 = 171, value transposes in x and y 18 x 9 = 162:
+# 1116 with k tabulated per Gauss point.  With k evaluated in the kernel, the nodal T^n is swept to the
+# Gauss points (243) and k0 + s T applied (27 x 2): 1413.
+HEAT_FLOPS_PER_CELL = {"tabulated": 1116, "inkernel": 1413}
 # The double-float kernel evaluates the same cell operator in pairs of fp32 (tabulated w h k): per
-# cell 8559 fp32 instructions, 11151 flops with an FMA counted as two (a pair product is 1 FMUL + 3
-# FFMA, a pair sum 8 FADD, a renormalisation 3 FADD): value sweeps 1674 / 2160, z fluxes 837 / 1134,
-# z test parts 972 / 1269, x and y gradients, fluxes and test parts 3240 / 4266, renormalisation 81 /
-# 81, transposed x and y sweeps 1170 / 1494, transposed z sweep 585 / 747.  Its roof is the fp32
-# pipe: 152 SMs x 128 lanes x 2 flops x 2.07 GHz (the profiling recipe's unit count and SM clock).
-HEAT_DF64_FLOPS_PER_CELL = 11151
-HEAT_DF64_INSTRUCTIONS_PER_CELL = 8559
+# cell 6525 fp32 instructions, 7335 flops with an FMA counted as two (a pair product is 1 FMUL + 3
+# FFMA, a pair sum 8 FADD, a renormalisation 3 FADD, a power of two 2 FMUL): value lines 27 x 58 / 67,
+# the mass term 108 / 189, derivative lines 27 x 44, the products with the coefficient 324 / 567,
+# derivative transposes 18 x 68, combined z transposes 9 x 113 / 122, value transposes 18 x 52 / 61,
+# renormalisations 162.  Its roof is the fp32 pipe: 152 SMs x 128 lanes x 2 flops x 2.07 GHz (the
+# profiling recipe's unit count and SM clock).
+HEAT_DF64_FLOPS_PER_CELL = 7335
+HEAT_DF64_INSTRUCTIONS_PER_CELL = 6525
 FP32_PEAK_TFLOPS = 152 * 128 * 2 * 2.07e9 / 1e12
 # Algorithmic HBM bytes of one heat apply: read u, write v, read the nodal T^n (3 words per DoF).
 HEAT_WORDS_PER_DOF = 3
@@ -141,7 +139,7 @@ class ClockSampler:
 
 
 KERNEL_SOURCES = ("apply_f64.cu", "apply_f32.cu", "apply_df64.cu", "apply_df64_uniform.cu", "df_pairs.cuh",
-                  "apply_kernels.cuh", "cellops.cuh", "scalar_local.cuh", "df64.cuh")
+                  "apply_kernels.cuh", "cellops.cuh", "scalar_local.cuh", "lines.cuh", "df64.cuh")
 
 
 def kernel_hash():

@@ -49,12 +49,11 @@ typedef int mf_status;
 
 /* MF_DF64: fp64 vectors, cell arithmetic in double-float (pairs of fp32 with error-free
  * products and sums, 47-48-bit significand) on the fp32 pipes, which GB300 runs at 64x its fp64
- * rate; accurate to a few 1e-14 relative to |A||u| componentwise.  On uniform meshes (Helmholtz,
- * heat without convection or Gauss-point rho_cp, Oseen without the melt-pool terms) the inputs are
- * scaled by a power of two per warp of 32 cells (Oseen: velocity and pressure separately), so any
- * fp64 magnitude keeps 47 bits relative to the largest input of those cells and inputs more than
- * 2^126 below it count as zero; the other operators keep the fp32 exponent range (magnitudes
- * between about 1e-38 and 3e38). */
+ * rate; accurate to a few 1e-14 relative to |A||u| componentwise.  Helmholtz, heat and Oseen on
+ * uniform meshes and reinitialisation on octrees scale the inputs by a power of two per warp of 32
+ * cells (Oseen: velocity and pressure separately), so any fp64 magnitude keeps 47 bits relative to
+ * the largest input of those cells and inputs more than 2^126 below it count as zero; the other
+ * operators keep the fp32 exponent range (magnitudes between about 1e-38 and 3e38). */
 typedef enum { MF_F64 = 0, MF_F32 = 1, MF_F16 = 2, MF_BF16 = 3, MF_DF64 = 4 } mf_dtype;
 /* mf_solver_params.inner_arith value beside the dtypes: fp32 inner applies on the tensor cores */
 enum { MF_INNER_TENSOR_CORES = 16 };
@@ -272,7 +271,9 @@ typedef struct {
                           device, eight per replay when n * nrhs <= 2^20 and one otherwise (a
                           system that has stopped is left untouched by the remaining steps; the
                           reported iterations are the steps it took), and each call of
-                          MF_PREC_BLOCK_TRIANGULAR (recorded at its second call) */
+                          MF_PREC_BLOCK_TRIANGULAR (recorded at its second call).  Single fp64
+                          systems with MF_PREC_JACOBI on the "q2_line" kernel run all CG steps in
+                          one launch, with or without it */
   double tol;          /* stop when ||b - A x||_2 <= tol ||b||_2 (x0 = 0) */
   double inner_tol;    /* defect correction: inner relative tolerance */
   double cheby_ratio;  /* Chebyshev interval [lambda_max/ratio, 1.1 lambda_max] */
@@ -397,7 +398,8 @@ mf_status mf_heat_step_gradient(mf_op* op, const mf_laser* laser, const mf_solve
  * right-hand sides for octree maps and on one for uniform ones; coefficient mode; one or nine threads
  * per cell for uniform Q2 Helmholtz and heat; fp64 pipes or double-float; Oseen: the fp64 loop order;
  * Q3 Helmholtz: the CUDA-core or the tensor-core kernel for fp32 applies, which then also serves the
- * fp32 applies inside solvers) and keep the fastest.  cache_path (may be NULL) is a
+ * fp32 applies inside solvers) and keep the fastest.  The tables of the fp32 applies are built here too,
+ * instead of at the first such apply.  cache_path (may be NULL) is a
  * text file of one JSON record per line, keyed by the operator's configuration (kind, degree, mesh
  * type and sizes, optional fields, melt-pool flags, the device's SM count): if it holds a record with
  * this operator's key, the last such record's choice is applied and nothing is timed; otherwise the
