@@ -130,6 +130,7 @@ mf_status launch_q2_line(mf_ctx* ctx, const mf_dofmap* m, const T* src, T* dst, 
 mf_status launch_q2_line_cg(mf_ctx* ctx, const mf_dofmap* m, const double* coef, double mass, const double* dinv, double* x,
                             double* r, double* z, double* p, double* p2, double* Ap, double tol, int maxit,
                             bool stop_indefinite, double* S, double* steps);
+int64_t q2_line_cg_cells(const mf_ctx* ctx);   // up to this many cells it is the faster way to solve
 mf_status launch_qk_diag(mf_ctx* ctx, const mf_dofmap* m, const double* coef, double mass, double* diag);
 // Q3 Helmholtz on the tensor cores (fp32 vectors, dst accumulated; coef per tile of 128 cells,
 // [tile][q][row], from launch_tc_coef_layout).  A launch returns MF_ETIMEOUT when an earlier one

@@ -330,6 +330,12 @@ mf_status launch_q2_line(mf_ctx* ctx, const mf_dofmap* m, const T* src, T* dst, 
 template mf_status launch_q2_line<double>(mf_ctx*, const mf_dofmap*, const double*, double*, const double*, double);
 template mf_status launch_q2_line<float>(mf_ctx*, const mf_dofmap*, const float*, float*, const float*, double);
 
+// Five rounds of the grid: with more cells per group of threads the eight warps per SM that the barriers
+// allow cost more than the launches of the separate kernels.  One launch against those kernels replayed as
+// a graph, ms per Helmholtz solve: 20^3 cells 8.5 / 11.9, 28^3 27.2 / 27.4, 32^3 39.5 / 38.3, 36^3 58.7 / 54.6,
+// 44^3 130 / 108.
+int64_t q2_line_cg_cells(const mf_ctx* ctx) { return int64_t(5) * kCgCells * ctx->sm_count; }
+
 mf_status launch_q2_line_cg(mf_ctx* ctx, const mf_dofmap* m, const double* coef, double mass, const double* dinv, double* x,
                             double* r, double* z, double* p, double* p2, double* Ap, double tol, int maxit,
                             bool stop_indefinite, double* S, double* steps) {

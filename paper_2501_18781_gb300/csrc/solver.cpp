@@ -582,7 +582,7 @@ template <typename T> struct CG {
   bool whole_solve_kernel() const {
     const int kind = scalar_kind(op);
     return sizeof(T) == 8 && nrhs == 1 && P->kind == MF_PREC_JACOBI && op->q2_line64 && op->f64_prec == PREC_F64 &&
-           op->n <= kSmallSystem && op->map[0]->uniform && op->map[0]->degree == 2 &&
+           op->ncells <= q2_line_cg_cells(op->ctx) && op->map[0]->uniform && op->map[0]->degree == 2 &&
            (kind == K_HELM || kind == K_HEAT) && !heat_convection(op) && !op->rhocp_user;
   }
 
