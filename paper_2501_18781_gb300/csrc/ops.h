@@ -175,10 +175,11 @@ mf_status launch_oseen_f32_tables(mf_ctx* ctx, const mf_dofmap* mu, const double
                                   const double* cb64, const double* nr64, float* cm, float* cv, float* cb, float* nr);
 mf_status launch_oseen_f32_uniform(mf_ctx* ctx, const mf_dofmap* mu, const float* src, float* dst, const float* cm,
                                    const float* cv, const float* cb, const float* nr);
-// double-float Oseen apply on uniform meshes: the folded coefficient tables cm, cv (27 per cell) and
-// cb (81 per cell) as float pairs from launch_oseen_df_split; nr: the melt-pool interface normal table
-// (81 per cell, pairs) for the trace correction, or NULL without the melt-pool terms
+// s c as float pairs, n values
 mf_status launch_split_pairs(mf_ctx* ctx, const double* c, int64_t n, double scale, float2* out);
+// double-float Oseen apply on uniform meshes: the folded coefficient tables cm, cv (27 per cell), cb (81 per
+// cell) and the melt-pool interface normal nr (81 per cell, for the trace correction; or NULL) as float
+// pairs per tile of 32 cells, from launch_oseen_df_split (tile_table_floats pairs each)
 mf_status launch_oseen_df_split(mf_ctx* ctx, const mf_dofmap* mu, const double* cm64, const double* cv64,
                                 const double* cb64, const double* nr64, float2* cm, float2* cv, float2* cb, float2* nr);
 mf_status launch_oseen_df_uniform(mf_ctx* ctx, const mf_dofmap* mu, const double* src, double* dst, const float2* cm,
@@ -230,8 +231,8 @@ struct mf_op {
   bool rhs_ready = false;
   float* rhs_work = nullptr;           // its work vectors while a solve lends them, else per call
   int64_t rhs_work_floats = 0;
-  mf::DevBuf cm_df, cv_df, cb_df;   // Oseen: folded coefficients as float pairs (high, then low parts)
-  mf::DevBuf nrm_df;                // Oseen melt-pool terms: the interface normal table as float pairs
+  mf::DevBuf cm_df, cv_df, cb_df;   // Oseen: folded coefficients as float pairs per tile of 32 cells
+  mf::DevBuf nrm_df;                // Oseen melt-pool terms: the interface normal, likewise
   bool diag_ready = false;
   // Chebyshev bounds: lambda_max of D^-1 A from the first solve's Lanczos run, kept until a field
   // changes (the same number of steps from the same start vector gives the same estimate)
