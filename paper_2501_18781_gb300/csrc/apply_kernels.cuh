@@ -108,7 +108,8 @@ __device__ __forceinline__ void scalar_cell(const ScalarArgs<typename Store<T>::
     T U[27], R[27];
     if (compute) {
       gather<T, OCT, KIND != K_MASS>(ug, og, L, A.src + r * A.ld, U);
-      scalar_local<T, KIND, MODE, BETA, TR>(A, L.cell, h, mh2, C, U, R);
+      scalar_local<T, KIND, MODE, BETA, TR, KIND == K_REINIT && (MODE == 0 || (OCT && sizeof(T) == 4))>(A, L.cell, h, mh2, C,
+                                                                                                        U, R);
     } else {
 #pragma unroll
       for (int q = 0; q < 27; ++q) R[q] = T(0);
@@ -120,12 +121,13 @@ __device__ __forceinline__ void scalar_cell(const ScalarArgs<typename Store<T>::
 
 // One launch sweeps all nwork work units; with fewer blocks than units (the persistent
 // variant, grid = a few blocks per SM) each block strides over them.  All right-hand sides of
-// a cell are applied while its coefficients sit in registers.  Two fp32 instances are held to four
-// blocks of 128 per SM: the octree reinitialisation, whose indirect gathers are latency-bound, and the
-// uniform heat operator without convection (five blocks spill in the difference form).
+// a cell are applied while its coefficients sit in registers.  The fp32 octree reinitialisation,
+// whose indirect gathers are latency-bound, works point by point (scalar_local) and is held to five blocks of
+// 128 per SM (four with the normals formed in the kernel); in difference form it spills from four on.  The fp32 uniform heat operator without
+// convection is held to four (five spill).
 template <typename T, int KIND, int MODE, bool BETA, bool TR, bool OCT>
-__global__ void __launch_bounds__(128, (sizeof(T) == 4 && ((OCT && KIND == K_REINIT) ||
-                                                           (!OCT && KIND == K_HEAT && !BETA))) ? 4 : 1)
+__global__ void __launch_bounds__(128, (sizeof(T) == 4 && OCT && KIND == K_REINIT) ? 4 + MODE :
+                                          (sizeof(T) == 4 && !OCT && KIND == K_HEAT && !BETA) ? 4 : 1)
     k_scalar(ScalarArgs<typename Store<T>::type> A, UniformGeom ug, OctGeom og,
                                                 int64_t nwork) {
   for (int64_t w = blockIdx.x; w < nwork; w += gridDim.x) {

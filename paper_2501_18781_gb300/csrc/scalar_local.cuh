@@ -27,7 +27,8 @@ template <typename T> __device__ __forceinline__ T heaviside(T phi, int kind, T 
 
 // U: nodal values of the cell (overwritten); R: the cell's contribution, at the nodes.
 // C: scalar coefficient at the Gauss points (in-kernel phi for MODE 0 reinit).
-template <typename T, int KIND, int MODE, bool BETA, bool TR>
+// POINTS: reinitialisation point by point, which holds two arrays of 27 values instead of three.
+template <typename T, int KIND, int MODE, bool BETA, bool TR, bool POINTS = (KIND == K_REINIT && MODE == 0)>
 __device__ __forceinline__ void scalar_local(const ScalarArgs<typename Store<T>::type>& A, int64_t cell, T h, T mh2,
                                              const T* C, T* U, T* R) {
   const T eps = T(A.eps);
@@ -45,8 +46,8 @@ __device__ __forceinline__ void scalar_local(const ScalarArgs<typename Store<T>:
       line(d, n, p0, p1, p2);
       line_values(U[p0], U[p1], U[p2]);
     }
-  if constexpr (KIND == K_REINIT && MODE == 0) {
-    // the normal of every point from the level set's gradient there: point by point
+  if constexpr (POINTS) {
+    // the normal of every point from the table, or from the level set's gradient there
 #pragma unroll
     for (int q = 0; q < 27; ++q) R[q] = T(0);
 #pragma unroll
@@ -55,10 +56,16 @@ __device__ __forceinline__ void scalar_local(const ScalarArgs<typename Store<T>:
       const T w = Tb<T>::W3(q);
       T gx, gy, gz, nx, ny, nz;
       grad_at<T>(U, qa, qb, qc, gx, gy, gz);
-      grad_at<T>(C, qa, qb, qc, nx, ny, nz);
-      const T nn = sqrt(nx * nx + ny * ny + nz * nz);
-      const T inv = nn < T(1e-12) ? T(0) : T(1) / nn;
-      nx *= inv; ny *= inv; nz *= inv;
+      if constexpr (MODE == 0) {
+        grad_at<T>(C, qa, qb, qc, nx, ny, nz);
+        const T nn = sqrt(nx * nx + ny * ny + nz * nz);
+        const T inv = nn < T(1e-12) ? T(0) : T(1) / nn;
+        nx *= inv; ny *= inv; nz *= inv;
+      } else {
+        nx = from_store<T>(__ldg(A.qvec + q * A.ncp + cell));
+        ny = from_store<T>(__ldg(A.qvec + (27 + q) * A.ncp + cell));
+        nz = from_store<T>(__ldg(A.qvec + (54 + q) * A.ncp + cell));
+      }
       const T s = w * (eps * (nx * gx + ny * gy + nz * gz));
       R[q] += w * (mh2 * U[q]);
       add_grad_test<T>(R, qa, qb, qc, s * nx, s * ny, s * nz);
