@@ -61,6 +61,7 @@ __global__ void __launch_bounds__(kOctThreads, 4) k_reinit_df_octree(const __gri
   const int32_t* __restrict__ map = og.cmap + cell;
   const int64_t nc = A.ncells;
   int bias = 0;
+  bool bad;   // an Inf or NaN among the cell's inputs
   {
     double X[27];
     uint32_t hanging = 0;
@@ -102,7 +103,7 @@ __global__ void __launch_bounds__(kOctThreads, 4) k_reinit_df_octree(const __gri
       emax = max(emax, unsigned(__double2hiint(v)) & 0x7FF00000u);
     }
     __syncwarp();
-    emax = __reduce_max_sync(0xffffffffu, emax) >> 20;
+    emax = finite_exponent(__reduce_max_sync(0xffffffffu, emax) >> 20, sU, kOctThreads, 27, bad);
     bias = emax ? int(emax) - 1023 : 0;
   }
 #pragma unroll 1
@@ -207,6 +208,7 @@ __global__ void __launch_bounds__(kOctThreads, 4) k_reinit_df_octree(const __gri
   }
   if (!active) return;
   double* __restrict__ dst = A.dst + rhs * A.ld;
+  const Scale scale(bias);
 #pragma unroll 1
   for (int c = 0; c < 3; ++c) {
     dd R[9];
@@ -225,10 +227,15 @@ __global__ void __launch_bounds__(kOctThreads, 4) k_reinit_df_octree(const __gri
     }
 #pragma unroll
     for (int b = 0; b < 3; ++b) dd_line_values_t(R[3 * b], R[3 * b + 1], R[3 * b + 2]);
+    if (scale.far) {
+#pragma unroll
+      for (int p = 0; p < 9; ++p) st2(sU + (9 * c + p) * kOctThreads, R[p]);
+      continue;
+    }
     uint32_t hanging = 0;
 #pragma unroll
     for (int p = 0; p < 9; ++p) {
-      const double v = f2d_bits(R[p].h, bias) + f2d_bits(R[p].l, bias);
+      const double v = scale.join(R[p]);
       if (id[p] >= 0) {
         if (!(og.dflag && __ldg(og.dflag + id[p]))) atomicAdd(dst + id[p], v);
       } else {
@@ -240,6 +247,22 @@ __global__ void __launch_bounds__(kOctThreads, 4) k_reinit_df_octree(const __gri
       const int p = __ffs(hanging) - 1;
       const double v = *reinterpret_cast<double*>(sU + (9 * c + p) * kOctThreads);
       const int r = -1 - __ldg(map + (9 * c + p) * og.ncp);
+      for (int e = __ldg(og.rowptr + r); e < __ldg(og.rowptr + r + 1); ++e) {
+        const int32_t m = __ldg(og.cols + e);
+        if (!(og.dflag && __ldg(og.dflag + m))) atomicAdd(dst + m, __ldg(og.w64 + e) * v);
+      }
+    }
+  }
+  if (bad || scale.far) {   // a NaN into every row of the cell; the test side of a warp with such a scale
+#pragma unroll 1
+    for (int l = 0; l < 27; ++l) {
+      const double v = bad ? __hiloint2double(0x7FF80000, 0) : scale.join_far(ld2(sU + l * kOctThreads));
+      const int32_t id = __ldg(map + l * og.ncp);
+      if (id >= 0) {
+        if (!(og.dflag && __ldg(og.dflag + id))) atomicAdd(dst + id, v);
+        continue;
+      }
+      const int r = -1 - id;
       for (int e = __ldg(og.rowptr + r); e < __ldg(og.rowptr + r + 1); ++e) {
         const int32_t m = __ldg(og.cols + e);
         if (!(og.dflag && __ldg(og.dflag + m))) atomicAdd(dst + m, __ldg(og.w64 + e) * v);

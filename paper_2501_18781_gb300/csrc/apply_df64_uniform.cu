@@ -11,7 +11,8 @@
 // to a few 1e-14 of |A||u| componentwise.  Doubles enter and leave the kernel by bit manipulation
 // (GB300 converts between fp64 and fp32 only at its fp64 rate), scaled by one power of two per warp so
 // that the warp's largest input lies in [1, 2): any fp64 magnitude is kept to 47 bits relative to that
-// largest input of the warp's 8 x 4 cells; inputs more than 2^126 below it count as zero.
+// largest finite input of the warp's 8 x 4 cells; inputs more than 2^126 below it count as zero, and the rows
+// of a cell with an Inf or NaN among its inputs get a NaN.
 //
 // One thread per cell in 8 x 4 x 4 bricks; the cell's values and test side live in the thread's own
 // columns of shared memory and every phase is a short rolled loop over them.  No thread of the scalar
@@ -44,10 +45,10 @@ __device__ __forceinline__ dd shfl_down_dd(dd v, int d) {
 
 // Scatter-add of one slab z = const of 9 nodes per cell of a warp of the 8 x 4 x 4 brick (dst at the
 // slab's first node): the faces shared by x and y neighbours inside the warp are folded by shuffles on
-// the pairs (all lanes share one scale), then every node is added to memory once per warp as the
-// double hi 2^bias + lo 2^bias.  Every lane calls this; inactive lanes pass zeros.
+// the pairs (all lanes share one scale), then every node is added to memory once per warp as a double (scale.far:
+// not for this path).  Every lane calls this; inactive lanes pass zeros.
 __device__ __forceinline__ void scatter_dd_slab(double* __restrict__ dst, int64_t sx, uint32_t dmask, dd* R, bool active,
-                                                int bias) {
+                                                const Scale& scale) {
   const int xl = threadIdx.x & 7, yl = (threadIdx.x >> 3) & 3;
 #pragma unroll
   for (int b = 0; b < 3; ++b) {
@@ -66,7 +67,20 @@ __device__ __forceinline__ void scatter_dd_slab(double* __restrict__ dst, int64_
   for (int l = 0; l < 9; ++l) {
     const int a = l % 3, b = l / 3;
     if ((a == 0 && xl > 0) || (b == 0 && yl > 0) || ((dmask >> l) & 1u)) continue;
-    atomicAdd(dst + a + sx * b, f2d_bits(R[l].h, bias) + f2d_bits(R[l].l, bias));
+    atomicAdd(dst + a + sx * b, scale.join(R[l]));
+  }
+}
+// What scatter_dd_slab leaves: the test side of a cell of a warp whose scale is far (col, slots STRIDE apart; dst
+// at the cell's first node), and a NaN into every row of a cell with an Inf or NaN among its inputs.
+template <int STRIDE>
+__device__ __forceinline__ void scatter_rare(double* __restrict__ dst, int64_t sx, int64_t sy, uint32_t dmask,
+                                             const float2* col, const Scale& scale, bool bad) {
+#pragma unroll 1
+  for (int l = 0; l < 27; ++l) {
+    const float2 v = col[l * STRIDE];
+    if (!((dmask >> l) & 1u))
+      atomicAdd(dst + l % 3 + sx * ((l / 3) % 3) + sy * (l / 9),
+                bad ? __hiloint2double(0x7FF80000, 0) : scale.join_far(dd{v.x, v.y}));
   }
 }
 
@@ -110,6 +124,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_scalar_df_uniform(const __grid_
     for (int q = lx; q < 27; q += 8) asm volatile("prefetch.global.L2 [%0];" ::"l"(p + q * nc));
   }
   int bias = 0;
+  bool bad;   // an Inf or NaN among the cell's inputs
   {
     // gather (Dirichlet nodes and lanes without a cell read as 0); right-hand side blockIdx.y
     const double* __restrict__ s = A.src + int64_t(blockIdx.y) * A.ld + base;
@@ -130,10 +145,10 @@ __global__ void __launch_bounds__(kThreads, 4) k_scalar_df_uniform(const __grid_
     unsigned emax = 0;
 #pragma unroll
     for (int l = 0; l < 27; ++l) emax = max(emax, unsigned(__double2hiint(X[l])) & 0x7FF00000u);
-    emax = __reduce_max_sync(0xffffffffu, emax) >> 20;
-    bias = emax ? int(emax) - 1023 : 0;
 #pragma unroll
     for (int l = 0; l < 27; ++l) *reinterpret_cast<double*>(sU + l * kThreads) = X[l];
+    emax = finite_exponent(__reduce_max_sync(0xffffffffu, emax) >> 20, sU, kThreads, 27, bad);
+    bias = emax ? int(emax) - 1023 : 0;
   }
 #pragma unroll 1
   for (float2* p = sU; p < sU + 27 * kThreads; p += 3 * kThreads) {
@@ -237,6 +252,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_scalar_df_uniform(const __grid_
     for (int c = 0; c < 3; ++c) st2(sV + (p + 9 * c) * kThreads, V[c]);
   }
   double* __restrict__ d = A.dst + int64_t(blockIdx.y) * A.ld + base;
+  const Scale scale(bias);
 #pragma unroll 1
   for (int c = 0; c < 3; ++c) {
     dd R[9];
@@ -255,8 +271,14 @@ __global__ void __launch_bounds__(kThreads, 4) k_scalar_df_uniform(const __grid_
 #pragma unroll
       for (int p = 0; p < 9; ++p) R[p] = dd{0.f, 0.f};
     }
-    scatter_dd_slab(d + ug.sy * c, ug.sx, (dmask >> (9 * c)) & 0x1FFu, R, active, bias);
+    if (scale.far) {
+#pragma unroll
+      for (int p = 0; p < 9; ++p) st2(sV + (9 * c + p) * kThreads, R[p]);
+    } else {
+      scatter_dd_slab(d + ug.sy * c, ug.sx, (dmask >> (9 * c)) & 0x1FFu, R, active, scale);
+    }
   }
+  if (active && (scale.far || bad)) scatter_rare<kThreads>(d, ug.sx, ug.sy, dmask, sV, scale, bad);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -308,6 +330,7 @@ template <bool EXT>
 __global__ void __launch_bounds__(96, 4) k_oseen_df_uniform(const __grid_constant__ DfOseenArgs A, UniformGeom ug) {
   extern __shared__ float2 df_smem[];
   __shared__ int sE[3];
+  __shared__ unsigned sBad[3];   // cells with an Inf or NaN among the component's inputs
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   float2* const sU = df_smem + lane;                    // component e, point q at sU[(27 e + q) * 32]
   float2* const sV = df_smem + 81 * 32 + w * 27 * 32 + lane;
@@ -370,14 +393,30 @@ __global__ void __launch_bounds__(96, 4) k_oseen_df_uniform(const __grid_constan
       *reinterpret_cast<double*>(sU + (27 * w + l) * 32) = X[l];
     }
   }
-  eu = __reduce_max_sync(0xffffffffu, eu) >> 20;
+  bool bad_u, bad_p = false;
+  eu = finite_exponent(__reduce_max_sync(0xffffffffu, eu) >> 20, sU + 27 * w * 32, 32, 27, bad_u);
   ep = __reduce_max_sync(0xffffffffu, ep) >> 20;   // the same cells in every warp
-  if (lane == 0) sE[w] = int(eu);
+  if (ep == 0x7FFu) {
+    ep = 0;
+#pragma unroll
+    for (int n = 0; n < 8; ++n) {
+      const unsigned e = unsigned(__double2hiint(Pn[n])) & 0x7FF00000u;
+      if (e == 0x7FF00000u) bad_p = true;
+      else ep = max(ep, e);
+    }
+    ep = __reduce_max_sync(0xffffffffu, ep) >> 20;
+  }
+  const unsigned bad_cells = __ballot_sync(0xffffffffu, bad_u);
+  if (lane == 0) {
+    sE[w] = int(eu);
+    sBad[w] = bad_cells;
+  }
   __syncthreads();
   const int em = max(sE[0], max(sE[1], sE[2]));
   const int bias_u = em ? em - 1023 : 0, bias_p = ep ? int(ep) - 1023 : 0;
   const int bias_out = max(bias_u, bias_p);
   const float su = pow2f(bias_u - bias_out);   // velocity terms into the output scale
+  const bool bad = ((sBad[0] | sBad[1] | sBad[2]) >> lane) & 1u;
   {
     float2* const p0 = sU + 27 * w * 32;
 #pragma unroll 1
@@ -552,11 +591,21 @@ __global__ void __launch_bounds__(96, 4) k_oseen_df_uniform(const __grid_constan
     const dd mh2{A.mh2.x, A.mh2.y};
     const int64_t pa = w == 0 ? 1 : (w == 1 ? px : pxy), pb = w == 1 ? 1 : px, pc = w == 2 ? 1 : pxy;
     double* const pd = A.dst + 3 * A.nu + pbase;
+    const Scale scale_u(bias_u);
 #pragma unroll
-    for (int n = 0; n < 8; ++n) {
-      const dd r = dd_mul(mh2, dd_norm(Rp[n]));
-      atomicAdd(pd + (n & 1) * pa + ((n >> 1) & 1) * pb + (n >> 2) * pc, f2d_bits(r.h, bias_u) + f2d_bits(r.l, bias_u));
+    for (int n = 0; n < 8; ++n) Rp[n] = dd_mul(mh2, dd_norm(Rp[n]));
+    if (scale_u.far) {
+#pragma unroll
+      for (int n = 0; n < 8; ++n)
+        atomicAdd(pd + (n & 1) * pa + ((n >> 1) & 1) * pb + (n >> 2) * pc, scale_u.join_far(Rp[n]));
+    } else {
+#pragma unroll
+      for (int n = 0; n < 8; ++n) atomicAdd(pd + (n & 1) * pa + ((n >> 1) & 1) * pb + (n >> 2) * pc, scale_u.join(Rp[n]));
     }
+    if (bad)
+#pragma unroll 1
+      for (int n = 0; n < 8; ++n)
+        atomicAdd(pd + (n & 1) * pa + ((n >> 1) & 1) * pb + (n >> 2) * pc, __hiloint2double(0x7FF80000, 0));
   }
   // planes (a, c): flux along c, transposes along c and a
 #pragma unroll 1
@@ -594,6 +643,7 @@ __global__ void __launch_bounds__(96, 4) k_oseen_df_uniform(const __grid_constan
     }
   }
   double* __restrict__ d = A.dst + w * A.nu + base;
+  const Scale scale(bias_out);
 #pragma unroll 1
   for (int c = 0; c < 3; ++c) {
     dd R[9];
@@ -610,8 +660,15 @@ __global__ void __launch_bounds__(96, 4) k_oseen_df_uniform(const __grid_constan
 #pragma unroll
       for (int p = 0; p < 9; ++p) R[p] = dd{0.f, 0.f};
     }
-    scatter_dd_slab(d + ug.sy * c, ug.sx, (dmask >> (9 * c)) & 0x1FFu, R, active, bias_out);
+    if (__builtin_expect(scale.far, 0)) {
+#pragma unroll
+      for (int p = 0; p < 9; ++p) st2(sV + (9 * c + p) * 32, R[p]);
+    } else {
+      scatter_dd_slab(d + ug.sy * c, ug.sx, (dmask >> (9 * c)) & 0x1FFu, R, active, scale);
+    }
   }
+  if (__builtin_expect(active && (scale.far || bad || bad_p), 0))
+    scatter_rare<32>(d, ug.sx, ug.sy, dmask, sV, scale, bad || bad_p);
 }
 
 // s c as float pairs
