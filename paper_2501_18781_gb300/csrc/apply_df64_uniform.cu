@@ -413,7 +413,9 @@ __global__ void __launch_bounds__(96, 4) k_oseen_df_uniform(const __grid_constan
   }
   __syncthreads();
   const int em = max(sE[0], max(sE[1], sE[2]));
-  const int bias_u = em ? em - 1023 : 0, bias_p = ep ? int(ep) - 1023 : 0;
+  // (a field that is zero in the whole block takes the other's scale: with 2^0 it would hide small values)
+  const int exp_u = em ? em : int(ep), exp_p = ep ? int(ep) : em;
+  const int bias_u = exp_u ? exp_u - 1023 : 0, bias_p = exp_p ? exp_p - 1023 : 0;
   const int bias_out = max(bias_u, bias_p);
   const float su = pow2f(bias_u - bias_out);   // velocity terms into the output scale
   const bool bad = ((sBad[0] | sBad[1] | sBad[2]) >> lane) & 1u;
