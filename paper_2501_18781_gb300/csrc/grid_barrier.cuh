@@ -63,22 +63,30 @@ __device__ __forceinline__ void grid_totals(const double* part, int n, unsigned 
   __syncthreads();
 }
 
-// Block sums of N values, value k to part[k * stride + blockIdx.x].  Pairs of floats down to one value per
-// warp: fp64 adds cost 16 cycles of the SM per warp instruction (a tree of them over the block's 32 warps
-// took longer than the step's stencil).
-template <int N> __device__ __forceinline__ void block_partials(Dot2f (&v)[N], double (*sh)[32], double* part, int64_t stride) {
+// Block sums of N values of the first ROWS threads, value k to part[k * stride + blockIdx.x]: one warp per value
+// adds ROWS / 32 pairs per lane exactly, then in fp64.  (fp64 adds cost 16 cycles of the SM per warp
+// instruction: a tree of them over the block's 32 warps took longer than the step's stencil.)
+template <int N, int ROWS>
+__device__ __forceinline__ void block_partials(const Dot2f (&v)[N], float2 (*sh)[ROWS], double* part, int64_t stride) {
+  if (threadIdx.x < ROWS)
 #pragma unroll
-  for (int k = 0; k < N; ++k) v[k].warp_sum();
-  if ((threadIdx.x & 31) == 0)
-#pragma unroll
-    for (int k = 0; k < N; ++k) sh[k][threadIdx.x >> 5] = v[k].value();
+    for (int k = 0; k < N; ++k) sh[k][threadIdx.x] = make_float2(v[k].s, v[k].c);
   __syncthreads();
   if (threadIdx.x < 32 * N) {
-    const int k = threadIdx.x >> 5;
-    double s = sh[k][threadIdx.x & 31];
+    const int k = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    double s = 0.0;
+#pragma unroll 1
+    for (int j = lane; j < ROWS; j += 256)
+      s += exact_sum<8>([&](int i) {
+        const float2 p = sh[k][j + 32 * i];
+        Dot2f a;
+        a.s = p.x;
+        a.c = p.y;
+        return a;
+      });
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-    if ((threadIdx.x & 31) == 0) part[k * stride + blockIdx.x] = s;
+    if (lane == 0) part[k * stride + blockIdx.x] = s;
   }
 }
 

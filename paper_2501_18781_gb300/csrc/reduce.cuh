@@ -7,11 +7,10 @@
 namespace mf {
 namespace {
 
-// Sums over a block of kRedThreads threads.  GB300's fp64 pipe takes 16 cycles of an SM per warp
+// Sums over a block of kRedThreads threads, in fp64.  GB300's fp64 pipe takes 16 cycles of an SM per warp
 // instruction, so a shuffle tree over every warp (five adds each) costs more than the data of a small
 // vector: the threads' values go to shared memory, and one warp per value adds eight of them per lane
-// before its shuffles (13 fp64 adds instead of 43; a 257 k element fp32 dot 14.7 -> 8.8 us with the grid cut
-// to the vector and 16-byte loads, the fp32 multidot of 5 vectors of 1.6 M 19.9 -> 12.1 us).  N values share the barrier; value k is summed by warp
+// before its shuffles (13 fp64 adds instead of 43).  N values share the barrier; value k is summed by warp
 // k in a fixed order and given to put(k, sum) by its first lane.  Every thread of the block calls this.
 __device__ __forceinline__ double (*red_area1())[kRedThreads] {   // one area for every instance in a kernel
   __shared__ double sh[1][kRedThreads];
@@ -63,38 +62,74 @@ struct Dot2f {
     c += ((s - (t - z)) + (p - z)) + e;
     s = t;
   }
-  // the sum of both pairs
-  __device__ __forceinline__ void merge(float os, float oc) {
-    const float t = s + os;
-    const float z = t - s;
-    c += oc + ((s - (t - z)) + (os - z));
-    s = t;
-  }
-  __device__ __forceinline__ void merge(const Dot2f& o) { merge(o.s, o.c); }
-  // lane 0: the sum over the warp (pairs of floats: no fp64 instruction)
-  __device__ __forceinline__ void warp_sum() {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1)
-      merge(__shfl_down_sync(0xffffffffu, s, o), __shfl_down_sync(0xffffffffu, c, o));
-  }
   __device__ __forceinline__ double value() const { return double(s) + double(c); }
 };
 
-// The same for pairs: summed over each warp as pairs, then the warps' sums in fp64.
-template <int N, typename F> __device__ __forceinline__ void block_sums(Dot2f (&v)[N], F&& put) {
+// A sum of pairs, exact beyond fp64: the high parts and then the low parts are added without error, what both
+// leave goes to a third float (72 bits).  Adding pairs as pairs loses bits against fp64 (sums of squares of
+// 4,096 to 1.6 M elements: 9e-16 of the sum; this way, as with every pair converted, 2e-16), and converting every
+// pair costs three fp64 instructions.  A sum past the largest float is an fp64 number: s is then Inf and c, l are
+// its bits.
+struct Sum3f {
+  float s = 0.f, c = 0.f, l = 0.f;
+  __device__ __forceinline__ void add(const Dot2f& a) { add(a.s, a.c, 0.f); }
+  __device__ __forceinline__ void add(const Sum3f& a) { add(a.s, a.c, a.l); }
+  __device__ __forceinline__ void add(float os, float oc, float ol) {
+    const float t = s + os, z = t - s, d = (s - (t - z)) + (os - z);
+    const float u = c + oc, y = u - c, e = (c - (u - y)) + (oc - y);
+    const float v = u + d, x = v - u, f = (u - (v - x)) + (d - x);
+    s = t;
+    c = v;
+    l = (l + ol) + (e + f);
+  }
+  __device__ __forceinline__ bool in_range() const { return fabsf(s) <= 3.402823466e38f; }
+  __device__ __forceinline__ double value() const {
+    return in_range() ? double(s) + (double(c) + double(l)) : __hiloint2double(__float_as_int(c), __float_as_int(l));
+  }
+};
+// fp64 sum of the N pairs or triples that load(0 .. N - 1) gives
+template <int N, typename L> __device__ __forceinline__ double exact_sum(L&& load) {
+  Sum3f t;
+#pragma unroll
+  for (int k = 0; k < N; ++k) t.add(load(k));
+  if (t.in_range()) return t.value();
+  double v = 0.0;
+#pragma unroll 1
+  for (int k = 0; k < N; ++k) v += load(k).value();
+  return v;
+}
+// a thread's N accumulators in one
+template <int N, typename A> __device__ __forceinline__ Sum3f thread_sum(const A (&a)[N]) {
+  Sum3f t;
+#pragma unroll
+  for (int k = 0; k < N; ++k) t.add(a[k]);
+  if (!t.in_range()) {
+    double v = 0.0;
+#pragma unroll
+    for (int k = 0; k < N; ++k) v += a[k].value();
+    t.s = __int_as_float(0x7F800000);
+    t.c = __int_as_float(__double2hiint(v));
+    t.l = __int_as_float(__double2loint(v));
+  }
+  return t;
+}
+// The block sums of pairs or triples: one warp per value adds eight threads' per lane exactly, then in fp64 (10 fp64
+// instructions per value).  The areas serve every instance in a kernel.
+template <typename P, int ROWS> __device__ __forceinline__ P (*exact_area())[kRedThreads] {
+  __shared__ __align__(16) char sh[ROWS * kRedThreads * sizeof(P)];
+  return reinterpret_cast<P(*)[kRedThreads]>(sh);
+}
+template <int N, typename P, typename F> __device__ __forceinline__ void block_sums_exact(const P (&v)[N], F&& put) {
   static_assert(N <= kRedThreads / 32, "one warp per value");
-  __shared__ double sh[N][kRedThreads / 32];
+  P(*sh)[kRedThreads] = N <= 2 ? exact_area<P, 2>() : exact_area<P, kRedThreads / 32>();
 #pragma unroll
-  for (int k = 0; k < N; ++k) v[k].warp_sum();
-  if ((threadIdx.x & 31) == 0)
-#pragma unroll
-    for (int k = 0; k < N; ++k) sh[k][threadIdx.x >> 5] = v[k].value();
+  for (int k = 0; k < N; ++k) sh[k][threadIdx.x] = v[k];
   __syncthreads();
   if (threadIdx.x < 32 * N) {
     const int k = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    double s = lane < kRedThreads / 32 ? sh[k][lane] : 0.0;
+    double s = exact_sum<kRedThreads / 32>([&](int j) { return sh[k][lane + 32 * j]; });
 #pragma unroll
-    for (int o = kRedThreads / 64; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
     if (lane == 0) put(k, s);
   }
   __syncthreads();

@@ -81,7 +81,8 @@ __device__ __forceinline__ float stencil_words(const SchurArgs& A, const uint4* 
 template <int PARTS>
 __global__ void __launch_bounds__(kThreads, 1) k_schur_cg(const SchurArgs A) {
   extern __shared__ uint4 coef[];
-  __shared__ double sh[2][32], tot[2];
+  __shared__ double tot[2];
+  __shared__ float2 sh[2][kThreads / PARTS];
   __shared__ float coef_s;   // beta, then alpha
   __shared__ bool done;
   __shared__ float ssum[PARTS > 1 ? PARTS : 1][kThreads / PARTS];
@@ -146,8 +147,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_schur_cg(const SchurArgs A) {
   double rz = 1.0, stop = 0.0;   // thread 0 of every block: fp64 divisions by one thread, not by 32 warps
   int k = 0;
   for (; k < A.maxit; ++k) {
-    Dot2f v2[2] = {arr, arz};
-    block_partials<2>(v2, sh, A.part, G);
+    const Dot2f v2[2] = {arr, arz};
+    block_partials<2, kRows>(v2, sh, A.part, G);
     if (!grid_barrier(A.bar, G, 2 * k + 1)) return;
     grid_totals(A.part, 2, G, tot);
     if (threadIdx.x == 0) {
@@ -160,7 +161,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_schur_cg(const SchurArgs A) {
     if (done) break;
     Dot2f v1[1];
     apply(k, coef_s, v1[0]);
-    block_partials<1>(v1, sh, A.part + 2 * int64_t(G), G);
+    block_partials<1, kRows>(v1, sh, A.part + 2 * int64_t(G), G);
     if (!grid_barrier(A.bar, G, 2 * k + 2)) return;
     grid_totals(A.part + 2 * int64_t(G), 1, G, tot);
     if (threadIdx.x == 0) {

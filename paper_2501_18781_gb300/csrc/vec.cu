@@ -1,6 +1,7 @@
-// Vector kernels of the Krylov solvers.  All reductions accumulate in fp64 over a fixed
-// grid of kRedBlocks blocks, then the last block to finish sums the partials in a fixed order,
-// so every dot product is deterministic.
+// Vector kernels of the Krylov solvers.  Reductions accumulate fp64 vectors in fp64 and fp32 vectors in
+// pairs of floats within a thread, and in fp64 across threads, over a grid that depends on the vector's
+// length alone (at most kRedBlocks blocks); the last block to finish, or a second launch, sums the partials in a
+// fixed order, so every dot product is deterministic.
 #include <algorithm>
 #include <mutex>
 #include <string>
@@ -27,21 +28,33 @@ template <> struct DotAcc<float> : Dot2f {};
 template <> struct DotAcc<double> {
   double s = 0.0;
   __device__ __forceinline__ void add(double a, double b) { s = fma(a, b, s); }
-  __device__ __forceinline__ void merge(const DotAcc<double>& o) { s += o.s; }
   __device__ __forceinline__ double value() const { return s; }
 };
-template <int N, typename F> __device__ __forceinline__ void block_sums(DotAcc<float> (&v)[N], F&& put) {
+// A thread's N accumulators in one, and the block sums of N such values or of N accumulators
+template <int N> __device__ __forceinline__ Sum3f acc_sum(const DotAcc<float> (&a)[N]) { return thread_sum(a); }
+template <int N> __device__ __forceinline__ double acc_sum(const DotAcc<double> (&a)[N]) {
+  double s = a[0].s;
+#pragma unroll
+  for (int k = 1; k < N; ++k) s += a[k].s;
+  return s;
+}
+template <int N, typename F> __device__ __forceinline__ void block_sums(const Sum3f (&v)[N], F&& put) {
+  block_sums_exact<N>(v, put);
+}
+template <int N, typename F> __device__ __forceinline__ void block_sums(const DotAcc<float> (&v)[N], F&& put) {
   Dot2f w[N];
 #pragma unroll
   for (int k = 0; k < N; ++k) w[k] = v[k];
-  block_sums<N>(w, put);
+  block_sums_exact<N>(w, put);
 }
-template <int N, typename F> __device__ __forceinline__ void block_sums(DotAcc<double> (&v)[N], F&& put) {
+template <int N, typename F> __device__ __forceinline__ void block_sums(const DotAcc<double> (&v)[N], F&& put) {
   double w[N];
 #pragma unroll
   for (int k = 0; k < N; ++k) w[k] = v[k].s;
   block_sums<N>(w, put);
 }
+template <typename T> struct ThreadSum { using type = double; };
+template <> struct ThreadSum<float> { using type = Sum3f; };
 
 // Per-block partial sums of x.y (and, TWO, x2.y2).  Each thread keeps an accumulator per element of a
 // 16-byte word (every vector aligned), and two words of each vector in flight; W = 1 where a vector is
@@ -57,8 +70,8 @@ __global__ void __launch_bounds__(kRedThreads) k_dot2_partial(const T* x, const 
   const int64_t st = int64_t(gridDim.x) * blockDim.x, t0 = int64_t(blockIdx.x) * blockDim.x + threadIdx.x, nw = n / W;
   const V *xw = reinterpret_cast<const V*>(x), *yw = reinterpret_cast<const V*>(y);
   const V *xw2 = reinterpret_cast<const V*>(x2), *yw2 = reinterpret_cast<const V*>(y2);
-  // words in flight per vector, and accumulators: one per element of a word, or per word of one element
-  constexpr int UN = W == 1 ? 4 : 2, NA = W == 1 ? UN : W;
+  // words in flight per vector, and accumulators: one per element of a word and (pairs) one for the remainder, or four
+  constexpr int UN = W == 1 ? 4 : 2, NA = W == 1 ? 4 : W + (sizeof(T) == 4);
   DotAcc<T> a[NA], b[NA];
   int64_t i = t0;
   for (; i + (UN - 1) * st < nw; i += UN * st) {
@@ -71,7 +84,7 @@ __global__ void __launch_bounds__(kRedThreads) k_dot2_partial(const T* x, const 
 #pragma unroll
     for (int u = 0; u < UN; ++u)
 #pragma unroll
-      for (int c = 0; c < W; ++c) a[W == 1 ? u : c].add(p[u].c[c], q[u].c[c]);
+      for (int c = 0; c < W; ++c) a[W == 1 ? u % NA : c].add(p[u].c[c], q[u].c[c]);
     if (TWO) {
 #pragma unroll
       for (int u = 0; u < UN; ++u) {
@@ -81,7 +94,7 @@ __global__ void __launch_bounds__(kRedThreads) k_dot2_partial(const T* x, const 
 #pragma unroll
       for (int u = 0; u < UN; ++u)
 #pragma unroll
-        for (int c = 0; c < W; ++c) b[W == 1 ? u : c].add(p[u].c[c], q[u].c[c]);
+        for (int c = 0; c < W; ++c) b[W == 1 ? u % NA : c].add(p[u].c[c], q[u].c[c]);
     }
   }
   for (; i < nw; i += st) {
@@ -94,20 +107,16 @@ __global__ void __launch_bounds__(kRedThreads) k_dot2_partial(const T* x, const 
       for (int c = 0; c < W; ++c) b[c].add(u0.c[c], v0.c[c]);
     }
   }
-  for (int64_t k = nw * W + t0; k < n; k += st) {   // the last n mod W elements
-    a[0].add(x[k], y[k]);
-    if (TWO) b[0].add(x2[k], y2[k]);
-  }
-#pragma unroll
-  for (int c = 1; c < NA; ++c) {
-    a[0].merge(a[c]);
-    if (TWO) b[0].merge(b[c]);
-  }
   double* const pr = part + int64_t(r) * 2 * gridDim.x + blockIdx.x;
   const int64_t g = gridDim.x;
-  DotAcc<T> v[TWO ? 2 : 1];
-  v[0] = a[0];
-  if (TWO) v[TWO ? 1 : 0] = b[0];
+  if (W > 1)   // the last n mod W elements, in accumulators of their own
+    for (int64_t k = nw * W + t0; k < n; k += st) {
+      a[NA - 1].add(x[k], y[k]);
+      if (TWO) b[NA - 1].add(x2[k], y2[k]);
+    }
+  typename ThreadSum<T>::type v[TWO ? 2 : 1];
+  v[0] = acc_sum(a);
+  if (TWO) v[TWO ? 1 : 0] = acc_sum(b);
   block_sums<TWO ? 2 : 1>(v, [&](int k, double t) { pr[k * g] = t; });
   finish_if_last(part, fin);
 }
@@ -150,16 +159,11 @@ __global__ void __launch_bounds__(kRedThreads) k_cg_xr(int64_t n, int64_t ld, T*
     elem(x[k], r[k], p[k], Ap[k], ZMODE == 1 ? dinv[k] : T(0), zi, 0);
     if (ZMODE == 1) z[k] = zi;
   }
-#pragma unroll
-  for (int c = 1; c < W; ++c) {
-    a[0].merge(a[c]);
-    if (ZMODE == 1) b[0].merge(b[c]);
-  }
   double* const pr = part + int64_t(rh) * 2 * gridDim.x + blockIdx.x;
   const int64_t g = gridDim.x;
-  DotAcc<T> v[ZMODE == 1 ? 2 : 1];
-  v[0] = a[0];
-  if (ZMODE == 1) v[ZMODE == 1 ? 1 : 0] = b[0];
+  typename ThreadSum<T>::type v[ZMODE == 1 ? 2 : 1];
+  v[0] = acc_sum(a);
+  if (ZMODE == 1) v[ZMODE == 1 ? 1 : 0] = acc_sum(b);
   block_sums<ZMODE == 1 ? 2 : 1>(v, [&](int k, double t) {
     pr[k * g] = t;
     if (ZMODE == 0) pr[g] = t;
