@@ -58,10 +58,12 @@ template <> struct ThreadSum<float> { using type = Sum3f; };
 
 // Per-block partial sums of x.y (and, TWO, x2.y2).  Each thread keeps an accumulator per element of a
 // 16-byte word (every vector aligned), and two words of each vector in flight; W = 1 where a vector is
-// not aligned, with four elements in flight.  The partition and the summation order are fixed, so results are reproducible
-// bit for bit.
+// not aligned (also every vector but the first of a batch with an odd stride), with 32 bytes of each in flight.  The
+// four blocks per SM of the grid may take 64 registers each in fp32: without that bound the compiler keeps 32, which
+// serialises the loads of the unaligned fp32 form (17 M elements: 55.0 us, 26.3 so).  The partition and the summation
+// order are fixed, so results are reproducible bit for bit.
 template <typename T, int W, bool TWO>
-__global__ void __launch_bounds__(kRedThreads) k_dot2_partial(const T* x, const T* y, const T* x2, const T* y2, int64_t n,
+__global__ void __launch_bounds__(kRedThreads, sizeof(T) == 4 ? 4 : 0) k_dot2_partial(const T* x, const T* y, const T* x2, const T* y2, int64_t n,
                                                              int64_t ld, double* part, Finish fin) {
   using V = Word<T, W>;
   const int r = blockIdx.y;
@@ -71,7 +73,7 @@ __global__ void __launch_bounds__(kRedThreads) k_dot2_partial(const T* x, const 
   const V *xw = reinterpret_cast<const V*>(x), *yw = reinterpret_cast<const V*>(y);
   const V *xw2 = reinterpret_cast<const V*>(x2), *yw2 = reinterpret_cast<const V*>(y2);
   // words in flight per vector, and accumulators: one per element of a word and (pairs) one for the remainder, or four
-  constexpr int UN = W == 1 ? 4 : 2, NA = W == 1 ? 4 : W + (sizeof(T) == 4);
+  constexpr int UN = W == 1 ? 32 / int(sizeof(T)) : 2, NA = W == 1 ? 4 : W + (sizeof(T) == 4);
   DotAcc<T> a[NA], b[NA];
   int64_t i = t0;
   for (; i + (UN - 1) * st < nw; i += UN * st) {
