@@ -855,12 +855,13 @@ static mf_status ensure_oseen_tiles(mf_op* op, bool* ok) {
   return MF_OK;
 }
 
-// Builds what the applies of a solve read before the solve records them into a graph.
-mf_status prepare_f32_applies(mf_op* op) {
+// Builds what applies to nrhs right-hand sides read, before a solve records them into a graph.
+mf_status prepare_f32_applies(mf_op* op, int nrhs) {
   bool ok;
   if (op->p.kind == MF_OP_OSEEN) return ensure_oseen_tiles(op, &ok);
   if (op->f32_prec == PREC_F32 && octree_rhs_lanes(op, 2)) return ensure_octree_rhs(op, &ok);
-  if (op->f32_prec == PREC_F32 && (op->mode32 == 1 || heat_tabulated(op))) return ensure_tiles(op, &ok);
+  if (op->f32_prec == PREC_F32 && (op->mode32 == 1 || heat_tabulated(op)) && march_serves(op->ctx, op->map[0], nrhs))
+    return ensure_tiles(op, &ok);
   return MF_OK;
 }
 
@@ -1053,7 +1054,7 @@ mf_status apply_impl(mf_op* op, const T* src, T* dst, int nrhs, int64_t ld, bool
   }
   if constexpr (sizeof(T) == 4) {
     // tabulated fp32 applies on uniform meshes: the marching kernel on its own coefficient tables
-    bool tiles = prec == PREC_F32 && m == 1 && nrhs <= 65535 && !op->general_f32;
+    bool tiles = prec == PREC_F32 && m == 1 && nrhs <= 65535 && !op->general_f32 && march_serves(c, op->map[0], nrhs);
     if (tiles) MF_TRY(ensure_tiles(op, &tiles));
     if (tiles) {
       const bool qm = kind == K_HEAT && op->rhocp_user;

@@ -148,6 +148,7 @@ mf_status tc_take_error();
 int64_t tile_table_floats(const mf_dofmap* m, int rows);
 mf_status launch_tile_table(mf_ctx* ctx, const mf_dofmap* m, int which, const double* c, float* out);
 mf_status launch_tile_table_plain(mf_ctx* ctx, const mf_dofmap* m, const double* c, int rows, double scale, float* out);
+bool march_serves(const mf_ctx* ctx, const mf_dofmap* m, int nrhs);   // or else the general kernel does
 mf_status launch_scalar_f32_uniform(mf_ctx* ctx, const mf_dofmap* m, const float* src, float* dst, int nrhs, int64_t ld,
                                     const float* c, const float* b, const float* qm, double mass, bool transpose);
 // fp32 reinitialisation apply to 2..8 right-hand sides on an octree map: per leaf in processing order its

@@ -23,7 +23,7 @@ bool heat_convection(const mf_op* op);
 int qk_degree(const mf_op* op);
 bool heat_tabulated(const mf_op* op);
 mf_status ensure_tables(mf_op* op);
-mf_status prepare_f32_applies(mf_op* op);
+mf_status prepare_f32_applies(mf_op* op, int nrhs);
 int64_t octree_rhs_work(const mf_op* op, int nrhs);
 int scalar_kind(const mf_op* op);
 double value_coef(const mf_op* op);
@@ -535,7 +535,7 @@ template <typename T> struct CG {
     nrhs = nr;
     const int64_t n = op->n * nrhs;
     if (sizeof(T) == 4) {
-      MF_TRY(prepare_f32_applies(op));
+      MF_TRY(prepare_f32_applies(op, nrhs));
       const int64_t floats = octree_rhs_work(op, nrhs);
       if (floats > 0) {
         const mf_status st = work.alloc(floats);
@@ -1230,7 +1230,7 @@ mf_status autotune_measure(mf_op* op) {
         }
       }
       op->df64_faster = df_ms < std::min(ms[0], ms[1]);
-      MF_TRY(prepare_f32_applies(op));
+      MF_TRY(prepare_f32_applies(op, 1));
       cudaEventDestroy(a0);
       cudaEventDestroy(a1);
       char buf[256];
@@ -1319,7 +1319,7 @@ mf_status autotune_measure(mf_op* op) {
     double f64_ms, df_ms, f32_ms, line64_ms = -1.0, line32_ms = -1.0;
     op->q2_line64 = op->q2_line32 = 0;
     MF_TRY(time_variant(PREC_F32, &f32_ms));
-    if (batch) MF_TRY(prepare_f32_applies(op));
+    if (batch) MF_TRY(prepare_f32_applies(op, 8));
     MF_TRY(time_variant(PREC_F64, &f64_ms));
     MF_TRY(time_variant(PREC_DF64, &df_ms));
     const int kind = scalar_kind(op);
