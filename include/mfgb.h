@@ -401,7 +401,9 @@ mf_status mf_heat_step_gradient(mf_op* op, const mf_laser* laser, const mf_solve
  * per cell for uniform Q2 Helmholtz and heat; fp64 pipes or double-float; Oseen: the fp64 loop order;
  * Q3 Helmholtz: the CUDA-core or the tensor-core kernel for fp32 applies, which then also serves the
  * fp32 applies inside solvers) and keep the fastest.  The tables of the fp32 applies are built here too,
- * instead of at the first such apply.  cache_path (may be NULL) is a
+ * instead of at the first such apply, and on octrees the context's pool is given the work area of batched fp32
+ * reinitialisation (64 bytes per DoF, rounded up to 32 MiB, for up to eight right-hand sides at a time; a first batch
+ * without tuning makes it).  The pool keeps it until the operator is destroyed.  cache_path (may be NULL) is a
  * text file of one JSON record per line, keyed by the operator's configuration (kind, degree, mesh
  * type and sizes, optional fields, melt-pool flags, the device's SM count): if it holds a record with
  * this operator's key, the last such record's choice is applied and nothing is timed; otherwise the

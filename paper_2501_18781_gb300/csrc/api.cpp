@@ -36,7 +36,6 @@ BlockPool::BlockPool() {
 }
 BlockPool::~BlockPool() {
   trim();
-  if (call_pool) cudaMemPoolDestroy(call_pool);
   std::lock_guard<std::mutex> lk(g_pools_mu);
   g_pools.erase(std::remove(g_pools.begin(), g_pools.end(), this), g_pools.end());
 }
@@ -75,36 +74,48 @@ void BlockPool::trim() {
   for (auto& kv : keep) cudaFree(kv.second);
   keep.clear();
   kept = 0;
-  if (call_pool) {
-    cudaDeviceSynchronize();
-    cudaMemPoolTrimTo(call_pool, 0);
-  }
+  calls->trim();
 }
-// Work memory of one call, in the order of its stream (hand back with cudaFreeAsync on that stream).  The
-// pool keeps what was handed back, at most the largest work areas that ran at once; NULL if there is none.
-mf_status BlockPool::call_get(size_t n, cudaStream_t s, void** out) {
+CallPool::~CallPool() {
+  if (pool) cudaMemPoolDestroy(pool);
+}
+mf_status CallPool::get(size_t n, cudaStream_t s, void** out) {
   *out = nullptr;
   std::lock_guard<std::mutex> lk(mu);
-  if (!call_pool) {
+  if (!pool) {
     cudaMemPoolProps p{};
     p.allocType = cudaMemAllocationTypePinned;
     p.location.type = cudaMemLocationTypeDevice;
     int dev = 0;
     MF_CUDA_TRY(cudaGetDevice(&dev));
     p.location.id = dev;
-    if (cudaMemPoolCreate(&call_pool, &p) != cudaSuccess) {
+    if (cudaMemPoolCreate(&pool, &p) != cudaSuccess) {
       cudaGetLastError();
-      call_pool = nullptr;
+      pool = nullptr;
       return MF_OK;
     }
-    uint64_t keep_all = UINT64_MAX;
-    cudaMemPoolSetAttribute(call_pool, cudaMemPoolAttrReleaseThreshold, &keep_all);
+    uint64_t keep = uint64_t(reserved);
+    cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
   }
-  if (cudaMallocFromPoolAsync(out, n, call_pool, s) != cudaSuccess) {
+  if (cudaMallocFromPoolAsync(out, n, pool, s) != cudaSuccess) {
     cudaGetLastError();
     *out = nullptr;
   }
   return MF_OK;
+}
+void CallPool::reserve(int64_t delta) {
+  std::lock_guard<std::mutex> lk(mu);
+  reserved += delta;
+  if (!pool) return;
+  uint64_t keep = uint64_t(reserved);
+  cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
+  if (delta < 0) cudaMemPoolTrimTo(pool, size_t(reserved));
+}
+void CallPool::trim() {
+  std::lock_guard<std::mutex> lk(mu);
+  if (!pool) return;
+  cudaDeviceSynchronize();
+  cudaMemPoolTrimTo(pool, 0);
 }
 void trim_block_pools() {
   std::lock_guard<std::mutex> lk(g_pools_mu);
@@ -855,6 +866,16 @@ static mf_status ensure_oseen_tiles(mf_op* op, bool* ok) {
   return MF_OK;
 }
 
+// The work area of batched fp32 octree applies, made before the first of them: reserved, and brought into the pool.
+mf_status reserve_octree_rhs(mf_op* op) {
+  const size_t bytes = sizeof(float) * size_t(octree_rhs_work(op, 8));
+  if (bytes == 0 || !op->rhs_reserve.raise(op->ctx->pool.calls, bytes)) return MF_OK;
+  void* p = nullptr;
+  MF_TRY(op->ctx->pool.calls->get(bytes, op->ctx->stream, &p));
+  if (p) MF_CUDA_TRY(cudaFreeAsync(p, op->ctx->stream));
+  return MF_OK;
+}
+
 // Builds what applies to nrhs right-hand sides read, before a solve records them into a graph.
 mf_status prepare_f32_applies(mf_op* op, int nrhs) {
   bool ok;
@@ -908,7 +929,8 @@ mf_status apply_impl(mf_op* op, const T* src, T* dst, int nrhs, int64_t ld, bool
       float* work = op->rhs_work && op->rhs_work_floats >= floats ? op->rhs_work : nullptr;
       void* own = nullptr;
       if (ok && !work && may_allocate(op)) {
-        MF_TRY(c->pool.call_get(sizeof(float) * floats, c->stream, &own));
+        op->rhs_reserve.raise(c->pool.calls, sizeof(float) * floats);
+        MF_TRY(c->pool.calls->get(sizeof(float) * floats, c->stream, &own));
         work = static_cast<float*>(own);
       }
       if (ok && work) {

@@ -5,6 +5,7 @@
 #include <stdint.h>
 
 #include <map>
+#include <memory>
 #include <mutex>
 #include <string>
 #include <vector>
@@ -71,6 +72,44 @@ struct DevBuf {
   }
 };
 
+// Stream-ordered work memory of single calls (hand back with cudaFreeAsync on the call's stream).  The pool keeps
+// what the live operators have reserved (a CallReserve each) and returns the rest to the device at the next
+// synchronisation.  Shared by a context and its operators, whichever goes last.
+struct CallPool {
+  std::mutex mu;
+  cudaMemPool_t pool = nullptr;   // created on first use
+  int64_t reserved = 0;
+  CallPool() = default;
+  CallPool(const CallPool&) = delete;
+  CallPool& operator=(const CallPool&) = delete;
+  ~CallPool();
+  mf_status get(size_t n, cudaStream_t s, void** out);   // *out NULL if there is none
+  void reserve(int64_t delta);                           // bytes more or less
+  void trim();
+};
+struct CallReserve {
+  // pools grow by 32 MiB: a release threshold below a whole step would give the memory back at every
+  // synchronisation (a batched apply on the base 5 + 1 octree, the stream idle before: 31 us, then 210)
+  static constexpr size_t kStep = size_t(32) << 20;
+  std::shared_ptr<CallPool> pool;
+  size_t bytes = 0;
+  CallReserve() = default;
+  CallReserve(const CallReserve&) = delete;
+  CallReserve& operator=(const CallReserve&) = delete;
+  ~CallReserve() {
+    if (pool) pool->reserve(-int64_t(bytes));
+  }
+  // at least n bytes, rounded up to whole steps, from now on; true if that is more than before
+  bool raise(const std::shared_ptr<CallPool>& p, size_t n) {
+    n = (n + kStep - 1) / kStep * kStep;
+    if (n <= bytes) return false;
+    pool = p;
+    pool->reserve(int64_t(n - bytes));
+    bytes = n;
+    return true;
+  }
+};
+
 // Device blocks a context keeps for reuse (the solvers' work vectors, allocated and freed on every
 // solve).  A block handed back may still be read by work queued on the context's stream; every
 // later user queues its work on the same stream, so the reuse needs no synchronisation.  Sizes
@@ -84,9 +123,7 @@ struct BlockPool {
   ~BlockPool();
   BlockPool(const BlockPool&) = delete;
   BlockPool& operator=(const BlockPool&) = delete;
-  // stream-ordered memory of single calls (created on first use; trimmed with the kept blocks)
-  cudaMemPool_t call_pool = nullptr;
-  mf_status call_get(size_t n, cudaStream_t s, void** out);
+  std::shared_ptr<CallPool> calls = std::make_shared<CallPool>();   // trimmed with the kept blocks
   static size_t rounded(size_t n) {
     const size_t big = size_t(2) << 20, small = 512;
     return n >= (size_t(1) << 20) ? (n + big - 1) / big * big : (n + small - 1) / small * small;

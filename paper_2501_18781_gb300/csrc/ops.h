@@ -230,7 +230,8 @@ struct mf_op {
   bool general_f32 = false;            // mf_autotune: time the general kernel
   mf::DevBuf rhs_map, rhs_nrm;         // fp32 octree kernel for several right-hand sides: per-leaf tables
   bool rhs_ready = false;
-  float* rhs_work = nullptr;           // its work vectors while a solve lends them, else per call
+  mf::CallReserve rhs_reserve;         // what the context's pool keeps for its work vectors, made per call
+  float* rhs_work = nullptr;           // or lent by a solve
   int64_t rhs_work_floats = 0;
   mf::DevBuf cm_df, cv_df, cb_df;   // Oseen: folded coefficients as float pairs per tile of 32 cells
   mf::DevBuf nrm_df;                // Oseen melt-pool terms: the interface normal, likewise

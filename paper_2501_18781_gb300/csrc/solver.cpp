@@ -25,6 +25,7 @@ bool heat_tabulated(const mf_op* op);
 mf_status ensure_tables(mf_op* op);
 mf_status prepare_f32_applies(mf_op* op, int nrhs);
 int64_t octree_rhs_work(const mf_op* op, int nrhs);
+mf_status reserve_octree_rhs(mf_op* op);
 int scalar_kind(const mf_op* op);
 double value_coef(const mf_op* op);
 template <typename T> ScalarArgs<T> scalar_args(const mf_op* op, const T* src, T* dst, int nrhs, int64_t ld);
@@ -1319,7 +1320,10 @@ mf_status autotune_measure(mf_op* op) {
     double f64_ms, df_ms, f32_ms, line64_ms = -1.0, line32_ms = -1.0;
     op->q2_line64 = op->q2_line32 = 0;
     MF_TRY(time_variant(PREC_F32, &f32_ms));
-    if (batch) MF_TRY(prepare_f32_applies(op, 8));
+    if (batch) {
+      MF_TRY(prepare_f32_applies(op, 8));
+      MF_TRY(reserve_octree_rhs(op));
+    }
     MF_TRY(time_variant(PREC_F64, &f64_ms));
     MF_TRY(time_variant(PREC_DF64, &df_ms));
     const int kind = scalar_kind(op);
