@@ -880,7 +880,7 @@ mf_status reserve_octree_rhs(mf_op* op) {
 mf_status prepare_f32_applies(mf_op* op, int nrhs) {
   bool ok;
   if (op->p.kind == MF_OP_OSEEN) return ensure_oseen_tiles(op, &ok);
-  if (op->f32_prec == PREC_F32 && octree_rhs_lanes(op, 2)) return ensure_octree_rhs(op, &ok);
+  if (op->f32_prec == PREC_F32 && octree_rhs_lanes(op, nrhs)) return ensure_octree_rhs(op, &ok);
   if (op->f32_prec == PREC_F32 && (op->mode32 == 1 || heat_tabulated(op)) && march_serves(op->ctx, op->map[0], nrhs))
     return ensure_tiles(op, &ok);
   return MF_OK;

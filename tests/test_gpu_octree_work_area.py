@@ -1,5 +1,5 @@
 """Work memory of batched fp32 applies on octrees: made when the operator is tuned, not by an apply, and given
-back with the operator."""
+back with the operator; solves of one right-hand side do not prepare for batches."""
 import gc
 
 import numpy as np
@@ -61,3 +61,20 @@ def test_memory_is_made_by_autotune_and_given_back():
     assert float((v - first).abs().max()) <= 1e-5 * float(first.abs().max())
     del op
     assert before - _free() < area // 4
+
+
+def test_single_solves_prepare_nothing_for_batches():
+    ctx, m = _world()
+    tables = 448 * m.n_cells        # node numbers, levels and normals per leaf
+    b = torch.tensor(syn.uniform_pm1(7, m.n_dofs), device="cuda")
+    kw = dict(solver="defect_correction", precond="jacobi", tol=1e-8)
+    used = []
+    for _ in range(2):              # the first one fills the context's block pool
+        op = _reinit(ctx, m)
+        op.apply(b.float())
+        start = _free()
+        _, info = op.solve(b, **kw)
+        assert info["status"] == 0
+        used.append(start - _free())
+        del op
+    assert used[1] < tables // 2, used
