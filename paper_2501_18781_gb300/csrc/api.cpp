@@ -534,6 +534,7 @@ mf_status mf_operator_set_field(mf_op* op, int field, const void* ptr, int dtype
   op->df_ready = false;
   op->tiles_ready = false;
   op->rhs_ready = false;
+  op->tiles_denied = op->rhs_denied = op->df_denied = false;
   op->diag_ready = false;
   op->lanczos_ready = false;
   op->h16_cnorm = 0.0f;
@@ -784,7 +785,7 @@ static mf_status ensure_tiles(mf_op* op, bool* ok) {
   const int kind = scalar_kind(op);
   *ok = op->map[0]->uniform && op->map[0]->degree == 2 && (kind == K_HELM || kind == K_HEAT);
   if (!*ok || op->tiles_ready) return MF_OK;
-  if (!may_allocate(op)) {
+  if (op->tiles_denied || !may_allocate(op)) {
     *ok = false;
     return MF_OK;
   }
@@ -803,6 +804,7 @@ static mf_status ensure_tiles(mf_op* op, bool* ok) {
     const mf_status st = parts[w].buf->alloc(sizeof(float) * tile_table_floats(op->map[0], parts[w].rows));
     if (st == MF_ENOMEM) {
       *ok = false;
+      op->tiles_denied = true;
       return MF_OK;
     }
     MF_TRY(st);
@@ -825,13 +827,14 @@ int64_t octree_rhs_work(const mf_op* op, int nrhs) {
 static mf_status ensure_octree_rhs(mf_op* op, bool* ok) {
   *ok = true;
   if (op->rhs_ready) return MF_OK;
-  *ok = may_allocate(op);
+  *ok = !op->rhs_denied && may_allocate(op);
   if (!*ok) return MF_OK;
   MF_TRY(ensure_tables(op));
   mf_status st = op->rhs_map.alloc(sizeof(int32_t) * 28 * op->ncells);
   if (st == MF_OK) st = op->rhs_nrm.alloc(sizeof(float) * 84 * op->ncells);
   if (st == MF_ENOMEM) {
     *ok = false;
+    op->rhs_denied = true;
     return MF_OK;
   }
   MF_TRY(st);
@@ -845,7 +848,7 @@ static mf_status ensure_octree_rhs(mf_op* op, bool* ok) {
 static mf_status ensure_oseen_tiles(mf_op* op, bool* ok) {
   *ok = true;
   if (op->tiles_ready) return MF_OK;
-  *ok = may_allocate(op);
+  *ok = !op->tiles_denied && may_allocate(op);
   if (!*ok) return MF_OK;
   MF_TRY(ensure_tables(op));
   const bool ext = op->p.oseen_flags != 0;
@@ -856,6 +859,7 @@ static mf_status ensure_oseen_tiles(mf_op* op, bool* ok) {
   if (st == MF_OK && ext) st = op->tile_n.alloc(3 * one);
   if (st == MF_ENOMEM) {
     *ok = false;
+    op->tiles_denied = true;
     return MF_OK;
   }
   MF_TRY(st);
@@ -879,6 +883,7 @@ mf_status reserve_octree_rhs(mf_op* op) {
 // Builds what applies to nrhs right-hand sides read, before a solve records them into a graph.
 mf_status prepare_f32_applies(mf_op* op, int nrhs) {
   bool ok;
+  op->tiles_denied = op->rhs_denied = false;
   if (op->p.kind == MF_OP_OSEEN) return ensure_oseen_tiles(op, &ok);
   if (op->f32_prec == PREC_F32 && octree_rhs_lanes(op, nrhs)) return ensure_octree_rhs(op, &ok);
   if (op->f32_prec == PREC_F32 && (op->mode32 == 1 || heat_tabulated(op)) && march_serves(op->ctx, op->map[0], nrhs))
@@ -960,8 +965,8 @@ mf_status apply_impl(mf_op* op, const T* src, T* dst, int nrhs, int64_t ld, bool
         // double-float: one warp per velocity component over a brick of 32 cells (the Darcy term is
         // folded into cm; the trace correction reads the interface normal pairs)
         const bool ext = op->p.oseen_flags != 0;
-        bool ok = true;
-        if (!op->df_ready) {
+        bool ok = !op->df_denied;
+        if (ok && !op->df_ready) {
           // tables per tile of 32 cells, padded to whole tiles; without the memory the fp64 pipes do it
           const size_t one = sizeof(float2) * tile_table_floats(op->map[0], 1);
           mf_status st = op->cm_df.alloc(one);
@@ -969,6 +974,7 @@ mf_status apply_impl(mf_op* op, const T* src, T* dst, int nrhs, int64_t ld, bool
           if (st == MF_OK) st = op->cb_df.alloc(3 * one);
           if (st == MF_OK && ext) st = op->nrm_df.alloc(3 * one);
           ok = st != MF_ENOMEM;
+          op->df_denied = !ok;
           if (ok) {
             MF_TRY(st);
             MF_TRY(launch_oseen_df_split(c, op->map[0], op->cm64.as<double>(), op->cv64.as<double>(), op->cb64.as<double>(),

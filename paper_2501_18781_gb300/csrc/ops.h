@@ -227,6 +227,9 @@ struct mf_op {
   mf::DevBuf tile_c, tile_b, tile_m;   // fp32 uniform kernels: coefficient tables per tile of cells (Oseen: cm, cb, cv)
   mf::DevBuf tile_n;                   // Oseen melt-pool terms: the interface normal per tile
   bool tiles_ready = false;
+  // no memory for these tables: applies take the general kernels and do not ask again before a field is set, the
+  // operator is tuned or an fp32 solve prepares (every failed allocation trims the pools and waits for the device)
+  bool tiles_denied = false, rhs_denied = false, df_denied = false;
   bool general_f32 = false;            // mf_autotune: time the general kernel
   mf::DevBuf rhs_map, rhs_nrm;         // fp32 octree kernel for several right-hand sides: per-leaf tables
   bool rhs_ready = false;

@@ -1155,6 +1155,7 @@ bool apply_cached_choice(mf_op* op, const char* cache_path) {
 mf_status autotune_measure(mf_op* op) {
   try {
     MF_TRY(check_fields(op));
+    op->tiles_denied = op->rhs_denied = op->df_denied = false;
     mf_ctx* c = op->ctx;
     const int64_t n = op->n;
     if (qk_degree(op) == 4) {  // Q4: one kernel variant per precision, nothing to choose
