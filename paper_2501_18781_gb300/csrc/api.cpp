@@ -772,7 +772,7 @@ mf_status apply_h16(mf_op* op, const float* src, float* dst, int nrhs, int64_t l
 }
 
 // Whether memory can be allocated now: not while the context's stream is being captured into a graph.
-static bool may_allocate(const mf_op* op) {
+bool may_allocate(const mf_op* op) {
   cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(op->ctx->stream, &st) != cudaSuccess) cudaGetLastError();
   return st == cudaStreamCaptureStatusNone;

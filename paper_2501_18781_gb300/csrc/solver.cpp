@@ -23,6 +23,7 @@ bool heat_convection(const mf_op* op);
 int qk_degree(const mf_op* op);
 bool heat_tabulated(const mf_op* op);
 mf_status ensure_tables(mf_op* op);
+bool may_allocate(const mf_op* op);
 mf_status prepare_f32_applies(mf_op* op, int nrhs);
 int64_t octree_rhs_work(const mf_op* op, int nrhs);
 mf_status reserve_octree_rhs(mf_op* op);
@@ -1232,7 +1233,6 @@ mf_status autotune_measure(mf_op* op) {
         }
       }
       op->df64_faster = df_ms < std::min(ms[0], ms[1]);
-      MF_TRY(prepare_f32_applies(op, 1));
       cudaEventDestroy(a0);
       cudaEventDestroy(a1);
       char buf[256];
@@ -1321,10 +1321,6 @@ mf_status autotune_measure(mf_op* op) {
     double f64_ms, df_ms, f32_ms, line64_ms = -1.0, line32_ms = -1.0;
     op->q2_line64 = op->q2_line32 = 0;
     MF_TRY(time_variant(PREC_F32, &f32_ms));
-    if (batch) {
-      MF_TRY(prepare_f32_applies(op, 8));
-      MF_TRY(reserve_octree_rhs(op));
-    }
     MF_TRY(time_variant(PREC_F64, &f64_ms));
     MF_TRY(time_variant(PREC_DF64, &df_ms));
     const int kind = scalar_kind(op);
@@ -1356,6 +1352,16 @@ mf_status autotune_measure(mf_op* op) {
   }
 }
 
+// What a tuned operator's fp32 applies read, so that none of them has to build it (under stream capture they
+// could not).  Tables that do not fit are left to the applies.
+mf_status build_tuned_tables(mf_op* op) {
+  if (!may_allocate(op)) return MF_OK;
+  mf_status st = ensure_tables(op);
+  if (st == MF_OK) st = prepare_f32_applies(op, 8);
+  if (st == MF_OK) st = reserve_octree_rhs(op);
+  return st == MF_ENOMEM ? MF_OK : st;
+}
+
 }  // namespace
 
 extern "C" {
@@ -1364,8 +1370,9 @@ mf_status mf_autotune(mf_op* op, const char* cache_path) {
   try {
     if (!op) return fail(MF_EINVAL, "NULL argument");
     MF_TRY(check_fields(op));
-    if (cache_path && apply_cached_choice(op, cache_path)) return MF_OK;
+    if (cache_path && apply_cached_choice(op, cache_path)) return build_tuned_tables(op);
     MF_TRY(autotune_measure(op));
+    MF_TRY(build_tuned_tables(op));
     const std::string rec = "{\"key\": \"" + tune_key(op) + "\", " + tune_choice(op) + ", \"timings\": " +
                             op->tune_record + "}";
     op->tune_record = rec;

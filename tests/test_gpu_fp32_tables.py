@@ -1,4 +1,7 @@
-"""When the tables of the fp32 kernels are built: once per set of fields where the memory is not there."""
+"""When the tables of the fp32 kernels are built: by mf_autotune also where it reads its choice from a record, so
+that an apply under stream capture finds them; and once per set of fields where the memory is not there."""
+import json
+
 import pytest
 
 import synthetic as syn
@@ -24,6 +27,33 @@ def _heat(ctx, n, beta=False):
     if beta:
         op.set_field("beta", torch.tensor(syn.uniform_pm1(5, 3 * m.n_dofs) / n, device="cuda"))
     return op
+
+
+def test_autotune_from_a_record_builds_the_tables(build, tmp_path):
+    from paper_2501_18781_gb300 import Context
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        ctx = Context(0, stream)
+        path = str(tmp_path / "tune.jsonl")
+        _heat(ctx, 12).autotune(path)
+        rec = json.loads(open(path).read().splitlines()[-1])
+        with open(path, "a") as f:   # the tabulated form with one thread per cell
+            f.write(json.dumps(dict(rec, mode32=1, q2_line32=0)) + "\n")
+        op = _heat(ctx, 12)
+        op.autotune(path)
+        u = torch.tensor(syn.uniform_pm1(11, op.n), device="cuda").float()
+        v = torch.zeros_like(u)
+    stream.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=stream):
+        op.apply(u, v)
+    assert "/f32/tabulated/march" in op.variant, op.variant
+    graph.replay()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(stream):
+        ref = op.apply(u.double())
+    stream.synchronize()
+    assert float((v.double() - ref).abs().max()) <= 2e-5 * float(ref.abs().max())
 
 
 def test_a_failed_build_is_not_repeated_by_every_apply(build):
