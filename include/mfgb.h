@@ -405,7 +405,8 @@ mf_status mf_heat_step_gradient(mf_op* op, const mf_laser* laser, const mf_solve
  * reinitialisation (64 bytes per DoF, rounded up to 32 MiB, for up to eight right-hand sides at a time; a first batch
  * without tuning makes it).  The pool keeps it until the operator is destroyed.  cache_path (may be NULL) is a
  * text file of one JSON record per line, keyed by the operator's configuration (kind, degree, mesh
- * type and sizes, optional fields, melt-pool flags, the device's SM count): if it holds a record with
+ * type and sizes, optional fields, melt-pool flags, the device's SM count, the generation of the library's
+ * kernels): if it holds a record with
  * this operator's key, the last such record's choice is applied and nothing is timed; otherwise the
  * variants are timed and the record (key, choice, timings) is appended.  Synchronising when it times. */
 mf_status mf_autotune(mf_op* op, const char* cache_path);

@@ -1089,15 +1089,18 @@ mf_status mf_heat_step_gradient(mf_op* op, const mf_laser* lz, const mf_solver_p
 namespace {
 
 // The configuration that decides which variant is fastest: operator kind and degree, mesh type
-// and sizes, the optional fields, the melt-pool flags and the device's SM count.
+// and sizes, the optional fields, the melt-pool flags and the device's SM count; and the generation of the
+// kernels that are chosen among, to be raised with every change of their speed: choices that an earlier
+// library timed are not applied to other kernels.
+constexpr int kTuneGeneration = 2;
 std::string tune_key(const mf_op* op) {
   const mf_dofmap* m = op->map[0];
   char buf[320];
   std::snprintf(buf, sizeof buf, "kind=%d deg=%d %s dofs=%lld cells=%lld con=%lld beta=%d kq=%d rhocp=%d betaq=%d "
-                "mode=%d flags=%d sms=%d", op->p.kind, m->degree, m->uniform ? "uniform" : "octree",
+                "mode=%d flags=%d sms=%d kernels=%d", op->p.kind, m->degree, m->uniform ? "uniform" : "octree",
                 (long long)op->n, (long long)op->ncells, (long long)(m->con_rowptr.empty() ? 0 : m->con_rowptr.size() - 1), op->beta ? 1 : 0,
                 op->kq_user ? 1 : 0, op->rhocp_user ? 1 : 0, op->betaq_user ? 1 : 0, op->p.coef_mode,
-                op->p.oseen_flags, op->ctx->sm_count);
+                op->p.oseen_flags, op->ctx->sm_count, kTuneGeneration);
   return buf;
 }
 
