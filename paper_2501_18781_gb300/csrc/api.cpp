@@ -690,8 +690,8 @@ template <typename T> ScalarArgs<T> scalar_args(const mf_op* op, const T* src, T
   a.k_slope = T(0.5 * op->p.k0 / (op->p.t_boil > 0 ? op->p.t_boil : 1.0));
   a.eps = T(op->p.eps);
   a.heaviside = op->p.heaviside;
-  a.block = op->block;
-  a.persistent_blocks = op->persistent_blocks;
+  a.block = nrhs > 1 ? op->batch_block : op->block;
+  a.persistent_blocks = nrhs > 1 ? op->batch_persistent : op->persistent_blocks;
   return a;
 }
 template ScalarArgs<double> scalar_args<double>(const mf_op*, const double*, double*, int, int64_t);
@@ -927,7 +927,7 @@ mf_status apply_impl(mf_op* op, const T* src, T* dst, int nrhs, int64_t ld, bool
   if (needs_tables) MF_TRY(ensure_tables(op));
   if constexpr (sizeof(T) == 4) {
     // fp32 reinitialisation of several right-hand sides on an octree: groups of eight, interleaved
-    if (prec == PREC_F32 && octree_rhs_lanes(op, nrhs)) {
+    if (prec == PREC_F32 && octree_rhs_lanes(op, nrhs) && !op->general_f32) {
       bool ok;
       MF_TRY(ensure_octree_rhs(op, &ok));
       const int64_t floats = octree_rhs_work(op, std::min(nrhs, 8));
@@ -1100,8 +1100,8 @@ mf_status apply_impl(mf_op* op, const T* src, T* dst, int nrhs, int64_t ld, bool
   op->variant = std::string(kind == K_HELM ? "helmholtz" : kind == K_HEAT ? "heat" : "reinit") +
                 (op->map[0]->uniform ? "/uniform" : "/octree") + pname +
                 (m == 0 ? "/inkernel" : "/tabulated") + (beta ? (transpose ? "/conv-T" : "/conv") : "") + "/block" +
-                std::to_string(op->map[0]->uniform ? 128 : op->block) +
-                (op->persistent_blocks > 0 ? "/persistent" + std::to_string(op->persistent_blocks) : "");
+                std::to_string(op->map[0]->uniform ? 128 : a.block) +
+                (a.persistent_blocks > 0 ? "/persistent" + std::to_string(a.persistent_blocks) : "");
   return MF_OK;
 }
 template mf_status apply_impl<double>(mf_op*, const double*, double*, int, int64_t, bool, int);

@@ -250,6 +250,7 @@ struct mf_op {
   float h16_cnorm = 0.0f;         // 16-bit applies: power of two >= every coefficient (0: not computed)
   int block = 128;                // octree cells per block (autotuned: 64 or 128)
   int persistent_blocks = 0;      // > 0: persistent launch with this many blocks per SM (autotuned)
+  int batch_block = 128, batch_persistent = 0;   // the same for applies to several right-hand sides
   bool df64_faster = false;
   int q2_line64 = 0, q2_line32 = 0;  // uniform Q2 Helmholtz / heat: the line-per-thread kernel (autotuned)       // autotuned: double-float beats the fp64 pipes (used when fp64_arith = 2)
   int oseen_qouter64 = 0;         // Oseen fp64 kernel variant (autotuned)

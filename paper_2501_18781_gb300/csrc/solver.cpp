@@ -1107,9 +1107,10 @@ std::string tune_key(const mf_op* op) {
 std::string tune_choice(const mf_op* op) {
   char buf[256];
   std::snprintf(buf, sizeof buf, "\"mode64\": %d, \"mode32\": %d, \"block\": %d, \"persistent_blocks\": %d, "
-                "\"df64_faster\": %d, \"oseen_qouter64\": %d, \"qk_f32_tc\": %d, \"q2_line64\": %d, "
-                "\"q2_line32\": %d", op->mode64, op->mode32, op->block, op->persistent_blocks, op->df64_faster ? 1 : 0,
-                op->oseen_qouter64, op->qk_f32_tc, op->q2_line64, op->q2_line32);
+                "\"batch_block\": %d, \"batch_persistent\": %d, \"df64_faster\": %d, \"oseen_qouter64\": %d, "
+                "\"qk_f32_tc\": %d, \"q2_line64\": %d, \"q2_line32\": %d", op->mode64, op->mode32, op->block,
+                op->persistent_blocks, op->batch_block, op->batch_persistent, op->df64_faster ? 1 : 0, op->oseen_qouter64,
+                op->qk_f32_tc, op->q2_line64, op->q2_line32);
   return buf;
 }
 
@@ -1133,12 +1134,16 @@ bool apply_cached_choice(mf_op* op, const char* cache_path) {
     line.clear();
   }
   std::fclose(fp);
-  int v[7];
-  const char* names[7] = {"mode64", "mode32", "block", "persistent_blocks", "df64_faster", "oseen_qouter64", "qk_f32_tc"};
+  int v[9];
+  const char* names[9] = {"mode64",         "mode32",    "block",       "persistent_blocks", "df64_faster",
+                          "oseen_qouter64", "qk_f32_tc", "batch_block", "batch_persistent"};
   if (hit.empty()) return false;
-  for (int i = 0; i < 7; ++i)
+  for (int i = 0; i < 9; ++i)
     if (!read_int(hit, names[i], &v[i])) return false;
-  if ((v[0] | v[1]) & ~1 || (v[2] != 64 && v[2] != 128) || v[3] < 0 || v[3] > 64) return false;
+  auto shape = [](int block, int persistent) {
+    return (block == 64 || block == 128) && persistent >= 0 && persistent <= 64;
+  };
+  if ((v[0] | v[1]) & ~1 || !shape(v[2], v[3]) || !shape(v[7], v[8])) return false;
   op->mode64 = v[0];
   op->mode32 = v[1];
   op->block = v[2];
@@ -1146,6 +1151,8 @@ bool apply_cached_choice(mf_op* op, const char* cache_path) {
   op->df64_faster = v[4] != 0;
   op->oseen_qouter64 = v[5] != 0;
   op->qk_f32_tc = v[6] != 0;
+  op->batch_block = v[7];
+  op->batch_persistent = v[8];
   // records written before the line kernel was a choice leave it off
   int l64 = 0, l32 = 0;
   read_int(hit, "q2_line64", &l64);
@@ -1258,9 +1265,9 @@ mf_status autotune_measure(mf_op* op) {
     MF_TRY(d32.alloc(sizeof(float) * n));
     MF_TRY(convert<double, float>(c, n, src.as<double>(), s32.as<float>()));
     // the launch shape of octree operators is timed on a batch of eight right-hand sides (one and eight
-    // prefer different shapes); the reinitialisation, whose fp32 batches have their own kernel, on one
+    // prefer different shapes); the reinitialisation, which is applied both ways, on each
     const bool batch = !op->map[0]->uniform && op->p.kind == MF_OP_REINIT;
-    const int shape_rhs = op->map[0]->uniform || batch ? 1 : 8;
+    const int shape_rhs = op->map[0]->uniform ? 1 : 8;
     DevBuf sb, db;
     if (shape_rhs > 1) {
       MF_TRY(sb.alloc(sizeof(float) * n * shape_rhs));
@@ -1306,18 +1313,29 @@ mf_status autotune_measure(mf_op* op) {
     };
     std::unique_ptr<Shapes> general(new Shapes(op));
     const int shapes[5][2] = {{128, 0}, {64, 0}, {128, 2}, {128, 4}, {64, 8}};
-    double shape_ms[5];
-    int best_shape = 0;
-    for (int si = 0; si < 5; ++si) {
-      shape_ms[si] = 1e30;
-      if (op->map[0]->uniform && shapes[si][0] != 128) continue;
-      op->block = shapes[si][0];
-      op->persistent_blocks = shapes[si][1];
-      MF_TRY(time_variant(PREC_F32, &shape_ms[si], shape_rhs));
-      if (shape_ms[si] < shape_ms[best_shape]) best_shape = si;
-    }
-    op->block = shapes[best_shape][0];
-    op->persistent_blocks = shapes[best_shape][1];
+    auto time_shapes = [&](int nr, int* block, int* persistent) -> mf_status {
+      double best = 1e30;
+      for (const auto& shape : shapes) {
+        if (op->map[0]->uniform && shape[0] != 128) continue;
+        op->block = op->batch_block = shape[0];
+        op->persistent_blocks = op->batch_persistent = shape[1];
+        double ms;
+        MF_TRY(time_variant(PREC_F32, &ms, nr));
+        if (ms >= best) continue;
+        best = ms;
+        *block = shape[0];
+        *persistent = shape[1];
+      }
+      return MF_OK;
+    };
+    int one[2] = {128, 0}, many[2] = {128, 0};
+    MF_TRY(time_shapes(shape_rhs, &many[0], &many[1]));
+    if (batch) MF_TRY(time_shapes(1, &one[0], &one[1]));
+    else std::copy(many, many + 2, one);
+    op->block = one[0];
+    op->persistent_blocks = one[1];
+    op->batch_block = many[0];
+    op->batch_persistent = many[1];
     general.reset();
     // 3) fp64-accurate arithmetic: fp64 pipes vs double-float on the fp32 pipes; on uniform Q2
     //    Helmholtz / heat operators also the line-per-thread kernel in fp64 and fp32 (small meshes)
