@@ -284,11 +284,9 @@ __global__ void __launch_bounds__(kCgThreads, 1) k_q2_line_cg(const __grid_const
       A.Ap[q] = 0.0;
       A.r[q] = r;
       v2[0] = fma(r, r, v2[0]);
-      if (A.dinv) {
-        const double z = A.dinv[q] * r;
-        A.z[q] = z;
-        v2[1] = fma(r, z, v2[1]);
-      }
+      const double z = A.dinv[q] * r;
+      A.z[q] = z;
+      v2[1] = fma(r, z, v2[1]);
     }
     double* const pr = A.part + (1 + 2 * (k & 1)) * int64_t(G);
     block_sums<2>(v2, [&](int w, double s) { pr[w * int64_t(G) + blockIdx.x] = s; });
@@ -339,6 +337,7 @@ int64_t q2_line_cg_cells(const mf_ctx* ctx) { return int64_t(5) * kCgCells * ctx
 mf_status launch_q2_line_cg(mf_ctx* ctx, const mf_dofmap* m, const double* coef, double mass, const double* dinv, double* x,
                             double* r, double* z, double* p, double* p2, double* Ap, double tol, int maxit,
                             bool stop_indefinite, double* S, double* steps) {
+  if (!dinv) return fail(MF_EINVAL, "the one-launch CG is Jacobi-preconditioned");
   LineCgArgs a{};
   a.line = line_args<double>(m, coef, mass);
   a.x = x;
