@@ -30,8 +30,7 @@ namespace {
 struct DfArgs {
   const double* src;
   double* dst;
-  int nrhs;           // right-hand sides, one per blockIdx.y
-  int64_t ld;         // distance between right-hand sides
+  int64_t ld;         // distance between right-hand sides, one per blockIdx.y
   const float2* c;    // [27][ncells] pairs of (5/3) w_q h c_q (c: conductivity or a(phi) at Gauss point q)
   const float2* b;    // convection: [3][27][ncells] pairs of w_q h^2 rho_cp beta_d / (2 delta), or NULL
   const float2* m;    // QM: [27][ncells] pairs of w_q h^3 m_q (m_q = rho_cp,q / dt) in place of wm
@@ -752,7 +751,6 @@ mf_status launch_scalar_df_uniform(mf_ctx* ctx, const mf_dofmap* m, const double
   DfArgs a{};
   a.src = src;
   a.dst = dst;
-  a.nrhs = nrhs;
   a.ld = ld;
   a.c = c;
   a.b = b;
