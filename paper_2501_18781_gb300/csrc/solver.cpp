@@ -899,7 +899,11 @@ mf_status solve_impl(mf_op* op, const mf_solver_params* sp, const double* b, dou
       int its = 0;
       double rr = 0;
       mf_status s2 = gmres(op, P, b + k * n, x + k * n, m, tol, maxit, transpose, &its, &rr);
-      if (s2 != MF_OK && s2 != MF_ENOTCONV) return s2;
+      if (s2 != MF_OK && s2 != MF_ENOTCONV) {
+        // a barrier's time-out belongs to this solve: its flag must not meet the next one
+        const mf_status bar = P.tri ? grid_barrier_take_error(c) : MF_OK;
+        return bar == MF_ETIMEOUT ? bar : s2;
+      }
       if (s2 == MF_ENOTCONV) st = s2;
       inf.iterations += its;
       rel[k] = rr;
