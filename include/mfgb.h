@@ -49,13 +49,13 @@ typedef int mf_status;
 
 /* MF_DF64: fp64 vectors, cell arithmetic in double-float (pairs of fp32 with error-free
  * products and sums, 47-48-bit significand) on the fp32 pipes, which GB300 runs at 64x its fp64
- * rate; accurate to a few 1e-14 relative to |A||u| componentwise.  Helmholtz, heat and Oseen on
- * uniform meshes and reinitialisation on octrees scale the inputs by a power of two per warp of 32
- * cells (Oseen: velocity and pressure separately), so any fp64 magnitude keeps 47 bits relative to
- * the largest input of those cells and inputs more than 2^126 below it count as zero; parts of a result
- * below the smallest normal double are flushed, results beyond the largest are Inf, and an Inf or NaN
- * among the inputs makes the rows of its cells NaN.  The other operators keep the fp32 exponent
- * range (magnitudes between about 1e-38 and 3e38). */
+ * rate; accurate to a few 1e-14 relative to |A||u| componentwise.  Helmholtz, Oseen and heat (but for a
+ * MF_FIELD_RHOCP_QPOINT without convection) on uniform meshes and reinitialisation on octrees scale the
+ * inputs by a power of two per warp of 32 cells (Oseen: velocity and pressure separately), so any fp64 magnitude
+ * keeps 47 bits relative to the largest input of those cells and inputs more than 2^126 below it count as
+ * zero; parts of a result below the smallest normal double may be flushed, results beyond the largest are Inf,
+ * and an Inf or NaN among the inputs makes the rows of its cells NaN.  The other operators, and the Gauss-point
+ * coefficients of all of them, keep the fp32 exponent range (magnitudes between about 1e-38 and 3e38). */
 typedef enum { MF_F64 = 0, MF_F32 = 1, MF_F16 = 2, MF_BF16 = 3, MF_DF64 = 4 } mf_dtype;
 /* mf_solver_params.inner_arith value beside the dtypes: fp32 inner applies on the tensor cores */
 enum { MF_INNER_TENSOR_CORES = 16 };
