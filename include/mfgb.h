@@ -311,7 +311,7 @@ typedef struct {
  * products and sums as unevaluated pairs of floats (the compensated dot product of Ogita, Rump
  * and Oishi, as accurate as evaluation in twice the fp32 precision; fp64 conversions would
  * bound the kernel by the fp64 rate instead of HBM), partials are combined in fp64.  Partial sums go to the context's
- * reduction workspace (allocated once with the context) over a fixed grid and are summed in a
+ * reduction workspace (allocated once with the context) over a grid that n fixes and are summed in a
  * fixed order, so the result is bit-reproducible.  Asynchronous. */
 mf_status mf_dot(mf_ctx* ctx, const void* x, const void* y, int64_t n, int64_t ld, int nvec, int dtype,
                  double* out);
@@ -329,7 +329,7 @@ mf_status mf_dot(mf_ctx* ctx, const void* x, const void* y, int64_t n, int64_t l
  * clearing between calls.
  * x, y: device vectors (MF_F64 or MF_F32) ld apart; out: device array of nvec doubles;
  * cuda_stream: the cudaStream_t to launch on (NULL = the legacy default stream).
- * Asynchronous; results equal mf_dot's bit for bit (same fixed grid, same summation order). */
+ * Asynchronous; results equal mf_dot's bit for bit (same grid, same summation order). */
 mf_status mf_dot_noalloc(const void* x, const void* y, int64_t n, int64_t ld, int nvec, int dtype, double* out,
                          void* cuda_stream);
 

@@ -208,7 +208,7 @@ __global__ void __launch_bounds__(kOctThreads, 4) k_reinit_df_octree(const __gri
   }
   if (!active) return;
   double* __restrict__ dst = A.dst + rhs * A.ld;
-  const Scale scale(bias);
+  const bool far = far_scale(bias);
 #pragma unroll 1
   for (int c = 0; c < 3; ++c) {
     dd R[9];
@@ -227,7 +227,7 @@ __global__ void __launch_bounds__(kOctThreads, 4) k_reinit_df_octree(const __gri
     }
 #pragma unroll
     for (int b = 0; b < 3; ++b) dd_line_values_t(R[3 * b], R[3 * b + 1], R[3 * b + 2]);
-    if (scale.far) {
+    if (far) {
 #pragma unroll
       for (int p = 0; p < 9; ++p) st2(sU + (9 * c + p) * kOctThreads, R[p]);
       continue;
@@ -235,7 +235,7 @@ __global__ void __launch_bounds__(kOctThreads, 4) k_reinit_df_octree(const __gri
     uint32_t hanging = 0;
 #pragma unroll
     for (int p = 0; p < 9; ++p) {
-      const double v = scale.join(R[p]);
+      const double v = join(R[p], bias);
       if (id[p] >= 0) {
         if (!(og.dflag && __ldg(og.dflag + id[p]))) atomicAdd(dst + id[p], v);
       } else {
@@ -253,10 +253,10 @@ __global__ void __launch_bounds__(kOctThreads, 4) k_reinit_df_octree(const __gri
       }
     }
   }
-  if (bad || scale.far) {   // a NaN into every row of the cell; the test side of a warp with such a scale
+  if (bad || far) {   // a NaN into every row of the cell; the test side of a warp with such a scale
 #pragma unroll 1
     for (int l = 0; l < 27; ++l) {
-      const double v = bad ? __hiloint2double(0x7FF80000, 0) : scale.join_far(ld2(sU + l * kOctThreads));
+      const double v = bad ? __hiloint2double(0x7FF80000, 0) : join_far(ld2(sU + l * kOctThreads), bias);
       const int32_t id = __ldg(map + l * og.ncp);
       if (id >= 0) {
         if (!(og.dflag && __ldg(og.dflag + id))) atomicAdd(dst + id, v);

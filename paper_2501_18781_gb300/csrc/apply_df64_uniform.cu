@@ -1,6 +1,7 @@
-// Double-float apply of the scalar Q2 operators on uniform meshes: Helmholtz and the implicit heat
-// step without convection (Section 2.3 coefficients, Appendix B matrix-free evaluation), with the
-// conductivity (or a(phi)) tabulated per Gauss point and a constant value coefficient.
+// Double-float applies on uniform meshes (Section 2.3 coefficients, Appendix B matrix-free evaluation).  First the
+// scalar Q2 operators: Helmholtz and the implicit heat step, without or with convection (also transposed, and
+// then also with a value coefficient per Gauss point), the conductivity (or a(phi)) tabulated per Gauss point; then
+// the Oseen operator, without and with the melt-pool terms.
 //
 // Vectors stay fp64 in HBM; in the kernel every value is a pair of floats hi + lo (48-bit
 // significand) and every operation is an error-free fp32 transformation on the fp32 pipes, which
@@ -44,10 +45,10 @@ __device__ __forceinline__ dd shfl_down_dd(dd v, int d) {
 
 // Scatter-add of one slab z = const of 9 nodes per cell of a warp of the 8 x 4 x 4 brick (dst at the
 // slab's first node): the faces shared by x and y neighbours inside the warp are folded by shuffles on
-// the pairs (all lanes share one scale), then every node is added to memory once per warp as a double (scale.far:
-// not for this path).  Every lane calls this; inactive lanes pass zeros.
+// the pairs (all lanes share one scale), then every node is added to memory once per warp as a double (not
+// for a far_scale).  Every lane calls this; inactive lanes pass zeros.
 __device__ __forceinline__ void scatter_dd_slab(double* __restrict__ dst, int64_t sx, uint32_t dmask, dd* R, bool active,
-                                                const Scale& scale) {
+                                                int bias) {
   const int xl = threadIdx.x & 7, yl = (threadIdx.x >> 3) & 3;
 #pragma unroll
   for (int b = 0; b < 3; ++b) {
@@ -66,20 +67,20 @@ __device__ __forceinline__ void scatter_dd_slab(double* __restrict__ dst, int64_
   for (int l = 0; l < 9; ++l) {
     const int a = l % 3, b = l / 3;
     if ((a == 0 && xl > 0) || (b == 0 && yl > 0) || ((dmask >> l) & 1u)) continue;
-    atomicAdd(dst + a + sx * b, scale.join(R[l]));
+    atomicAdd(dst + a + sx * b, join(R[l], bias));
   }
 }
 // What scatter_dd_slab leaves: the test side of a cell of a warp whose scale is far (col, slots STRIDE apart; dst
 // at the cell's first node), and a NaN into every row of a cell with an Inf or NaN among its inputs.
 template <int STRIDE>
 __device__ __forceinline__ void scatter_rare(double* __restrict__ dst, int64_t sx, int64_t sy, uint32_t dmask,
-                                             const float2* col, const Scale& scale, bool bad) {
+                                             const float2* col, int bias, bool bad) {
 #pragma unroll 1
   for (int l = 0; l < 27; ++l) {
     const float2 v = col[l * STRIDE];
     if (!((dmask >> l) & 1u))
       atomicAdd(dst + l % 3 + sx * ((l / 3) % 3) + sy * (l / 9),
-                bad ? __hiloint2double(0x7FF80000, 0) : scale.join_far(dd{v.x, v.y}));
+                bad ? __hiloint2double(0x7FF80000, 0) : join_far(dd{v.x, v.y}, bias));
   }
 }
 
@@ -251,7 +252,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_scalar_df_uniform(const __grid_
     for (int c = 0; c < 3; ++c) st2(sV + (p + 9 * c) * kThreads, V[c]);
   }
   double* __restrict__ d = A.dst + int64_t(blockIdx.y) * A.ld + base;
-  const Scale scale(bias);
+  const bool far = far_scale(bias);
 #pragma unroll 1
   for (int c = 0; c < 3; ++c) {
     dd R[9];
@@ -270,14 +271,14 @@ __global__ void __launch_bounds__(kThreads, 4) k_scalar_df_uniform(const __grid_
 #pragma unroll
       for (int p = 0; p < 9; ++p) R[p] = dd{0.f, 0.f};
     }
-    if (scale.far) {
+    if (far) {
 #pragma unroll
       for (int p = 0; p < 9; ++p) st2(sV + (9 * c + p) * kThreads, R[p]);
     } else {
-      scatter_dd_slab(d + ug.sy * c, ug.sx, (dmask >> (9 * c)) & 0x1FFu, R, active, scale);
+      scatter_dd_slab(d + ug.sy * c, ug.sx, (dmask >> (9 * c)) & 0x1FFu, R, active, bias);
     }
   }
-  if (active && (scale.far || bad)) scatter_rare<kThreads>(d, ug.sx, ug.sy, dmask, sV, scale, bad);
+  if (active && (far || bad)) scatter_rare<kThreads>(d, ug.sx, ug.sy, dmask, sV, bias, bad);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -296,9 +297,9 @@ __global__ void __launch_bounds__(kThreads, 4) k_scalar_df_uniform(const __grid_
 // whole test side, and the value transpose along a.  So each derivative is taken by whole lines, and the
 // rolled loops over planes keep the three warps inside a short instruction body.
 // Bound: fp32 instruction issue at 12 warps per SM (48 KB of shared memory per block).  45.9k instead of
-// 72.9k instructions per 32 cells at 63 % instead of 46 % of the issue slots: 64^3 1105 -> 505 us (539 with
-// tables over cells, whose rows took 64-bit address arithmetic; per tile they share the offsets of the
-// shared arrays, and one instruction per table fetches a tile into L2).
+// 72.9k instructions per 32 cells at 63 % instead of 46 % of the issue slots: 64^3 1105 -> 505 us (512 since any scale can
+// leave the kernel; 539 with tables over cells, whose rows took 64-bit address arithmetic; per tile they share
+// the offsets of the shared arrays, and one instruction per table fetches a tile into L2).
 
 struct DfOseenArgs {
   const double* src;
@@ -329,7 +330,7 @@ template <bool EXT>
 __global__ void __launch_bounds__(96, 4) k_oseen_df_uniform(const __grid_constant__ DfOseenArgs A, UniformGeom ug) {
   extern __shared__ float2 df_smem[];
   __shared__ int sE[3];
-  __shared__ unsigned sBad[3];   // cells with an Inf or NaN among the component's inputs
+  __shared__ unsigned sBad[4];   // cells with an Inf or NaN among the component's inputs, among the pressures
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   float2* const sU = df_smem + lane;                    // component e, point q at sU[(27 e + q) * 32]
   float2* const sV = df_smem + 81 * 32 + w * 27 * 32 + lane;
@@ -405,10 +406,11 @@ __global__ void __launch_bounds__(96, 4) k_oseen_df_uniform(const __grid_constan
     }
     ep = __reduce_max_sync(0xffffffffu, ep) >> 20;
   }
-  const unsigned bad_cells = __ballot_sync(0xffffffffu, bad_u);
+  const unsigned cells_u = __ballot_sync(0xffffffffu, bad_u), cells_p = __ballot_sync(0xffffffffu, bad_p);
   if (lane == 0) {
     sE[w] = int(eu);
-    sBad[w] = bad_cells;
+    sBad[w] = cells_u;
+    if (w == 0) sBad[3] = cells_p;
   }
   __syncthreads();
   const int em = max(sE[0], max(sE[1], sE[2]));
@@ -417,7 +419,6 @@ __global__ void __launch_bounds__(96, 4) k_oseen_df_uniform(const __grid_constan
   const int bias_u = exp_u ? exp_u - 1023 : 0, bias_p = exp_p ? exp_p - 1023 : 0;
   const int bias_out = max(bias_u, bias_p);
   const float su = pow2f(bias_u - bias_out);   // velocity terms into the output scale
-  const bool bad = ((sBad[0] | sBad[1] | sBad[2]) >> lane) & 1u;
   {
     float2* const p0 = sU + 27 * w * 32;
 #pragma unroll 1
@@ -592,18 +593,17 @@ __global__ void __launch_bounds__(96, 4) k_oseen_df_uniform(const __grid_constan
     const dd mh2{A.mh2.x, A.mh2.y};
     const int64_t pa = w == 0 ? 1 : (w == 1 ? px : pxy), pb = w == 1 ? 1 : px, pc = w == 2 ? 1 : pxy;
     double* const pd = A.dst + 3 * A.nu + pbase;
-    const Scale scale_u(bias_u);
-#pragma unroll
-    for (int n = 0; n < 8; ++n) Rp[n] = dd_mul(mh2, dd_norm(Rp[n]));
-    if (scale_u.far) {
+    if (__builtin_expect(far_scale(bias_u), 0)) {
 #pragma unroll
       for (int n = 0; n < 8; ++n)
-        atomicAdd(pd + (n & 1) * pa + ((n >> 1) & 1) * pb + (n >> 2) * pc, scale_u.join_far(Rp[n]));
+        atomicAdd(pd + (n & 1) * pa + ((n >> 1) & 1) * pb + (n >> 2) * pc,
+                  join_far(dd_mul(mh2, dd_norm(Rp[n])), bias_u));
     } else {
 #pragma unroll
-      for (int n = 0; n < 8; ++n) atomicAdd(pd + (n & 1) * pa + ((n >> 1) & 1) * pb + (n >> 2) * pc, scale_u.join(Rp[n]));
+      for (int n = 0; n < 8; ++n)
+        atomicAdd(pd + (n & 1) * pa + ((n >> 1) & 1) * pb + (n >> 2) * pc, join(dd_mul(mh2, dd_norm(Rp[n])), bias_u));
     }
-    if (bad)
+    if (__builtin_expect(((sBad[0] | sBad[1] | sBad[2]) >> lane) & 1u, 0))
 #pragma unroll 1
       for (int n = 0; n < 8; ++n)
         atomicAdd(pd + (n & 1) * pa + ((n >> 1) & 1) * pb + (n >> 2) * pc, __hiloint2double(0x7FF80000, 0));
@@ -644,7 +644,7 @@ __global__ void __launch_bounds__(96, 4) k_oseen_df_uniform(const __grid_constan
     }
   }
   double* __restrict__ d = A.dst + w * A.nu + base;
-  const Scale scale(bias_out);
+  const bool far = far_scale(bias_out);
 #pragma unroll 1
   for (int c = 0; c < 3; ++c) {
     dd R[9];
@@ -661,15 +661,15 @@ __global__ void __launch_bounds__(96, 4) k_oseen_df_uniform(const __grid_constan
 #pragma unroll
       for (int p = 0; p < 9; ++p) R[p] = dd{0.f, 0.f};
     }
-    if (__builtin_expect(scale.far, 0)) {
+    if (__builtin_expect(far, 0)) {
 #pragma unroll
       for (int p = 0; p < 9; ++p) st2(sV + (9 * c + p) * 32, R[p]);
     } else {
-      scatter_dd_slab(d + ug.sy * c, ug.sx, (dmask >> (9 * c)) & 0x1FFu, R, active, scale);
+      scatter_dd_slab(d + ug.sy * c, ug.sx, (dmask >> (9 * c)) & 0x1FFu, R, active, bias_out);
     }
   }
-  if (__builtin_expect(active && (scale.far || bad || bad_p), 0))
-    scatter_rare<32>(d, ug.sx, ug.sy, dmask, sV, scale, bad || bad_p);
+  const bool bad = ((sBad[0] | sBad[1] | sBad[2] | sBad[3]) >> lane) & 1u;
+  if (__builtin_expect(active && (far || bad), 0)) scatter_rare<32>(d, ug.sx, ug.sy, dmask, sV, bias_out, bad);
 }
 
 // s c as float pairs

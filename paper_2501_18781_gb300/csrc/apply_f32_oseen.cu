@@ -6,7 +6,7 @@
 // diagonal flux along a, the flux along b and the continuity share, then planes (a, c) with the flux along
 // c.  The components' Gauss-point values and test sides live in shared memory, so the loops over planes stay
 // rolled and the register count low.  One thread per cell held all three components: 255 registers, 8 warps per SM, 31 % of the
-// issue slots.  Bound now: L1 accesses and issue (60 and 50 %).  Melt-pool apply at 64^3 163 -> 137 us, at 40^3
+// issue slots.  Bound now: L1 accesses and issue (60 and 50 %).  Melt-pool apply at 64^3 164 -> 139 us, at 40^3
 // 62.7 (with the separate copy of the Dirichlet rows) -> 39.6 us.
 #include "lines.cuh"
 #include "ops.h"

@@ -33,28 +33,23 @@ __device__ __forceinline__ dd d2dd_bits(double x, int bias) {
   const float l = __fmul_rn(__fmul_rn(mf, 0x1p-52f), __uint_as_float(Ef << 23));
   return {h, __uint_as_float(__float_as_uint(l) | sign)};
 }
-// f 2^bias as a double, by bits (exact for normal floats; zero and subnormals give 0); |bias| < 896, where no
+// f 2^bias as a double, by bits (exact for normal floats; zero and subnormals give 0); bias not far_scale, so that no
 // exponent leaves the range of doubles
 __device__ __forceinline__ double f2d_bits(float f, int bias) {
   const unsigned b = __float_as_uint(f), e = (b >> 23) & 0xFFu;
   const unsigned hi = e ? (b & 0x80000000u) | (unsigned(int(e) + 896 + bias) << 20) | ((b >> 3) & 0xFFFFFu) : 0u;
   return __hiloint2double(int(hi), e ? int(b << 29) : 0);
 }
-// A warp's scale 2^bias, by bits as far as f2d_bits goes.  The rest (inputs all below 2^-895, or some above 2^895)
-// is an fp64 product, which flushes and overflows as fp64 does; the kernels join the results of such warps in a
-// path of its own (range checks in f2d_bits took 4 % of an apply, a test before each product 3 to 7 %).
-struct Scale {
-  int bits;
-  double rest;
-  bool far;
-  __device__ __forceinline__ explicit Scale(int bias) {
-    bits = min(max(bias, -895), 895);
-    far = bits != bias;
-    rest = __hiloint2double((1023 + bias - bits) << 20, 0);
-  }
-  __device__ __forceinline__ double join(dd v) const { return f2d_bits(v.h, bits) + f2d_bits(v.l, bits); }
-  __device__ __forceinline__ double join_far(dd v) const { return join(v) * rest; }
-};
+__device__ __forceinline__ double join(dd v, int bias) { return f2d_bits(v.h, bias) + f2d_bits(v.l, bias); }
+// Warps whose inputs lie all below 2^-895, or some above 2^895, join their results by fp64 conversions and
+// products instead, which flush and overflow as fp64 does, in paths of their own that keep nothing in registers for
+// it (range checks in f2d_bits took 4 % of an apply, a test before each product 3 to 7 %).
+__device__ __forceinline__ bool far_scale(int bias) { return unsigned(bias + 895) > 1790u; }
+__device__ __forceinline__ double join_far(dd v, int bias) {
+  const int part = bias / 2;
+  return (double(v.h) + double(v.l)) * __hiloint2double((1023 + part) << 20, 0) *
+         __hiloint2double((1023 + bias - part) << 20, 0);
+}
 // The biased exponent of the largest magnitude in a warp's columns of n doubles, where emax is that over all
 // of them: Inf and NaN (0x7FF) are left out, and bad says whether the thread's own column holds one.
 __device__ __forceinline__ unsigned finite_exponent(unsigned emax, const float2* col, int stride, int n, bool& bad) {

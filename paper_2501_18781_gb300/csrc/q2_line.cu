@@ -190,7 +190,7 @@ __global__ void __launch_bounds__(line_threads<kCells>()) k_q2_line(const __grid
 // other of two buffers), and p . A p is summed over the cells, so a step is
 //   cells: Ap += A_cell p, p . A_cell p          barrier
 //   rows:  p, x, r, z, r . r, r . z, Ap = 0      barrier
-// 16^3 cells, 256 steps: 11.0 -> 4.4 ms; each of the five kernels of a step had paid a launch and a drained grid.
+// 16^3 cells, 255 steps: 10.7 -> 4.6 ms; each of the five kernels of a step had paid a launch and a drained grid.
 constexpr int kCgCells = 28, kCgThreads = kRedThreads;   // 252 of 256 threads work on cells
 
 struct LineCgArgs {

@@ -580,7 +580,7 @@ template <typename T> struct CG {
   }
 
   // Small uniform Q2 Helmholtz and heat systems on the line-per-thread kernel: the whole Jacobi-CG in one
-  // cooperative launch (16^3 cells: 17 us per step, 35 us as five kernels).
+  // cooperative launch (16^3 cells: 18 us per step, 42 us as five kernels).
   bool whole_solve_kernel() const {
     const int kind = scalar_kind(op);
     return sizeof(T) == 8 && nrhs == 1 && P->kind == MF_PREC_JACOBI && op->q2_line64 && op->f64_prec == PREC_F64 &&

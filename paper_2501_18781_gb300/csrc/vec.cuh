@@ -6,7 +6,7 @@
 
 namespace mf {
 
-constexpr int kRedBlocks = 608;   // 4 x 152 SMs: fixed grid, so reductions are deterministic
+constexpr int kRedBlocks = 608;   // 4 x 152 SMs: the largest grid of a reduction (it depends on the length alone)
 constexpr int kRedThreads = 256;
 constexpr size_t kScratchDoubles = size_t(2) * kRedBlocks * 64;  // up to 64 right-hand sides
 
