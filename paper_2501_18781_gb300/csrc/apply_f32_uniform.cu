@@ -264,16 +264,18 @@ mf_status launch_tile_table_plain(mf_ctx* ctx, const mf_dofmap* m, const double*
 
 // Whether this kernel, rather than the one-thread-per-cell kernel, serves an apply to nrhs right-hand sides.  Lanes
 // without a cell cost it more (their nodes are masked plane by plane, and both kernels' warps are 8 x 4 columns):
-// up to 9 of 16 lanes with a cell the general kernel is the faster one (us, marching / general: 3 x 200 x 40 cells
-// 9.2 / 6.6, 9 x 100 x 100 17.4 / 12.2, 1 x 1 x 4000 17.8 / 9.4; at three in four lanes they meet).  The general
-// kernel takes the right-hand sides one after another, though, so below three tiles per SM it serves a single
-// one only (eight right-hand sides, 17^3 cells: 9.7 / 16.7; 9 x 5 x 300: 30.4 / 22.8).
+// up to 9 of 16 lanes with a cell the general kernel is the faster one on large meshes (us, marching / general: 3 x
+// 200 x 40 cells 9.2 / 6.6, 9 x 100 x 100 17.4 / 12.2, 1 x 1 x 4000 17.8 / 9.4; at three in four lanes they meet).
+// But it takes the right-hand sides one after another and leaves Dirichlet rows to a launch of their own (2 us):
+// below three tiles per SM (six with Dirichlet rows) it serves only what has neither (eight right-hand sides, 17^3
+// cells: 9.7 / 16.7; one, 4^3 cells with Dirichlet rows: 6.2 / 8.2, without: 6.2 / 6.2; 2 x 40 x 40 with: 5.1 / 5.8).
 bool march_serves(const mf_ctx* ctx, const mf_dofmap* m, int nrhs) {
   if (!m->uniform) return false;
   const UniformGeom ug = uniform_geom(m);
   const int64_t ncol = int64_t((ug.nx + 7) / 8) * ((ug.ny + 3) / 4);
   if (16 * int64_t(ug.nx) * ug.ny > 9 * 32 * ncol) return true;
-  return nrhs > 1 && ncol * ug.nz < 3 * int64_t(ctx->sm_count);
+  const bool rows = !m->dirichlet_list.empty();
+  return ncol * ug.nz < (rows ? 6 : 3) * int64_t(ctx->sm_count) && (nrhs > 1 || rows);
 }
 
 mf_status launch_scalar_f32_uniform(mf_ctx* ctx, const mf_dofmap* m, const float* src, float* dst, int nrhs, int64_t ld,
