@@ -286,9 +286,9 @@ __global__ void __launch_bounds__(kThreads, 4) k_scalar_df_uniform(const __grid_
 // as float pairs).  A block of three warps owns an 8 x 4 x 1 brick of 32 cells; warp C evaluates the
 // test functions of velocity component C for the brick's cells, reading the other components'
 // Gauss-point values (for the symmetric part of the stress) from shared memory.  Velocity and pressure
-// inputs are scaled by their own powers of two (the block's largest velocity / pressure input in
-// [1, 2)); velocity fluxes and value terms are rescaled by an exact power of two so that every
-// velocity test term is accumulated in the larger of the two scales.
+// inputs are scaled by their own powers of two (the block's largest finite velocity / pressure input in
+// [1, 2); a field that is zero in the block takes the other's); velocity fluxes and value terms are rescaled
+// by an exact power of two so that every velocity test term is accumulated in the larger of the two scales.
 //
 // All three warps run one code path on permuted axes: a = the warp's own component direction C, b
 // and c the other two.  Planes (a, b) first: value terms, the diagonal flux along a (with the
@@ -297,9 +297,9 @@ __global__ void __launch_bounds__(kThreads, 4) k_scalar_df_uniform(const __grid_
 // whole test side, and the value transpose along a.  So each derivative is taken by whole lines, and the
 // rolled loops over planes keep the three warps inside a short instruction body.
 // Bound: fp32 instruction issue at 12 warps per SM (48 KB of shared memory per block).  45.9k instead of
-// 72.9k instructions per 32 cells at 63 % instead of 46 % of the issue slots: 64^3 1105 -> 505 us (512 since any scale can
-// leave the kernel; 539 with tables over cells, whose rows took 64-bit address arithmetic; per tile they share
-// the offsets of the shared arrays, and one instruction per table fetches a tile into L2).
+// 72.9k instructions per 32 cells at 63 % instead of 46 % of the issue slots: 64^3 1105 -> 505 us (539 with tables over cells,
+// whose rows took 64-bit address arithmetic; per tile they share the offsets of the shared arrays, and one
+// instruction per table fetches a tile into L2).
 
 struct DfOseenArgs {
   const double* src;

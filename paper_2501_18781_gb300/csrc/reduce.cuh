@@ -71,7 +71,9 @@ struct Dot2f {
 // pair costs three fp64 instructions.  A sum past the largest float is an fp64 number: s is then Inf and c, l are
 // its bits.
 struct Sum3f {
-  float s = 0.f, c = 0.f, l = 0.f;
+  float s, c, l;
+  Sum3f() = default;
+  __device__ __forceinline__ explicit Sum3f(const Dot2f& a) : s(a.s), c(a.c), l(0.f) {}
   __device__ __forceinline__ void add(const Dot2f& a) { add(a.s, a.c, 0.f); }
   __device__ __forceinline__ void add(const Sum3f& a) { add(a.s, a.c, a.l); }
   __device__ __forceinline__ void add(float os, float oc, float ol) {
@@ -89,9 +91,9 @@ struct Sum3f {
 };
 // fp64 sum of the N pairs or triples that load(0 .. N - 1) gives
 template <int N, typename L> __device__ __forceinline__ double exact_sum(L&& load) {
-  Sum3f t;
+  Sum3f t(load(0));
 #pragma unroll
-  for (int k = 0; k < N; ++k) t.add(load(k));
+  for (int k = 1; k < N; ++k) t.add(load(k));
   if (t.in_range()) return t.value();
   double v = 0.0;
 #pragma unroll 1
@@ -100,9 +102,9 @@ template <int N, typename L> __device__ __forceinline__ double exact_sum(L&& loa
 }
 // a thread's N accumulators in one
 template <int N, typename A> __device__ __forceinline__ Sum3f thread_sum(const A (&a)[N]) {
-  Sum3f t;
+  Sum3f t(a[0]);
 #pragma unroll
-  for (int k = 0; k < N; ++k) t.add(a[k]);
+  for (int k = 1; k < N; ++k) t.add(a[k]);
   if (!t.in_range()) {
     double v = 0.0;
 #pragma unroll
