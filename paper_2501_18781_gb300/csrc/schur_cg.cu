@@ -39,10 +39,10 @@ struct SchurArgs {
   int nx, ny, nz, maxit;
 };
 
-// Words K0 .. K0 + K - 1 (8 entries each) of stencil row i times v, in eight partial sums (error of a row of 125
-// against 64 bits, of the sum of magnitudes: 1.0e-8 rms, with two 1.7e-8); w: the row's first word (words 32
-// apart, the scaled fp16 tiled layout of stencil_at).  Entries toward nodes outside the grid are 0, and their loads
-// are clamped into it; v changes during the launch: plain loads.
+// Words K0 .. K0 + K - 1 (8 entries each) of stencil row i times v, in five partial sums (error of a row of 125
+// against 64 bits, of the sum of magnitudes: 1.2e-8 rms, with two 1.7e-8; eight cost 1 % of a 64^3 step); w: the
+// row's first word (words 32 apart, the scaled fp16 tiled layout of stencil_at).  Entries toward nodes outside the
+// grid are 0, and their loads are clamped into it; v changes during the launch: plain loads.
 template <int K0, int K>
 __device__ __forceinline__ float stencil_words(const SchurArgs& A, const uint4* w, const float* v, int i) {
   const int px = A.nx + 1, pxy = px * (A.ny + 1);
@@ -54,7 +54,7 @@ __device__ __forceinline__ float stencil_words(const SchurArgs& A, const uint4* 
     oy[d] = px * min(max(iy + d - 2, 0), A.ny);
     oz[d] = pxy * min(max(iz + d - 2, 0), A.nz);
   }
-  float s[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+  float s[5] = {0.f, 0.f, 0.f, 0.f, 0.f};   // by x offset
 #pragma unroll
   for (int c = 0; c < K / 4; ++c) {
     uint4 q[4];
@@ -69,13 +69,13 @@ __device__ __forceinline__ float stencil_words(const SchurArgs& A, const uint4* 
         memcpy(&h2, &pair[j], 4);
         const float2 f = __half22float2(h2);
         const int o = 8 * (K0 + 4 * c + k) + 2 * j;
-        float &s0 = s[2 * j], &s1 = s[2 * j + 1];
-        if (o < 125) s0 = fmaf(f.x, v[ox[o % 5] + oy[(o / 5) % 5] + oz[o / 25]], s0);
-        if (o + 1 < 125) s1 = fmaf(f.y, v[ox[(o + 1) % 5] + oy[((o + 1) / 5) % 5] + oz[(o + 1) / 25]], s1);
+        if (o < 125) s[o % 5] = fmaf(f.x, v[ox[o % 5] + oy[(o / 5) % 5] + oz[o / 25]], s[o % 5]);
+        if (o + 1 < 125)
+          s[(o + 1) % 5] = fmaf(f.y, v[ox[(o + 1) % 5] + oy[((o + 1) / 5) % 5] + oz[(o + 1) / 25]], s[(o + 1) % 5]);
       }
     }
   }
-  return ((s[0] + s[1]) + (s[2] + s[3])) + ((s[4] + s[5]) + (s[6] + s[7]));
+  return ((s[0] + s[1]) + (s[2] + s[3])) + s[4];
 }
 
 // PARTS threads share a row (warp by warp, so that every thread's entries are known at compile time).  With two
