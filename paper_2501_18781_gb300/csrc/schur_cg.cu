@@ -10,8 +10,9 @@
 // outer iteration's count.  Every block adds the per-block partial sums in the same order, so all blocks
 // hold the same scalars and the result does not depend on timing.  A barrier gives up after one second
 // of %globaltimer and sets a flag.
-// Bound: latency of the barriers and of the two dependent passes, 15 us per step at 40^3 (303 us per
-// call); the 40^3 step's Schur solves went from 30 to 8.8 ms.  The fp64 scalars are one thread's work:
+// Bound: latency of the barriers and of the two dependent passes, 16 us per step at 40^3 (325 us per
+// call; 303 with the block sums in fewer bits and two partial sums per row and thread); the 40^3 step's Schur
+// solves went from 30 to 9.1 ms.  The fp64 scalars are one thread's work:
 // divisions in all 32 warps took 8 us per step, the fp64 sums over all of them 5 us.
 #include <cuda_fp16.h>
 
